@@ -99,7 +99,7 @@ typedef struct mrcqr_opts {
                              mrcqr_sketch_ex hold them in their workspace. */
   double ortho_tol;   /* acceptance threshold on ||I - Q^T Q||_F (default 1e-13) */
   void* stats_device; /* optional DEVICE pointer to an mrcqr_stats_t written at the end */
-  int32_t fp64_products; /* 0 (default): the FP64 sketch, the off-diagonal updates of W = A R_s^{-1},
+  int32_t fp64_products; /* 0 (default): the FP64 sketch, the triangular solve W = A R_s^{-1},
                             the Gram matrix W^T W, the product Q = W R_c^{-1} and the check Q^T Q
                             as emulated FP64 on the FP16 tensor cores (exact 8-bit digit slicing,
                             integer recombination, one final rounding; see mrcqr_trsm, mrcqr_gram
@@ -294,10 +294,13 @@ int mrcqr_cholqr_precond(int64_t m, int64_t n, const double* A, int64_t lda, con
  * triangular with nonzero diagonal).  A: DEVICE double m x n, column-major,
  * ld lda >= m; R: DEVICE double n x n, column-major, ld ldr >= n, only the
  * upper triangle is read; W: DEVICE double m x n, ld ldw >= m, must not
- * overlap A or R.  fp64_products = 0: blocked by 16 columns, the off-diagonal
- * updates W_{<J} R_{<J,J} as emulated FP64 on the FP16 tensor cores (one
- * rounding each, then one FP64 subtraction from A_J), the 16 x 16 diagonal
- * blocks by FP64 substitution; 1: FP64 substitution throughout.
+ * overlap A or R.  fp64_products = 0: by panels of 32 columns, each one emulated
+ * FP64 product on the FP16 tensor cores, W_t = A_t X_t + W_{<t} Z_t with X_t =
+ * R_tt^{-1} and Z_t = -R_{<t,t} X_t formed to 2^-61 of their column maxima (one
+ * rounding per entry); a panel whose X_t would amplify the product's error more
+ * than 512-fold is solved by FP64 substitution on its diagonal block instead.  A
+ * non-finite entry of A makes its row of W NaN from the entry's panel on.
+ * fp64_products = 1: FP64 substitution throughout.
  * 1 <= n <= 512, 1 <= m < 2^31.  Allocates its workspace with cudaMallocAsync
  * on `stream`. */
 int mrcqr_trsm(int64_t m, int64_t n, const double* A, int64_t lda, const double* R, int64_t ldr, double* W,

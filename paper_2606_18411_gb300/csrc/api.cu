@@ -66,8 +66,8 @@ Plan make_plan(int64_t m, int n, int s, int tf = T_DCT, bool planes = false) {
   p.off_xt = take(sizeof(double) * (size_t)n * p.npad);
   p.off_e = take(sizeof(double) * (size_t)n * n);
   p.off_feat = take(sizeof(float) * kNumFeatures);
-  p.off_oze = take(sizeof(uint32_t) * (size_t)oz_x_cols(n));
-  p.off_ozx = take(oz_xs_bytes(n));
+  p.off_oze = take(rp_fin_ints_bytes(n));
+  p.off_ozx = take(rp_digit_bytes(n));
   p.oz = syrk_oz_plan(m, n);
   p.sk = sketch_oz_plan(m, n, s);
   p.off_colhi = take(syrk_oz_colhi_bytes(n));
@@ -79,8 +79,8 @@ Plan make_plan(int64_t m, int n, int s, int tf = T_DCT, bool planes = false) {
   p.ozpart_bytes = std::max({syrk_oz_part_bytes(p.oz), sketch_oz_part_bytes(p.sk), sketch_ozp_part_bytes(m, n, s, q_bytes),
                              planes ? sketch_ozp_part_bytes(m, n, s, p.planes_bytes) : size_t(0)});
   p.off_ozpart = take(p.ozpart_bytes);   // the Gram, the check and the FP64 sketch use it one after the other
-  p.off_tcole = take(trsm_oz_cole_bytes(n));
-  p.off_trd = take(trsm_oz_rd_bytes(n));
+  p.off_tcole = take(rp_trsm_ints_bytes(n));
+  p.off_trd = take(rp_digit_bytes(n));
   p.off_tabd = take(16ull * (size_t)(m + 1));   // FP16 digits of the quarter-wave table
   if (planes) p.off_planes = take(p.planes_bytes);
   p.total = o;
@@ -293,7 +293,7 @@ void enqueue_stage2(const Plan& p, void* ws, const double* A, int64_t lda, doubl
   long long* ozpart = at<long long>(ws, p.off_ozpart);
   if (emu)
     launch(SG_TRSM, lvl, st, [&] {
-      launch_trsm_oz(p.m, p.n, A, lda, RsT, rinv, at<uint32_t>(ws, p.off_tcole), at<unsigned char>(ws, p.off_trd), Q,
+      launch_trsm_oz(p.m, p.n, A, lda, RsT, rinv, at<int>(ws, p.off_tcole), at<unsigned char>(ws, p.off_trd), Q,
                      ldq, ctl, lvl, st, colhi);
     });
   else
@@ -312,7 +312,7 @@ void enqueue_stage2(const Plan& p, void* ws, const double* A, int64_t lda, doubl
     launch(SG_FINALIZE, lvl, st, [&] { launch_finalize(p.m, p.n, Q, ldq, XT, ctl, lvl, st); });
   else
     launch(SG_FINALIZE, lvl, st, [&] {
-      launch_finalize_oz(p.m, p.n, Q, ldq, XT, at<uint32_t>(ws, p.off_oze), at<unsigned char>(ws, p.off_ozx), ctl,
+      launch_finalize_oz(p.m, p.n, Q, ldq, XT, at<int>(ws, p.off_oze), at<unsigned char>(ws, p.off_ozx), ctl,
                          lvl, st, check ? colhi : nullptr);
     });
   if (check && emu) {
@@ -582,7 +582,7 @@ int mrcqr_regime_estimate(int64_t m, int64_t n, const double* A, int64_t lda, in
     // Q = A R^{-1} and E = Q^T Q: the CholQR run whose loss of orthogonality bounds kappa
     double* W = at<double>(ws, off_w);
     launch(SG_TRSM, 0, st, [&] {
-      launch_trsm_oz(p.m, p.n, A, lda, RsT, rinv, at<uint32_t>(ws, p.off_tcole), at<unsigned char>(ws, p.off_trd), W,
+      launch_trsm_oz(p.m, p.n, A, lda, RsT, rinv, at<int>(ws, p.off_tcole), at<unsigned char>(ws, p.off_trd), W,
                      m, ctl, 0, st, colhi);
     });
     launch(SG_CHECK, 0, st, [&] { launch_syrk_oz(p.m, p.n, W, m, p.oz, colhi, part, E, ctl, 0, st, true); });
@@ -643,7 +643,7 @@ int mrcqr_trsm(int64_t m, int64_t n, const double* A, int64_t lda, const double*
   launch(SG_PREP, 0, st, [&] { launch_rs_prepare((int)n, Rp, RsT, rinv, st); });
   if (fp64_products == 0)
     launch(SG_TRSM, 0, st, [&] {
-      launch_trsm_oz(m, (int)n, A, lda, RsT, rinv, at<uint32_t>(ws, p.off_tcole), at<unsigned char>(ws, p.off_trd), W,
+      launch_trsm_oz(m, (int)n, A, lda, RsT, rinv, at<int>(ws, p.off_tcole), at<unsigned char>(ws, p.off_trd), W,
                      ldw, ctl, 0, st);
     });
   else
@@ -705,7 +705,7 @@ int mrcqr_finalize_q(int64_t m, int64_t n, double* Q, int64_t ldq, const double*
     launch(SG_FINALIZE, 0, st, [&] { launch_finalize(m, (int)n, Q, ldq, XT, ctl, 0, st); });
   else
     launch(SG_FINALIZE, 0, st, [&] {
-      launch_finalize_oz(m, (int)n, Q, ldq, XT, at<uint32_t>(ws, p.off_oze), at<unsigned char>(ws, p.off_ozx), ctl,
+      launch_finalize_oz(m, (int)n, Q, ldq, XT, at<int>(ws, p.off_oze), at<unsigned char>(ws, p.off_ozx), ctl,
                          0, st);
     });
   cudaFreeAsync(ws, st);

@@ -61,9 +61,9 @@ struct OzWs {
   SketchOzPlan kp;
   uint32_t* colhi;
   long long* part;
-  uint32_t* tcole;
+  int* tcole;
   unsigned char* trd;
-  uint32_t* oze;
+  int* oze;
   unsigned char* ozx;
   uint64_t seed;
 };
@@ -226,10 +226,10 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
     auto& g = ozoff[i];
     g[0] = take(syrk_oz_colhi_bytes(P.n));
     g[1] = take(std::max(syrk_oz_part_bytes(z.sp), sketch_oz_part_bytes(z.kp)));
-    g[2] = take(trsm_oz_cole_bytes(P.n));
-    g[3] = take(trsm_oz_rd_bytes(P.n));
-    g[4] = take(sizeof(uint32_t) * (size_t)oz_x_cols(P.n));
-    g[5] = take(oz_xs_bytes(P.n));
+    g[2] = take(rp_trsm_ints_bytes(P.n));
+    g[3] = take(rp_digit_bytes(P.n));
+    g[4] = take(rp_fin_ints_bytes(P.n));
+    g[5] = take(rp_digit_bytes(P.n));
   }
   const size_t probs_off = take(sizeof(Prob) * (size_t)count);
   const size_t map_bytes = sketch_tc_map_bytes();
@@ -334,12 +334,13 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
       for (int i : live) {
         const Prob& P = pl.probs[i];
         const OzWs& z = pl.oz[i];
-        for (int b = 0; b < blocks(P.n, 8); ++b) z_rs.push_back(make_int4(i, b, 0, 0));
-        for (int c = 0; c < (P.n + 15) / 16 * 16; ++c) z_pr.push_back(make_int4(i, c, 0, 0));
+        if (P.n > kRpOwnScale)
+          for (int b = 0; b < blocks(P.n, 8); ++b) z_rs.push_back(make_int4(i, b, 0, 0));
+        for (int c = 0; c < rp_panels(P.n); ++c) z_pr.push_back(make_int4(i, c, 0, 0));
         for (int b = 0; b < blocks(P.m, 128); ++b) z_tr.push_back(make_int4(i, b, 0, 0));
         for (int t = 0; t < z.sp.ntiles * z.sp.slabs; ++t) z_sy.push_back(make_int4(i, t, 0, 0));
         for (int b = 0; b < blocks((int64_t)P.n * P.n, 256); ++b) z_gr.push_back(make_int4(i, b, 0, 0));
-        for (int j = 0; j < oz_x_cols(P.n); ++j) z_px.push_back(make_int4(i, j, 0, 0));
+        for (int j = 0; j < rp_cols(P.n); ++j) z_px.push_back(make_int4(i, j, 0, 0));
         for (int b = 0; b < blocks(P.m, 128); ++b) z_fi.push_back(make_int4(i, b, 0, 0));
       }
     if (pl.emu && pl.oz_grouped) {   // W = A R_s^{-1} (folding W's column maxima), G = W^T W
@@ -423,9 +424,9 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
     auto& g = ozoff[i];
     z.colhi = reinterpret_cast<uint32_t*>(base + g[0]);
     z.part = reinterpret_cast<long long*>(base + g[1]);
-    z.tcole = reinterpret_cast<uint32_t*>(base + g[2]);
+    z.tcole = reinterpret_cast<int*>(base + g[2]);
     z.trd = reinterpret_cast<unsigned char*>(base + g[3]);
-    z.oze = reinterpret_cast<uint32_t*>(base + g[4]);
+    z.oze = reinterpret_cast<int*>(base + g[4]);
     z.ozx = reinterpret_cast<unsigned char*>(base + g[5]);
   }
   for (int i = 0; i < (int)pl.oz.size(); ++i) {
@@ -435,7 +436,7 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
     P.oz_kp = z.kp;
     P.oz_colhi = z.colhi;
     P.oz_part = z.part;
-    P.oz_cole = reinterpret_cast<int*>(z.tcole);
+    P.oz_cole = z.tcole;
     P.oz_rd = z.trd;
     P.oz_xe = z.oze;
     P.oz_xs = z.ozx;
@@ -526,14 +527,14 @@ void enqueue(mrcqr_batched_plan_s& pl, cudaStream_t st) {
 }
 
 // Kernels one execute launches (each emulated heavy phase of a problem is
-// several kernels: sketch 3; TRSM 3 + Gram 3; finalize 2 + check 3).
+// several kernels: sketch 3; TRSM 2 or 3 + Gram 3; finalize 2 + check 3).
 int count_kernels(const mrcqr_batched_plan_s& pl) {
   int k = 0;
   for (const Launch& L : pl.launches) {
     switch (L.kind) {
       case K_FORK: case K_JOIN: break;
       case K_OZ_SKETCH: k += 3; break;
-      case K_OZ_STAGE2A: k += 6; break;
+      case K_OZ_STAGE2A: k += pl.probs[L.param].n > kRpOwnScale ? 6 : 5; break;
       case K_OZ_STAGE2B: k += pl.probs[L.param].check ? 5 : 2; break;
       default: k += 1;
     }
@@ -685,6 +686,7 @@ int plan_create(int count, const int64_t* m, const int64_t* n, const double* con
   };
   prepare_g_kernels(2 * 512);
   prepare_g_oz_kernels();
+  prepare_g_rowprod();
   prepare_g_sketch_tc();
   if (tune) {
     cudaStream_t ts;

@@ -54,9 +54,9 @@ struct Prob {
   SketchOzPlan oz_kp;
   uint32_t* oz_colhi;     // column maxima of A, W or Q (high words)
   long long* oz_part;     // Gram / check / FP64-sketch partials
-  int* oz_cole;           // TRSM: column exponents of D^-1 R, then e_k (2 x n16 ints)
-  unsigned char* oz_rd;   // TRSM: digit panels of D^-1 R
-  uint32_t* oz_xe;        // finalize: column exponents of R_c^-1
+  int* oz_cole;           // TRSM: multiplier column exponents, e_k (n32 ints each), panel flags
+  unsigned char* oz_rd;   // TRSM: digit panels of the multiplier
+  int* oz_xe;             // finalize: column exponents of R_c^-1
   unsigned char* oz_xs;   // finalize: digit panels of R_c^-1
   // tensor-core sketch (grouped): TMA maps of A with slabs of 64 rows (FP16/BF16) and 32 rows (FP32);
   // null when A is not eligible (16-byte alignment, even lda)
@@ -89,13 +89,14 @@ void launch_g_rmul(const Group& g, int level, cudaStream_t st);
 void launch_g_finalize(const Group& g, int level, cudaStream_t st);
 void launch_g_judge(const Group& g, int level, cudaStream_t st);
 void launch_g_publish(const Group& g, cudaStream_t st);
-// grouped emulated-FP64 heavy phases (ozaki.cu): one persistent launch per kernel over the work list
+// grouped emulated-FP64 heavy phases (ozaki.cu, rowprod.cu): one persistent launch per kernel over the work list
 //   colhi        items {i, column}: column maxima of A (FP64 sketch)
 //   sketch_oz    items {i, item of the problem's SketchOzPlan}   sketch_oz_reduce {i, 256-entry block}
-//   row_scale    items {i, 8-row block of R_s}                   prep_r {i, column < n16}
+//   row_scale    items {i, 8-row block of R_s}                   prep_r {i, 32-column panel}
 //   trsm_oz      items {i, 128-row block}
 //   syrk_oz      items {i, item of the problem's SyrkOzPlan}     syrk_oz_reduce {i, 256-entry block}
-//   prep_x       items {i, column < n64}                         finalize_oz {i, 128-row block}
+//   prep_x       items {i, column < n32}                         finalize_oz {i, 128-row block}
+void prepare_g_rowprod();      // kernel attributes of rowprod.cu; call outside stream capture
 void prepare_g_oz_kernels();   // kernel attributes; call outside stream capture
 void launch_g_oz_colhi(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_sketch(const Group& g, int level, cudaStream_t st);
@@ -172,7 +173,6 @@ void launch_finalize(int64_t m, int n, double* Q, int64_t ldq, const double* XT,
 void launch_judge(int n, const double* E, int check, Ctl* ctl, int level, cudaStream_t st);
 
 // --- emulated FP64 products on tensor cores (ozaki.cu) ---------------------------
-size_t oz_xs_bytes(int n);
 // rows_per_slab > 0: that slab height (a tuned value); 0: slabs chosen so tiles x slabs fills the GPU
 SyrkOzPlan syrk_oz_plan(int64_t m, int n, int64_t rows_per_slab = 0);
 size_t syrk_oz_part_bytes(const SyrkOzPlan& P);
@@ -182,26 +182,31 @@ size_t syrk_oz_colhi_bytes(int n);
 void launch_syrk_oz(int64_t m, int n, const double* W, int64_t ldw, const SyrkOzPlan& P, uint32_t* colHi,
                     long long* part, double* out, Ctl* ctl, int level, cudaStream_t st, bool colhi_ready = false);
 SketchOzPlan sketch_oz_plan(int64_t m, int n, int s);
-// W = A R^{-1} (k_trsm_oz, 16-column blocks): workspace of the R digit panels and exponents
-size_t trsm_oz_rd_bytes(int n);
-// columns of the finalize's X digits and exponents (n padded to its tile width)
-int oz_x_cols(int n);
-size_t trsm_oz_cole_bytes(int n);
-void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double* RT, const double* rinv,
-                    uint32_t* colE, unsigned char* Rd, double* W, int64_t ldw, Ctl* ctl, int level, cudaStream_t st,
-                    uint32_t* colHiOut = nullptr);
 size_t sketch_oz_part_bytes(const SketchOzPlan& P);
 void launch_sketch_oz(int64_t m, int n, int s, const double* A, int64_t lda, const uint32_t* idx, const double* tab,
                       uint64_t seed, const SketchOzPlan& P, uint32_t* colHi, long long* part, double* Y, Ctl* ctl,
                       int level, cudaStream_t st, int tf = 0);
-void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* XT, uint32_t* colE,
-                        unsigned char* Xs, Ctl* ctl, int level, cudaStream_t st, uint32_t* colHiOut = nullptr);
 // column maxima of |X| (high words) into colHi, and Y from FP64-sketch partials (P.slabs row slabs)
 void launch_oz_col_hi(int64_t m, int n, const double* X, int64_t ldx, uint32_t* colHi, const Ctl* ctl, int level,
                       cudaStream_t st);
 void launch_sketch_oz_reduce(int n, int s, const uint32_t* colHi, const uint32_t* idx, const SketchOzPlan& P,
                              const long long* part, double* Y, Ctl* ctl, int level, cudaStream_t st, int tf,
                              int64_t m);
+
+// --- W = A R^{-1} and Q = W X in emulated FP64 (rowprod.cu) -----------------------
+// Workspace: digit panels of the multiplier (each product), the TRSM's integers (column exponents, row
+// scalings, panel flags), the finalize's column exponents; columns and 32-column panels of n.
+constexpr int kRpOwnScale = 128;   // up to this n the TRSM's preparation finds the row scalings itself (no launch)
+size_t rp_digit_bytes(int n);
+size_t rp_trsm_ints_bytes(int n);
+size_t rp_fin_ints_bytes(int n);
+int rp_cols(int n);
+int rp_panels(int n);
+void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double* RT, const double* rinv, int* ints,
+                    unsigned char* Rd, double* W, int64_t ldw, Ctl* ctl, int level, cudaStream_t st,
+                    uint32_t* colHiOut = nullptr);
+void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* XT, int* colE, unsigned char* Xs,
+                        Ctl* ctl, int level, cudaStream_t st, uint32_t* colHiOut = nullptr);
 
 // --- FP64 sketch from digit planes (ozaki_planes.cu) -----------------------------
 // The planes of D A (16 bytes per entry) go to `scratch` in row chunks of sketch_ozp_chunk_rows rows

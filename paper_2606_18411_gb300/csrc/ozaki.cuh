@@ -48,16 +48,32 @@ __device__ __forceinline__ uint32_t exp_field(uint32_t hi) { return (hi >> 20) &
 // d_a + 128; the carries do the rest).  Zero and subnormal x give I = 0.  The
 // power-of-two scale eoff (a diagonal scaling D of a product (X D)(D^-1 Y))
 // never rounds.
+//
+// The slicing kernels spend most of their instructions here and in
+// digits8_pack, on the 64-lane integer pipe, so the common case is kept short:
+// with the significand M left-aligned in 64 bits, I = M >> t plus bit t - 1 of
+// M (round half up in magnitude), t = Eref - eoff - E + 1 >= 1.  For t <= 32
+// these are three funnel shifts.  Values below 2^-31 of the reference, zeros
+// and subnormals (t > min(32, Eref - eoff): E = 0 gives t = Eref - eoff + 1)
+// take the general form in a branch that a warp normally skips.
 __device__ __forceinline__ uint64_t biased_fixed63(uint32_t hi, uint32_t lo, int Eref, int eoff) {
+  const int top = Eref - eoff;
   const int E = (int)exp_field(hi);
-  uint64_t v = 0;
-  if (E != 0) {
-    const uint64_t M = ((uint64_t)(hi & 0xFFFFFu) << 32 | lo) | (1ull << 52);
-    const int sh = E + eoff - Eref + 10;   // I = round(M 2^sh), sh <= 10
-    if (sh >= 0) v = M << sh;
-    else if (sh > -64) v = (M + (1ull << (-sh - 1))) >> (-sh);
+  const int t = top + 1 - E;
+  const uint32_t mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
+  uint32_t rl = __funnelshift_rc(ml, mh, (uint32_t)t), rh = __funnelshift_rc(mh, 0u, (uint32_t)t);
+  uint32_t rb = __funnelshift_rc(ml, mh, (uint32_t)(t - 1)) & 1u;
+  if (t > min(32, top)) {
+    uint64_t v = 0;
+    if (E != 0 && t <= 64) {
+      const uint64_t M = (uint64_t)mh << 32 | ml;
+      v = ((M >> (t - 1)) + 1ull) >> 1;
+    }
+    rl = (uint32_t)v;
+    rh = (uint32_t)(v >> 32);
+    rb = 0u;
   }
-  return v + 0x0080808080808080ull;
+  return ((uint64_t)rh << 32 | rl) + rb + 0x0080808080808080ull;
 }
 
 // Signed digits d[0..7] of x 2^eoff (see biased_fixed63), sign of x included.
@@ -80,26 +96,57 @@ __device__ __forceinline__ void digits8(uint32_t hi, uint32_t lo, int Eref, int*
 
 // The eight digits of two values as packed FP16 pairs (digit a of x0 in the
 // low half of out[a], of x1 in the high half), straight from the bytes of
-// their biased fixed-point words J0, J1 and their signs: FP16 bits
-// 0x6580 + byte are the value 1536 + d_a (one binade, spacing 1), and one
-// fused multiply-add (1536 + d) s - 1536 s = s d per pair applies the sign
-// exactly.
-__device__ __forceinline__ void digits8_pack(uint64_t J0, uint64_t J1, uint32_t neg0, uint32_t neg1, uint32_t* out) {
-  const uint32_t l0 = (uint32_t)J0, h0 = (uint32_t)(J0 >> 32), l1 = (uint32_t)J1, h1 = (uint32_t)(J1 >> 32);
-  const uint32_t sgn = (neg0 << 15) | (neg1 << 31);
-  const uint32_t sb = 0x3C003C00u | sgn;   // (+-1, +-1)
-  const uint32_t cb = 0xE600E600u ^ sgn;   // (-+1536, -+1536)
+// their biased fixed-point words (hi J0h, lo J0l; J1h, J1l) and the sign bits
+// of h0, h1: the FP16 bits 0x6400 + byte are the value 1024 + byte (one
+// binade, spacing 1), and one fused multiply-add (1024 + byte) s - c s, c =
+// 1024 for digit 0 and 1152 (1024 + the bias 128) for the others, is s d
+// exactly.  Bytes move in two permutes per 16 bits of both words (pair the
+// halves, then put the 0x64 between the bytes): twelve per pair of values and
+// no masks.
+__device__ __forceinline__ void digits8_pack(uint32_t J0h, uint32_t J0l, uint32_t J1h, uint32_t J1l, uint32_t h0,
+                                             uint32_t h1, uint32_t* out) {
+  const uint32_t x = __byte_perm(h0, h1, 0x7030u);            // sign bytes of both values
+  const uint32_t sb = (x & 0x80008000u) | 0x3C003C00u;        // (+-1, +-1)
+  const uint32_t cb = (x & 0x80008000u) ^ 0xE480E480u;        // (-+1152, -+1152)
+  const uint32_t c0 = (x & 0x80008000u) ^ 0xE400E400u;        // (-+1024, -+1024)
   const __half2 s2 = *reinterpret_cast<const __half2*>(&sb);
-  const __half2 c2 = *reinterpret_cast<const __half2*>(&cb);
 #pragma unroll
-  for (int a = 0; a < kSlices; ++a) {
-    const int k = a < 4 ? 3 - a : 7 - a;   // byte of the 32-bit word holding digit a
-    const uint32_t w0 = a < 4 ? h0 : l0, w1 = a < 4 ? h1 : l1;
-    uint32_t t = __byte_perm(w0, w1, (uint32_t)(k | (k << 4) | ((4 + k) << 8) | ((4 + k) << 12))) & 0x00FF00FFu;
-    t += a == 0 ? 0x66006600u : 0x65806580u;
-    const __half2 r = __hfma2(*reinterpret_cast<const __half2*>(&t), s2, c2);
-    out[a] = *reinterpret_cast<const uint32_t*>(&r);
+  for (int w = 0; w < 4; ++w) {            // 16 bits of each word, from the top: digits 2 w and 2 w + 1
+    const uint32_t p = __byte_perm(w < 2 ? J0h : J0l, w < 2 ? J1h : J1l, (w & 1) ? 0x5410u : 0x7632u);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int a = 2 * w + k;
+      const uint32_t t = __byte_perm(p, 0x64646464u, k == 0 ? 0x4341u : 0x4240u);
+      const uint32_t c = a == 0 ? c0 : cb;
+      const __half2 r = __hfma2(*reinterpret_cast<const __half2*>(&t), s2, *reinterpret_cast<const __half2*>(&c));
+      out[a] = *reinterpret_cast<const uint32_t*>(&r);
+    }
   }
+}
+__device__ __forceinline__ void digits8_pack(uint64_t J0, uint64_t J1, uint32_t neg0, uint32_t neg1, uint32_t* out) {
+  digits8_pack((uint32_t)(J0 >> 32), (uint32_t)J0, (uint32_t)(J1 >> 32), (uint32_t)J1, neg0 << 31, neg1 << 31, out);
+}
+
+// The biased fixed-point word of biased_fixed63 without a branch, for
+// 0 <= k = E + eoff - Eref + 31 <= 31 (every value from the reference's binade
+// down to 2^-31 of it): I = (M 2^k + 2^20) >> 21 with M the 53-bit
+// significand.  The variable shift is a multiplication by 2^k, which runs on
+// the FMA pipe beside the integer pipe that bounds the slicing, with the
+// rounding and the byte biases (shifted up by 21) as its addends; k for
+// the caller's range check is OR-ed into kor, c = 31 + eoff - Eref.
+__device__ __forceinline__ void fixed63_fast(uint32_t h, uint32_t l, int c, uint32_t& Jh, uint32_t& Jl, uint32_t& kor) {
+  // (bias << 21) + 2^20 split at bit 64: the low part is below 2^61, so adding it to l p < 2^63 does not carry out
+  constexpr uint64_t kBias = 0x0080808080808080ull;
+  constexpr uint64_t kLow = (kBias << 21) + (1ull << 20);
+  constexpr uint64_t kHigh = (kBias >> 43) << 32;
+  static_assert(kLow < (1ull << 61), "fixed63_fast: carry");
+  const uint32_t k = exp_field(h) + (uint32_t)c;
+  kor |= k;
+  const uint32_t p = __funnelshift_l(0u, 1u, k);   // 2^(k mod 32)
+  const uint64_t a = (uint64_t)l * p + kLow;
+  const uint64_t b = (uint64_t)((h & 0xFFFFFu) | 0x100000u) * p + (kHigh | (a >> 32));
+  Jl = __funnelshift_r((uint32_t)a, (uint32_t)b, 21);
+  Jh = __funnelshift_r((uint32_t)b, (uint32_t)(b >> 32), 21);
 }
 
 // Exact float of a small signed integer (|v| < 2^22) without a conversion
@@ -108,9 +155,8 @@ __device__ __forceinline__ float small_int_to_float(int v) {
   return __int_as_float(0x4B400000 + v) - 12582912.0f;
 }
 
-// Adds one level's exact FP32 accumulator (an integer, |v| <= 2^24) into the
-// 64-bit halves of T.
-// The shift is a multiply by 2^(8 (3 - L % 4)) fused with the 64-bit add
+// Adds one level's exact FP32 accumulator (an integer, |v| <= 2^24) into a
+// 64-bit half of T.  The shift is a multiply by 2^(8 (3 - L % 4)) fused with the 64-bit add
 // (one mad.wide.s32: a sign-extended 32 x 32 -> 64-bit product plus the
 // accumulator), exact for every |v| < 2^31.
 __device__ __forceinline__ long long mad_wide_s32(int a, int b, long long c) {
@@ -119,11 +165,13 @@ __device__ __forceinline__ long long mad_wide_s32(int a, int b, long long c) {
   return r;
 }
 
-__device__ __forceinline__ void add_level(int L, float v, long long& hi, long long& lo) {
-  const int iv = __float2int_rn(v);
-  if (L < 4) hi = mad_wide_s32(iv, 1 << (8 * (3 - L)), hi);
-  else lo = mad_wide_s32(iv, 1 << (8 * (7 - L)), lo);
-}
+// An integer |v| <= 2^22 in FP32 without a conversion instruction (those issue
+// at a sixteenth of the FMA rate, and a readout has 128 per thread): the bits
+// of v + 1.5 2^23 are kSmallBias + v.  kLevelBias is the bias's share of the
+// four levels of a half.
+constexpr int kSmallBias = 0x4B400000;
+constexpr long long kLevelBias = (long long)kSmallBias * ((1ll << 24) + (1ll << 16) + (1ll << 8) + 1);
+__device__ __forceinline__ int small_float_bits(float v) { return __float_as_int(v + 12582912.0f); }
 
 // Signed 128-bit integer as (high word th, low word tl): two's complement.
 struct I128 {
@@ -199,6 +247,53 @@ __device__ __forceinline__ double i128_to_double(I128 t, int scale) {
 // (hi 2^32 + lo) 2^scale rounded once to FP64.
 __device__ __forceinline__ double i128_to_double(long long hi, long long lo, int scale) {
   return i128_to_double(i128_from_parts(hi, lo), scale);
+}
+
+// Out of line: the rare results of the two conversions below (a copy at each of their
+// unrolled uses would fill the instruction cache).
+static __device__ __noinline__ double t96_general(long long hi, long long lo, int scale) {
+  return i128_to_double(hi, lo, scale);
+}
+
+// The same for the level sums of one tile entry, |hi|, |lo| < 2^50: 96-bit
+// arithmetic on three words, the leading bit found in the upper two of them
+// (a smaller or out-of-range result takes the general form).  About 37
+// integer-pipe instructions.
+__device__ __forceinline__ double t96_to_double(long long hi, long long lo, int scale) {
+  const long long s = hi + (lo >> 32);            // T = s 2^32 + l
+  uint32_t b = (uint32_t)((uint64_t)s >> 32), a = (uint32_t)s, l = (uint32_t)lo;
+  const uint32_t sg = (uint32_t)((int)b >> 31);   // |T|
+  const uint64_t al = (((uint64_t)a << 32 | l) ^ ((uint64_t)sg << 32 | sg)) + (sg & 1u);
+  b = (b ^ sg) + ((sg != 0u && al == 0) ? 1u : 0u);
+  a = (uint32_t)(al >> 32);
+  l = (uint32_t)al;
+  const bool small = b == 0u;
+  const uint32_t x2 = small ? a : b, x1 = small ? l : a, x0 = small ? 0u : l;
+  const int z = __clz((int)x2);
+  const uint32_t y2 = __funnelshift_l(x1, x2, z), y1 = __funnelshift_l(x0, x1, z), y0 = x0 << (z & 31);
+  // bits 63 .. 11 of (y2, y1) are the significand; round to nearest even on the rest
+  const uint32_t rest = (y1 & 0x7FFu) | (y0 != 0u ? 1u : 0u);
+  const uint32_t up = (rest + 0x3FFu + ((y1 >> 11) & 1u)) >> 11;
+  const int E = (small ? 63 : 95) - z + scale + 1023;
+  if (x2 == 0u || (uint32_t)(E - 1) >= 2045u) return t96_general(hi, lo, scale);
+  const uint64_t bits = ((uint64_t)y2 << 21 | (y1 >> 11)) + up + ((uint64_t)(uint32_t)(E - 1) << 52);
+  return __longlong_as_double((long long)(bits | (uint64_t)(sg & 0x80000000u) << 32));
+}
+
+// The same with two FP64 additions (the FP64 pipe is otherwise idle in the
+// kernels that use this; a warp's addition holds it for 64 cycles, about what
+// the integer form takes in all, so they convert half of their entries each
+// way): s 2^32 - 2^52 and 2^52 + l are exact, and their sum T is rounded once.
+__device__ __forceinline__ double t96_to_double_fp64(long long hi, long long lo, int scale) {
+  const long long s = hi + (lo >> 32);
+  const uint32_t l = (uint32_t)lo;
+  constexpr double kC = 1.5 * 19342813113834066795298816.0 + 4503599627370496.0;   // 1.5 2^84 + 2^52
+  const double a = __hiloint2double((int)((uint64_t)s >> 32) + 0x45380000, (int)(uint32_t)s);   // 1.5 2^84 + s 2^32
+  const double r = (a - kC) + __hiloint2double(0x43300000, (int)l);
+  const uint32_t h = (uint32_t)__double2hiint(r);
+  const uint32_t e = exp_field(h), E = e + (uint32_t)scale;
+  if (e == 0u || E - 1u >= 2045u) return t96_general(hi, lo, scale);
+  return __hiloint2double((int)(h + ((uint32_t)scale << 20)), __double2loint(r));
 }
 
 }  // namespace oz

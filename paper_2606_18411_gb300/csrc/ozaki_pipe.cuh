@@ -49,36 +49,166 @@ __device__ __forceinline__ void oz_issue_chunk(uint32_t tmem, uint32_t ab, uint3
   }
 }
 
-// Adds the exact level sums of TMEM lane 32 q + lane, columns 16 g .. 16 g + 15
-// (warp w: q = w % 4, g = w / 4) into the 64-bit halves hi / lo.
-__device__ __forceinline__ void oz_readout(uint32_t tmem, int q, int g, long long* hi, long long* lo) {
-  const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * 16);
-#pragma unroll 1
-  for (int L = 0; L < oz::kLevels; ++L) {
-    float v[16];
-    tc::tmem_ld16(base + (uint32_t)(L * kN), v);
-    tc::tmem_wait_ld();
+// Adds the exact level sums of 16 TMEM columns from `base` (level L at column
+// offset L * stride) into the 64-bit halves hi / lo.  The sums of |v| over eight
+// columns bound every |v|: below 2^22 (for digits of ordinary data about 2^20)
+// no conversion instruction is needed; a warp that meets a larger sum corrects
+// the readout with conversions.  kLoop: small loop bodies (in the digit-plane
+// sketch the unrolled form spills: 63 against 55 ms at m = 2^20, n = 512); else
+// unrolled, two levels of eight columns per wait (2 to 4% faster in the others).
+template <int kStride, bool kLoop>
+__device__ __forceinline__ void oz_readout_cols(uint32_t base, long long* hi, long long* lo) {
+  float big = 0.0f;
+  if (kLoop) {
 #pragma unroll
-    for (int c = 0; c < 16; ++c) oz::add_level(L, v[c], hi[c], lo[c]);
+    for (int half = 0; half < 2; ++half) {   // levels 0 .. 3 into hi, levels 4 .. 7 into lo
+      long long* x = half ? lo : hi;
+      int mul = 1 << 24;
+#pragma unroll 1
+      for (int L = 4 * half; L < 4 * half + 4; ++L) {
+        float v[16];
+        tc::tmem_ld16(base + (uint32_t)(L * kStride), v);
+        tc::tmem_wait_ld();
+#pragma unroll
+        for (int h = 0; h < 16; h += 8) {
+          float sum = 0.0f;
+#pragma unroll
+          for (int c = h; c < h + 8; ++c) {
+            sum += fabsf(v[c]);
+            x[c] = oz::mad_wide_s32(oz::small_float_bits(v[c]), mul, x[c]);
+          }
+          big = fmaxf(big, sum);
+        }
+        mul >>= 8;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < 16; h += 8) {
+#pragma unroll
+      for (int L = 0; L < oz::kLevels; L += 2) {
+        float v[2][8];
+        tc::tmem_ld8(base + (uint32_t)(L * kStride + h), v[0]);
+        tc::tmem_ld8(base + (uint32_t)((L + 1) * kStride + h), v[1]);
+        tc::tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          long long* x = L < 4 ? hi : lo;
+          float sum = 0.0f;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            sum += fabsf(v[u][c]);
+            x[h + c] = oz::mad_wide_s32(oz::small_float_bits(v[u][c]), 1 << (24 - 8 * ((L + u) & 3)), x[h + c]);
+          }
+          big = fmaxf(big, sum);
+        }
+      }
+    }
   }
+#pragma unroll
+  for (int c = 0; c < 16; ++c) hi[c] -= oz::kLevelBias, lo[c] -= oz::kLevelBias;
+  if (__any_sync(0xffffffffu, !(big < 4194304.0f))) {   // replace the sums' contributions by exact conversions
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      long long* x = half ? lo : hi;
+#pragma unroll 1
+      for (int L = 0; L < 4; ++L) {
+        float v[16];
+        tc::tmem_ld16(base + (uint32_t)((4 * half + L) * kStride), v);
+        tc::tmem_wait_ld();
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          const long long d = (long long)__float2int_rn(v[c]) - ((long long)oz::small_float_bits(v[c]) - oz::kSmallBias);
+          x[c] += d << (24 - 8 * L);
+        }
+      }
+    }
+  }
+}
+
+// The level sums of TMEM lane 32 q + lane, columns 16 g .. 16 g + 15 of a
+// 128 x 64 tile (warp w: q = w % 4, g = w / 4).
+template <bool kLoop>
+__device__ __forceinline__ void oz_readout(uint32_t tmem, int q, int g, long long* hi, long long* lo) {
+  oz_readout_cols<kN, kLoop>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * 16), hi, lo);
 }
 
 // Digits of two values (FP64 bits, sign flips f0 / f1 applied, scaled by
 // 2^eo0 / 2^eo1) against the reference exponent E, packed in pairs into the
-// eight digit panels at dst.
+// eight digit panels at the shared address dst (and dst2, if nonzero).
 __device__ __forceinline__ void oz_store_pair(double v0, double v1, uint32_t f0, uint32_t f1, int E,
-                                              unsigned char* dst, uint32_t pstride, int eo0 = 0, int eo1 = 0,
-                                              unsigned char* dst2 = nullptr, uint32_t pstride2 = 0) {
+                                              uint32_t dst, uint32_t pstride, int eo0 = 0, int eo1 = 0,
+                                              uint32_t dst2 = 0, uint32_t pstride2 = 0) {
   const uint32_t h0 = (uint32_t)__double2hiint(v0), h1 = (uint32_t)__double2hiint(v1);
   const uint64_t J0 = oz::biased_fixed63(h0, (uint32_t)__double2loint(v0), E, eo0);
   const uint64_t J1 = oz::biased_fixed63(h1, (uint32_t)__double2loint(v1), E, eo1);
   uint32_t w[oz::kSlices];
   oz::digits8_pack(J0, J1, (h0 >> 31) ^ f0, (h1 >> 31) ^ f1, w);
 #pragma unroll
-  for (int a = 0; a < oz::kSlices; ++a) *reinterpret_cast<uint32_t*>(dst + a * pstride) = w[a];
+  for (int a = 0; a < oz::kSlices; ++a) tc::st_shared(dst + a * pstride, w[a]);
   if (dst2) {
 #pragma unroll
-    for (int a = 0; a < oz::kSlices; ++a) *reinterpret_cast<uint32_t*>(dst2 + a * pstride2) = w[a];
+    for (int a = 0; a < oz::kSlices; ++a) tc::st_shared(dst2 + a * pstride2, w[a]);
+  }
+}
+
+// Digits of four values adjacent along K (reference exponent E, cr = 31 - E or
+// a large negative number that forces the general form; sign flips in bits 0 .. 3 of
+// flips) stored as 8 bytes per digit panel at the shared address dst (and
+// dst2, if nonzero).  Straight-line code with one range check at the end:
+// values below 2^-31 of the reference, zeros and subnormals make the thread
+// write its digits again from biased_fixed63.
+template <bool kFlips = false>
+__device__ __forceinline__ void oz_store_quad(const double (&v)[4], uint32_t flips, int E, int cr, uint32_t dst,
+                                              uint32_t pstride, uint32_t dst2 = 0, uint32_t pstride2 = 0) {
+  uint32_t kor = 0u;
+  uint32_t o[2][oz::kSlices];
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    uint32_t h[2], Jh[2], Jl[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      h[k] = (uint32_t)__double2hiint(v[2 * p + k]);
+      oz::fixed63_fast(h[k], (uint32_t)__double2loint(v[2 * p + k]), cr, Jh[k], Jl[k], kor);
+      if (kFlips) h[k] ^= (flips << (31 - 2 * p - k)) & 0x80000000u;
+    }
+    oz::digits8_pack(Jh[0], Jl[0], Jh[1], Jl[1], h[0], h[1], o[p]);
+  }
+#pragma unroll
+  for (int a = 0; a < oz::kSlices; ++a) tc::st_shared2(dst + a * pstride, o[0][a], o[1][a]);
+  if (dst2) {
+#pragma unroll
+    for (int a = 0; a < oz::kSlices; ++a) tc::st_shared2(dst2 + a * pstride2, o[0][a], o[1][a]);
+  }
+  if (kor > 31u) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+      oz_store_pair(v[2 * p], v[2 * p + 1], kFlips ? (flips >> (2 * p)) & 1u : 0u,
+                    kFlips ? (flips >> (2 * p + 1)) & 1u : 0u, E, dst + 4 * p, pstride, 0, 0, dst2 ? dst2 + 4 * p : 0u,
+                    pstride2);
+  }
+}
+
+// Constant of oz_store_quad for the reference exponent E (tiny references
+// take the general form: a zero's exponent field must not pass for a value's).
+__device__ __forceinline__ int oz_quad_cr(int E) { return E > 31 ? 31 - E : -(1 << 30); }
+
+// Four rows from r of one column (col: the column's base), zero from r_end on; vec: the column is
+// 16-byte aligned at even rows.
+__device__ __forceinline__ void oz_load_quad(const double* __restrict__ col, int64_t r, int64_t r_end, bool vec,
+                                             double (&v)[4]) {
+  if (r + 4 <= r_end) {
+    if (vec) {
+      const double2 x = __ldg(reinterpret_cast<const double2*>(col + r));
+      const double2 y = __ldg(reinterpret_cast<const double2*>(col + r + 2));
+      v[0] = x.x, v[1] = x.y, v[2] = y.x, v[3] = y.y;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = __ldg(col + r + i);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = r + i < r_end ? __ldg(col + r + i) : 0.0;
   }
 }
 
@@ -116,8 +246,8 @@ __device__ __forceinline__ void oz_store_cols(const double (&v)[NC / 32][2], con
   for (int it = 0; it < NC / 32; ++it) {
     const int c = 32 * it + 2 * warp + h;
     const bool d = dup >= 0 && c >= dup && c < dup + kN;   // uniform per it (dup a multiple of 64)
-    oz_store_pair(v[it][0], v[it][1], f0, f1, E[c], panel + tc::sw64_offset(c, 2 * p, 2), pstride, 0, 0,
-                  d ? bpanel + tc::sw64_offset(c - dup, 2 * p, 2) : nullptr, kBPanel);
+    oz_store_pair(v[it][0], v[it][1], f0, f1, E[c], tc::smem_u32(panel) + tc::sw64_offset(c, 2 * p, 2), pstride, 0, 0,
+                  d ? tc::smem_u32(bpanel) + tc::sw64_offset(c - dup, 2 * p, 2) : 0u, kBPanel);
   }
 }
 
@@ -162,7 +292,7 @@ __device__ __forceinline__ bool oz_run(OzPipe& P, unsigned char* smem, int nchun
     if (__syncthreads_or(!ok)) return false;
     if (ch > 0 && (ch - 1) % kGroupChunks == kGroupChunks - 1) {   // group closed at ch - 1
       tc::fence_after();
-      oz_readout(P.tmem, P.q, P.g, hi, lo);
+      oz_readout<false>(P.tmem, P.q, P.g, hi, lo);
       tc::fence_before();
       __syncthreads();
     }
@@ -177,7 +307,7 @@ __device__ __forceinline__ bool oz_run(OzPipe& P, unsigned char* smem, int nchun
     const bool ok = oz_wait_mma(P, 0);
     if (__syncthreads_or(!ok)) return false;
     tc::fence_after();
-    oz_readout(P.tmem, P.q, P.g, hi, lo);
+    oz_readout<false>(P.tmem, P.q, P.g, hi, lo);
     tc::fence_before();
     __syncthreads();
   }

@@ -197,7 +197,7 @@ __device__ __forceinline__ bool sketch_ozp_item(const CUtensorMap* tmap, int64_t
       if (__syncthreads_or(!ok) || *S.abort_flag) return false;
       if (gstart && ch > 0) {   // group closed at ch - 1: its level sums before the next group overwrites them
         tc::fence_after();
-        oz_readout(P.tmem, P.q, P.g, hi, lo);
+        oz_readout<true>(P.tmem, P.q, P.g, hi, lo);
         tc::fence_before();
         __syncthreads();
       }
@@ -219,7 +219,7 @@ __device__ __forceinline__ bool sketch_ozp_item(const CUtensorMap* tmap, int64_t
     ok = oz_wait_mma(P, (int)(S.gch + nchunks - 1)) && ok;
     if (__syncthreads_or(!ok) || *S.abort_flag) return false;
     tc::fence_after();
-    oz_readout(P.tmem, P.q, P.g, hi, lo);
+    oz_readout<true>(P.tmem, P.q, P.g, hi, lo);
     tc::fence_before();
     __syncthreads();
     S.gch += (uint32_t)nchunks;
