@@ -29,8 +29,8 @@ struct Plan {
   int tf = T_DCT;   // sketch transform; s counts the rows of Y (2 x bins for T_RFFT_REIM)
   size_t off_ctl = 0, off_idx = 0, off_tab = 0, off_ypart = 0, off_y = 0, off_sqr = 0, off_rs = 0, off_rst = 0,
          off_rinv = 0, off_gpart = 0, off_rc = 0, off_xt = 0, off_e = 0, off_feat = 0, off_oze = 0, off_ozx = 0,
-         off_colhi = 0, off_ozpart = 0, off_tcole = 0, off_trd = 0, off_tabd = 0, off_planes = 0, total = 0;
-  size_t ozpart_bytes = 0, planes_bytes = 0;
+         off_colhi = 0, off_ozpart = 0, off_tcole = 0, off_trd = 0, off_tabd = 0, off_planes = 0, off_fd = 0, total = 0;
+  size_t ozpart_bytes = 0, planes_bytes = 0, fd_scratch = 0;   // fd_scratch: scratch the four-step FP64 sketch is planned for
   SyrkOzPlan oz{};
   SketchOzPlan sk{};
 };
@@ -78,6 +78,11 @@ Plan make_plan(int64_t m, int n, int s, int tf = T_DCT, bool planes = false) {
   if (planes) p.planes_bytes = 16ull * (size_t)n * (size_t)mr;
   p.ozpart_bytes = std::max({syrk_oz_part_bytes(p.oz), sketch_oz_part_bytes(p.sk), sketch_ozp_part_bytes(m, n, s, q_bytes),
                              planes ? sketch_ozp_part_bytes(m, n, s, p.planes_bytes) : size_t(0)});
+  if (tf == T_DCT) {
+    p.fd_scratch = planes ? p.planes_bytes : q_bytes;
+    p.ozpart_bytes = std::max(p.ozpart_bytes, sketch_fd_part_bytes(m, n, s, p.fd_scratch));
+    p.off_fd = take(sketch_fd_ints_bytes(m, s));
+  }
   p.off_ozpart = take(p.ozpart_bytes);   // the Gram, the check and the FP64 sketch use it one after the other
   p.off_tcole = take(rp_trsm_ints_bytes(n));
   p.off_trd = take(rp_digit_bytes(n));
@@ -242,11 +247,12 @@ int make_ladder(int p, bool escalate, int* lv) {
 int g_sketch_variant_last = 0;
 
 // Sketch Y of level `lvl` (Algorithm 2 steps 2-4).  FP64: emulated FP64 on the
-// tensor cores unless the SIMT variant or FP64-FMA products are asked for,
-// from digit planes written into `scratch` (variant 5) where it is large and
-// aligned enough and the variant allows, else sliced per work item (3).
+// tensor cores unless the SIMT variant or FP64-FMA products are asked for:
+// the four-step form (variant 6) where its sizes and `scratch` allow, else
+// from digit planes written into `scratch` (5) where it is large and aligned
+// enough and the variant allows, else sliced per work item (3).
 // Returns the variant that ran (1 SIMT, 2 tensor-core dense rows, 3 emulated
-// FP64 sliced per item, 4 four-step, 5 emulated FP64 from digit planes).
+// FP64 sliced per item, 4 four-step, 5 emulated FP64 from digit planes, 6 four-step emulated FP64).
 int enqueue_sketch(const Plan& p, void* ws, int prec, int variant, int fp64_products, const double* A, int64_t lda,
                    uint64_t seed, double* Y, Ctl* ctl, int lvl, cudaStream_t st, void* scratch = nullptr,
                    size_t scratch_bytes = 0) {
@@ -256,6 +262,14 @@ int enqueue_sketch(const Plan& p, void* ws, int prec, int variant, int fp64_prod
   if (prec == P_FP64 && variant != 1 && fp64_products == 0) {
     uint32_t* colhi = at<uint32_t>(ws, p.off_colhi);
     long long* part = at<long long>(ws, p.off_ozpart);
+    if ((variant == 0 || variant == 6) && scratch_bytes >= p.fd_scratch &&
+        sketch_fd_eligible(p.m, p.n, p.s, p.tf, scratch, p.fd_scratch)) {
+      launch(SG_SKETCH, lvl, st, [&] {
+        launch_sketch_fd(p.m, p.n, p.s, A, lda, idx, at<uint4>(ws, p.off_tabd), seed, colhi, part, at<void>(ws, p.off_fd),
+                         Y, scratch, p.fd_scratch, ctl, lvl, st);
+      });
+      return 6;
+    }
     const bool planes = variant != 3 && sketch_ozp_eligible(p.m, p.n, scratch, scratch_bytes) &&
                         sketch_ozp_part_bytes(p.m, p.n, p.s, scratch_bytes) <= p.ozpart_bytes;
     used = 3;

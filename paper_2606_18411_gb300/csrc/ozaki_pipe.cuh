@@ -251,6 +251,28 @@ __device__ __forceinline__ void oz_store_cols(const double (&v)[NC / 32][2], con
   }
 }
 
+// --- the 128 x 32 tile of the kernels with two CTAs per SM (rowprod.cu, sketch_fd.cu): half of the TMEM each
+constexpr int kRN = 32;                           // output tile width = MMA N per level, and K chunk depth
+constexpr int kRThreads = 256;
+constexpr uint32_t kRBPanel = kRN * 64;           // one digit of a 32 x 32 multiplier block (2 KiB)
+constexpr uint32_t kRABytes = oz::kSlices * kAPanel;    // 64 KiB: digits of a 128 x 32 chunk
+constexpr uint32_t kRBBytes = oz::kSlices * kRBPanel;   // 16 KiB: digits of a multiplier block
+constexpr uint32_t kRTmem = oz::kLevels * kRN;    // 256 columns
+
+// The digit-pair products of one chunk (two K steps of 16): A digit a against
+// the stacked B digits 0 .. 7 - a (N = 32 (8 - a)), written from the column of
+// level a on.  Issued by one thread.
+__device__ __forceinline__ void rp_issue(uint32_t tmem, uint32_t ab, uint32_t bb, bool first) {
+  const uint64_t da = tc::sw64_desc(ab), db = tc::sw64_desc(bb);
+#pragma unroll
+  for (int kk = 0; kk < kRN; kk += 16)
+#pragma unroll
+    for (int a = 0; a < oz::kLevels; ++a)
+      tc::mma_f16(tmem + (uint32_t)(kRN * a), da + (uint64_t)((a * kAPanel + kk * 2) >> 4),
+                  db + (uint64_t)((kk * 2) >> 4), tc::idesc(tc::F16, kM, kRN * (oz::kLevels - a)),
+                  (kk == 0 && a == 0 && first) ? 0u : 1u);
+}
+
 struct OzPipe {
   uint64_t* bar;      // [2]: oz_run commits every batch to bar[0]; two batches in flight alternate bar[0] / bar[1]
   uint32_t tmem, idesc;

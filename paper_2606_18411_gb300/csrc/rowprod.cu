@@ -49,13 +49,7 @@ namespace {
 // convert, the other's MMAs run.  A 128 x 64 tile per CTA would take 10% fewer
 // MMA cycles and slice the chunk half as often, but holds all of TMEM and
 // leaves the tensor cores idle in every other phase of a row block.
-constexpr int kRN = 32;                           // output tile width = MMA N per level, and K chunk depth
-constexpr int kRThreads = 256;
-constexpr uint32_t kRBPanel = kRN * 64;           // one digit of a 32 x 32 multiplier block (2 KiB)
-constexpr uint32_t kRABytes = oz::kSlices * kAPanel;    // 64 KiB: digits of a 128 x 32 chunk
-constexpr uint32_t kRBBytes = oz::kSlices * kRBPanel;   // 16 KiB: digits of a multiplier block
 constexpr size_t kRSmem = (size_t)kRABytes + 2 * (size_t)kRBBytes + 1024;
-constexpr uint32_t kRTmem = oz::kLevels * kRN;    // 256 columns
 constexpr int kNoEntry = -100000, kNonfinite = 100000;
 constexpr float kAmpLimit = 512.0f;
 
@@ -146,20 +140,6 @@ __device__ __forceinline__ void rp_slice(const double (&v)[4][4], const int* es,
       oz_store_pair(v[j][2], v[j][3], 0u, 0u, Eref, as + off[j] + 4, kAPanel, e.z, e.w);
     }
   }
-}
-
-// The digit-pair products of one chunk (two K steps of 16): A digit a against
-// the stacked B digits 0 .. 7 - a (N = 32 (8 - a)), written from the column of
-// level a on.  Issued by one thread.
-__device__ __forceinline__ void rp_issue(uint32_t tmem, uint32_t ab, uint32_t bb, bool first) {
-  const uint64_t da = tc::sw64_desc(ab), db = tc::sw64_desc(bb);
-#pragma unroll
-  for (int kk = 0; kk < kRN; kk += 16)
-#pragma unroll
-    for (int a = 0; a < oz::kLevels; ++a)
-      tc::mma_f16(tmem + (uint32_t)(kRN * a), da + (uint64_t)((a * kAPanel + kk * 2) >> 4),
-                  db + (uint64_t)((kk * 2) >> 4), tc::idesc(tc::F16, kM, kRN * (oz::kLevels - a)),
-                  (kk == 0 && a == 0 && first) ? 0u : 1u);
 }
 
 // Per-problem state of a CTA: e_k, the column maxima.
