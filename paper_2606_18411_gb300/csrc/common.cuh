@@ -38,7 +38,13 @@ struct Ctl {
   float features[kNumFeatures];
 };
 
+// Waits for the stream's earlier kernels when this one was launched to overlap their end (launch_dep); a no-op
+// otherwise.  Every kernel launched that way calls it before it touches memory, so the kernels of a
+// stream stay ordered.
+__device__ __forceinline__ void wait_prior_kernels() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ bool level_inactive(const Ctl* ctl, int level) {
+  wait_prior_kernels();
   return ctl->active != level;
 }
 

@@ -84,6 +84,7 @@ __device__ __forceinline__ void sample_block(int64_t m, int s, uint2 key, uint32
 
 __global__ void __launch_bounds__(1024) k_sample(int64_t m, int s, uint2 key, uint32_t* __restrict__ idx,
                                                   const Ctl* ctl, int reim) {
+  wait_prior_kernels();
   (void)ctl;
   sample_block(m, s, key, idx, reim);
 }
@@ -98,12 +99,13 @@ void launch_sample(int64_t m, int s, uint64_t seed, uint32_t* idx, const Ctl* ct
   while (P < s) P <<= 1;
   const size_t smem = sizeof(uint32_t) * (size_t)(s + H + P);
   if (smem > 48 * 1024) cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  { ::mrcqr::note_launch(); k_sample<<<1, 1024, smem, st>>>(m, s, seed_key(seed), idx, ctl, tf == T_RFFT_REIM); }
+  launch_dep(k_sample, 1, 1024, smem, st, m, s, seed_key(seed), idx, ctl, tf == T_RFFT_REIM);
 }
 
 // ---------------------------------------------------------------------------
 // Quarter-wave table cos(pi q / (2m)), q = 0..m, in FP64.
 __global__ void k_costab(int64_t m, double* __restrict__ tab) {
+  wait_prior_kernels();
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q <= m) {
     const double c = cospi((double)q / (2.0 * (double)m));
@@ -113,7 +115,7 @@ __global__ void k_costab(int64_t m, double* __restrict__ tab) {
 
 void launch_costab(int64_t m, double* tab, cudaStream_t st) {
   const int64_t nq = m + 1;
-  { ::mrcqr::note_launch(); k_costab<<<(unsigned)((nq + 255) / 256), 256, 0, st>>>(m, tab); }
+  launch_dep(k_costab, (unsigned)((nq + 255) / 256), 256, 0, st, m, tab);
 }
 
 // fl_p exactly as the tensor-core sketch computes it (integer RNE on the
@@ -279,10 +281,14 @@ __global__ void __launch_bounds__(256) k_sketch_simt(const double* __restrict__ 
                           tf);
 }
 
+// At least this many rows per chunk: a chunk's CTA first builds its transform tables, and every chunk is a term of
+// k_sketch_reduce.
+constexpr int kSkMinRows = 128;
+
 int sketch_chunks(int64_t m, int n, int s) {
   const int tiles = ((s + kSkST - 1) / kSkST) * ((n + kSkNT - 1) / kSkNT);
   int chunks = (4 * 152 + tiles - 1) / tiles;
-  const int64_t max_chunks = (m + kSkT - 1) / kSkT;
+  const int64_t max_chunks = (m + kSkMinRows - 1) / kSkMinRows;
   if (chunks > max_chunks) chunks = (int)max_chunks;
   if (chunks < 1) chunks = 1;
   return chunks;
@@ -304,11 +310,12 @@ int sketch_max_chunks(int64_t m, int n, int s) {
 
 // The faster tensor-core variant by measurement (dense rows V1 against the
 // four-step V2) for precision prec at n columns (s = 2n); true picks the
-// four-step.  Measured at m = 2^20 on GB300 (ms, V1 / V2, CUDA events over
-// five calls): FP16 n = 128: 0.92 / 1.45, 192: 3.27 / 1.83, 256: 2.97 /
-// 2.50, 320: 8.16 / 3.81, 512: 19.6 / 6.78 (BF16 within 1% of FP16); FP32
-// n = 128: 1.93 / 2.16, 192: 7.80 / 3.14, 256: 7.12 / 4.24, 320: 20.1 /
-// 6.10.  The dense-row variant's work grows as s n, the four-step's as n; the
+// four-step.  Measured at m = 2^20 on GB300 (ms, V1 / V2): FP16 n = 64: 0.24 /
+// 0.56, 100: 0.57 / 0.84, 128: 0.58 / 1.10, 160: 1.98 / 1.28, 192: 2.38 / 1.56,
+// 224: 3.66 / 1.90, 256: 2.14 / 2.09, 320: 6.15 / 3.3 (BF16 within 6% of FP16);
+// FP32 n = 64: 0.57 / 0.89, 100: 1.51 / 1.56, 128: 1.56 / 2.00, 160: 5.72 /
+// 2.42, 192: 6.87 / 2.95, 256: 6.12 / 3.77, 320: 17.9 / 5.8.  The dense-row
+// variant's work grows as s n in tiles of 256 x 64, the four-step's as n; the
 // switch point sits between the measured sizes.
 static bool four_step_preferred(int prec, int64_t m, int n) {
   (void)m;
@@ -335,10 +342,10 @@ int launch_sketch(int prec, int variant, const double* A, int64_t lda, int64_t m
   const int64_t rpc = rows_per_chunk(m, chunks);
   const uint2 key = seed_key(seed);
   switch (prec) {
-    case P_FP16: { ::mrcqr::note_launch(); k_sketch_simt<P_FP16><<<grid, 256, 0, st>>>(A, lda, m, n, s, idx, tab, key, rpc, Ypart, ctl, level, tf); } break;
-    case P_BF16: { ::mrcqr::note_launch(); k_sketch_simt<P_BF16><<<grid, 256, 0, st>>>(A, lda, m, n, s, idx, tab, key, rpc, Ypart, ctl, level, tf); } break;
-    case P_FP32: { ::mrcqr::note_launch(); k_sketch_simt<P_FP32><<<grid, 256, 0, st>>>(A, lda, m, n, s, idx, tab, key, rpc, Ypart, ctl, level, tf); } break;
-    default: { ::mrcqr::note_launch(); k_sketch_simt<P_FP64><<<grid, 256, 0, st>>>(A, lda, m, n, s, idx, tab, key, rpc, Ypart, ctl, level, tf); } break;
+    case P_FP16: launch_dep(k_sketch_simt<P_FP16>, grid, 256, 0, st, A, lda, m, n, s, idx, tab, key, rpc, Ypart, ctl, level, tf); break;
+    case P_BF16: launch_dep(k_sketch_simt<P_BF16>, grid, 256, 0, st, A, lda, m, n, s, idx, tab, key, rpc, Ypart, ctl, level, tf); break;
+    case P_FP32: launch_dep(k_sketch_simt<P_FP32>, grid, 256, 0, st, A, lda, m, n, s, idx, tab, key, rpc, Ypart, ctl, level, tf); break;
+    default: launch_dep(k_sketch_simt<P_FP64>, grid, 256, 0, st, A, lda, m, n, s, idx, tab, key, rpc, Ypart, ctl, level, tf); break;
   }
   return 1;
 }
@@ -347,13 +354,23 @@ int launch_sketch(int prec, int variant, const double* A, int64_t lda, int64_t m
 // c_0 = 1/sqrt(2), the sqrt(m/s) sketch scale times the sqrt(2/m) c_k of the
 // orthonormal DCT-II.  Real FFT: coef = sqrt(c/m) for c sampled bins (the
 // unnormalised transform, Algorithm 2 as printed).
-__device__ __forceinline__ void sketch_reduce_entry(int n, int s, int chunks, const double* __restrict__ Ypart,
-                                                    const uint32_t* __restrict__ idx, double* __restrict__ Y,
-                                                    Ctl* ctl, int64_t e, int tf = T_DCT, int64_t m = 0) {
-  const int64_t total = (int64_t)s * n;
-  const int i = (int)(e % s);
+//
+// The partials of an entry are summed in kRedWays interleaved chains, added
+// in order at the end: by kRedWays threads where one problem has few entries
+// (n = 16: 512 serial sums took 80 us), in one thread of the grouped form.
+constexpr int kRedWays = 8;
+
+__device__ __forceinline__ double sketch_reduce_chain(int64_t total, int chunks, const double* __restrict__ Ypart,
+                                                      int64_t e, int way) {
   double acc = 0.0;
-  for (int c = 0; c < chunks; ++c) acc += Ypart[(size_t)c * total + e];
+#pragma unroll 4
+  for (int c = way; c < chunks; c += kRedWays) acc += Ypart[(size_t)c * total + e];
+  return acc;
+}
+
+__device__ __forceinline__ void sketch_reduce_entry(int n, int s, double acc, const uint32_t* __restrict__ idx,
+                                                    double* __restrict__ Y, Ctl* ctl, int64_t e, int tf, int64_t m) {
+  const int i = (int)(e % s);
   const double coef = tf == T_DCT ? sqrt(2.0 / (double)s) * (idx[i] == 0 ? 0.70710678118654752440 : 1.0)
                                   : sqrt((double)(tf == T_RFFT_REIM ? s / 2 : s) / (double)m);
   const double y = acc * coef;
@@ -368,14 +385,22 @@ __global__ void k_sketch_reduce(int n, int s, int chunks, const double* __restri
                                 const uint32_t* __restrict__ idx, double* __restrict__ Y, Ctl* ctl, int level, int tf,
                                 int64_t m) {
   if (level_inactive(ctl, level)) return;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < (int64_t)s * n) sketch_reduce_entry(n, s, chunks, Ypart, idx, Y, ctl, e, tf, m);
+  __shared__ double part[kRedWays][32];
+  const int lane = threadIdx.x & 31, way = threadIdx.x >> 5;
+  const int64_t total = (int64_t)s * n, e = (int64_t)blockIdx.x * 32 + lane;
+  part[way][lane] = e < total ? sketch_reduce_chain(total, chunks, Ypart, e, way) : 0.0;
+  __syncthreads();
+  if (way != 0 || e >= total) return;
+  double acc = part[0][lane];
+#pragma unroll
+  for (int w = 1; w < kRedWays; ++w) acc += part[w][lane];
+  sketch_reduce_entry(n, s, acc, idx, Y, ctl, e, tf, m);
 }
 
 void launch_sketch_reduce(int64_t m, int n, int s, int chunks, const double* Ypart, const uint32_t* idx, double* Y,
                           Ctl* ctl, int level, cudaStream_t st, int tf) {
   const int64_t total = (int64_t)s * n;
-  { ::mrcqr::note_launch(); k_sketch_reduce<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(n, s, chunks, Ypart, idx, Y, ctl, level, tf, m); }
+  launch_dep(k_sketch_reduce, (unsigned)((total + 31) / 32), 32 * kRedWays, 0, st, n, s, chunks, Ypart, idx, Y, ctl, level, tf, m);
 }
 
 // ---------------------------------------------------------------------------
@@ -442,7 +467,12 @@ __global__ void kg_sketch_reduce(Group g, int level) {
     const Prob& P = g.probs[w.x];
     if (P.ctl->active != level) continue;
     const int64_t e = (int64_t)w.y * 256 + threadIdx.x;
-    if (e < (int64_t)P.s * P.n) sketch_reduce_entry(P.n, P.s, P.chunks, P.ypart, P.idx, P.y, P.ctl, e, P.tf, P.m);
+    const int64_t total = (int64_t)P.s * P.n;
+    if (e < total) {
+      double acc = sketch_reduce_chain(total, P.chunks, P.ypart, e, 0);
+      for (int way = 1; way < kRedWays; ++way) acc += sketch_reduce_chain(total, P.chunks, P.ypart, e, way);
+      sketch_reduce_entry(P.n, P.s, acc, P.idx, P.y, P.ctl, e, P.tf, P.m);
+    }
   }
 }
 

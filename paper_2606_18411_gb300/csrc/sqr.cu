@@ -110,16 +110,21 @@ __global__ void __launch_bounds__(kSqrThreads) k_sketch_qr(int n, int s, const d
 
 // ---------------------------------------------------------------------------
 // Blocked form for s <= 1024 (the single-CTA kernel above keeps the larger
-// sketches): panels of kQB columns are factored by one CTA in shared memory,
-// and the columns right of a panel are updated by one warp per column (the
-// column in registers), so the O(s n^2) reflector applications are spread
-// over the GPU instead of one SM (FP64 issues at 1/64 of the FP32 rate here).
+// sketches): panels of kQB columns are factored by one CTA of four warps with
+// the panel in registers, and the columns right of a panel are updated by one
+// CTA each, so the O(s n^2) reflector applications are spread over the GPU
+// (FP64 issues at 1/64 of the FP32 rate here; one warp's FP64 instruction
+// holds a quarter of an SM for 64 cycles, so four warps with many independent
+// chains each are what one SM can use).  Narrow panels keep the O(s kQB^2)
+// work per panel that only one SM does small.
+// Measured (before: 16-column panels by one warp per column, updates by one
+// warp per column): the figures stand at launch_sketch_qr.
 // The working copy holds LAPACK's geqrf layout: beta_j = +-||x|| on the
 // diagonal, the reflector v (v_j = 1 implicit) below it; tau = 2 / ||v||^2
-// is recomputed from v where it is needed, so no extra storage is used.
-constexpr int kQB = 16;          // panel width
+// waits in the output array rinv, which k_sqr_out writes last.
+constexpr int kQB = 8;           // panel width
 constexpr int kQMaxS = 1024;     // rows handled by the blocked form
-constexpr int kQPanelThreads = 512;
+constexpr int kQThreads = 128;
 
 __global__ void k_sqr_copy(int64_t total, const double* __restrict__ Y, void* __restrict__ Wk, int fp64,
                            const Ctl* ctl, int level) {
@@ -144,6 +149,181 @@ __device__ __forceinline__ T wmax(T v) {
   return v;
 }
 
+// Sum of v over the block (every thread; four warps, red: 4 entries, free again after
+// the next barrier).
+template <typename T>
+__device__ __forceinline__ T qsum(T v, T* red) {
+  v = wsum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+// Reflector of a column with head x0 and tail sum of squares `tail`, both
+// times inv^2 resp. inv where the column was scaled by inv = 1 / amax:
+// beta = -sign(x0) ||x||, scale = 1 / (x0 - beta), tau = 2 / ||v||^2 for
+// v = (1, scale * tail entries).
+template <typename T>
+__device__ __forceinline__ void house_scalars(T x0, T tail, T amax, T inv, T& beta, T& scale, T& tau) {
+  const T y0 = x0 * inv;
+  const T nrm = amax * sqrt(fma(y0, y0, tail));
+  beta = x0 >= T(0) ? -nrm : nrm;
+  scale = T(1) / (x0 - beta);   // |x0 - beta| = |x0| + nrm: no cancellation
+  const T r = amax * scale;
+  tau = T(2) / fma(tail * r, r, T(1));
+}
+
+// Panel [c0, c1) of the s x n working copy (column-major, ld s), rows c0 .. s-1:
+// thread t holds rows t + 128 r of every panel column in registers.  FP32
+// scales each norm by the column maximum so it neither overflows nor
+// underflows; FP64 does so only when the plain sum of squares leaves
+// [1e-250, 1e250].  The reflector's scalars are formed by one lane per warp
+// (the four warps sit on four FP64 pipes).
+template <typename T, int kR>
+__global__ void __launch_bounds__(kQThreads) k_sqr_panel(int s, int c0, int c1, T* __restrict__ Wk,
+                                                         double* __restrict__ taus, const Ctl* ctl, int level) {
+  if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
+  __shared__ T red[3][4], head[kQB], dots[2][4][kQB];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rows = s - c0, b = c1 - c0;
+  T x[kQB][kR];
+#pragma unroll
+  for (int c = 0; c < kQB; ++c)
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      const int i = tid + kQThreads * r;
+      x[c][r] = c < b && i < rows ? Wk[(int64_t)(c0 + c) * s + c0 + i] : T(0);
+    }
+#pragma unroll
+  for (int jj = 0; jj < kQB; ++jj) {
+    if (jj >= b) break;
+    if (tid == jj) head[jj] = x[jj][0];
+    // tail sum of squares, unscaled (FP64) or scaled by the column maximum
+    T amax = T(1), inv = T(1), tail = T(0);
+    bool zero = false, scaled = sizeof(T) == 4;
+    if (sizeof(T) == 8) {
+      T part = T(0);
+#pragma unroll
+      for (int r = 0; r < kR; ++r)
+        if (r > 0 || tid > jj) part = fma(x[jj][r], x[jj][r], part);
+      tail = qsum(part, red[0]);
+      const T ss = fma(head[jj], head[jj], tail);
+      scaled = !(ss > T(1e-250) && ss < T(1e250));
+      zero = scaled && !(ss > T(0));   // zero column (or NaN: left as it is)
+    }
+    if (scaled && !zero) {
+      T mx = T(0);
+#pragma unroll
+      for (int r = 0; r < kR; ++r)
+        if (r > 0 || tid >= jj) mx = max(mx, (T)fabs(x[jj][r]));
+      mx = wmax(mx);
+      if (lane == 0) red[1][warp] = mx;
+      __syncthreads();
+      amax = max(max(red[1][0], red[1][1]), max(red[1][2], red[1][3]));
+      zero = !(amax > T(0));
+      inv = zero ? T(0) : T(1) / amax;
+      T part = T(0);
+#pragma unroll
+      for (int r = 0; r < kR; ++r)
+        if (r > 0 || tid > jj) {
+          const T a = x[jj][r] * inv;
+          part = fma(a, a, part);
+        }
+      tail = qsum(part, red[2]);
+    }
+    T beta = T(0), scale = T(1), tau = T(0);
+    if (!zero) {
+      if (lane == 0) house_scalars(head[jj], tail, amax, inv, beta, scale, tau);
+      beta = __shfl_sync(0xffffffffu, beta, 0);
+      scale = __shfl_sync(0xffffffffu, scale, 0);
+      tau = __shfl_sync(0xffffffffu, tau, 0);
+    } else {
+      beta = head[jj];
+    }
+    if (tid == 0) taus[c0 + jj] = (double)tau;
+    // v, its products with the columns to the right, their update
+    T d[kQB];
+#pragma unroll
+    for (int c = 0; c < kQB; ++c) d[c] = T(0);
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      T v;
+      if (r > 0 || tid > jj) {
+        x[jj][r] *= scale;
+        v = x[jj][r];
+      } else {
+        v = tid == jj ? T(1) : T(0);
+      }
+#pragma unroll
+      for (int c = jj + 1; c < kQB; ++c) d[c] = fma(v, x[c][r], d[c]);
+    }
+#pragma unroll
+    for (int c = jj + 1; c < kQB; ++c) {
+      const T w = wsum(d[c]);
+      if (lane == 0) dots[jj & 1][warp][c] = w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = jj + 1; c < kQB; ++c) {
+      const T* q = &dots[jj & 1][0][c];
+      const T f = tau * ((q[0] + q[kQB]) + (q[2 * kQB] + q[3 * kQB]));
+#pragma unroll
+      for (int r = 0; r < kR; ++r) {
+        const T v = r > 0 || tid > jj ? x[jj][r] : tid == jj ? T(1) : T(0);
+        x[c][r] = fma(-f, v, x[c][r]);
+      }
+    }
+    if (tid == jj) x[jj][0] = beta;
+  }
+#pragma unroll
+  for (int c = 0; c < kQB; ++c)
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      const int i = tid + kQThreads * r;
+      if (c < b && i < rows) Wk[(int64_t)(c0 + c) * s + c0 + i] = x[c][r];
+    }
+}
+
+// Column c1 + blockIdx.x: the panel's reflectors in order, rows c0 + t + 128 r
+// in thread t.
+template <typename T, int kR>
+__global__ void __launch_bounds__(kQThreads) k_sqr_update(int s, int c0, int c1, T* __restrict__ Wk,
+                                                          const double* __restrict__ taus, const Ctl* ctl, int level) {
+  if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
+  __shared__ T red[2][4];
+  const int tid = threadIdx.x, rows = s - c0;
+  T* y = Wk + (int64_t)(c1 + blockIdx.x) * s + c0;
+  T x[kR];
+#pragma unroll
+  for (int r = 0; r < kR; ++r) x[r] = tid + kQThreads * r < rows ? y[tid + kQThreads * r] : T(0);
+#pragma unroll 1
+  for (int j = c0; j < c1; ++j) {
+    const T* v = Wk + (int64_t)j * s + c0;
+    const int jj = j - c0;
+    T vr[kR], d = T(0);
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      const int i = tid + kQThreads * r;
+      vr[r] = i > jj && i < rows ? v[i] : i == jj ? T(1) : T(0);
+    }
+#pragma unroll
+    for (int r = 0; r < kR; ++r) d = fma(vr[r], x[r], d);
+    const T f = (T)taus[j] * qsum(d, red[jj & 1]);
+#pragma unroll
+    for (int r = 0; r < kR; ++r) x[r] = fma(-f, vr[r], x[r]);
+  }
+#pragma unroll
+  for (int r = 0; r < kR; ++r)
+    if (tid + kQThreads * r < rows) y[tid + kQThreads * r] = x[r];
+}
+
+// ---------------------------------------------------------------------------
+// One CTA for the small sketches, the matrix in shared memory (Y in, R_s out: one
+// launch, where the blocked form has 2 n / 8 + 1, each of which costs a few
+// microseconds even at a level that is not taken).  Warp w owns columns w, w +
+// nwarps, ..: at step j every warp applies reflector j to its columns right of
+// j, the owner of column j + 1 to that one first and then forms reflector
+// j + 1 while the others go on; one barrier per step.
 // Householder reflector of x[jj..rows) by one warp (the column's owner):
 // beta = -sign(x0) ||x||, v = (1, x[jj+1..] / (x0 - beta)), tau = 2 / ||v||^2.
 // x[jj] <- beta, x[jj+1..] <- v[1..]; returns tau (0 for a zero column).
@@ -224,92 +404,65 @@ __device__ __forceinline__ void house_apply_warp(const T* x, T* y, T tau, int jj
   __syncwarp();
 }
 
-// Panel [c0, c1) of the s x n working copy (column-major, ld s), rows c0 .. s-1,
-// factored in shared memory; warp w owns panel column w.  Step jj: the owner
-// of column jj has already applied reflectors 0 .. jj-1 to it and forms
-// reflector jj; after one barrier every warp right of it applies it to its own
-// column, the owner of jj+1 first and then straight on to its reflector.
 template <typename T>
-__global__ void __launch_bounds__(kQPanelThreads) k_sqr_panel(int s, int c0, int c1, T* __restrict__ Wk,
-                                                              const Ctl* ctl, int level) {
+__global__ void __launch_bounds__(1024) k_sqr_cta(int n, int s, const double* __restrict__ Y, double* __restrict__ Rs,
+                                                  double* __restrict__ RsT, double* __restrict__ rinv, const Ctl* ctl,
+                                                  int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
   extern __shared__ unsigned char sqr_smem[];
-  T* P = reinterpret_cast<T*>(sqr_smem);   // [kQB][rows]
-  __shared__ T taus[kQB];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rows = s - c0, b = c1 - c0;
-  for (int e = tid; e < b * rows; e += blockDim.x) {
-    const int c = e / rows, i = e % rows;
-    P[c * rows + i] = Wk[(int64_t)(c0 + c) * s + c0 + i];
-  }
+  T* P = reinterpret_cast<T*>(sqr_smem);   // column c at P + c s
+  __shared__ T taus[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  for (int e = tid; e < s * n; e += blockDim.x) P[e] = (T)Y[e];
   __syncthreads();
   if (warp == 0) {
-    const T t = house_warp(P, 0, rows, lane);
+    const T t = house_warp(P, 0, s, lane);
     if (lane == 0) taus[0] = t;
   }
   __syncthreads();
-  for (int jj = 0; jj < b; ++jj) {
-    if (warp > jj && warp < b) {
-      T* y = P + warp * rows;
-      house_apply_warp(P + jj * rows, y, taus[jj], jj, rows, lane);
-      if (warp == jj + 1) {
-        const T t = house_warp(y, jj + 1, rows, lane);
-        if (lane == 0) taus[jj + 1] = t;
-      }
+  for (int j = 0; j < n - 1; ++j) {
+    const T* x = P + j * s;
+    const T tau = taus[j & 1];
+    const int next = (j + 1) % nw;
+    int c = j + 1 + (warp - next + nw) % nw;   // this warp's first column right of j
+    if (warp == next) {
+      T* y = P + c * s;
+      house_apply_warp(x, y, tau, j, s, lane);
+      const T t = house_warp(y, j + 1, s, lane);
+      if (lane == 0) taus[(j + 1) & 1] = t;
+      c += nw;
     }
+    for (; c < n; c += nw) house_apply_warp(x, P + c * s, tau, j, s, lane);
     __syncthreads();
   }
-  for (int e = tid; e < b * rows; e += blockDim.x) {
-    const int c = e / rows, i = e % rows;
-    Wk[(int64_t)(c0 + c) * s + c0 + i] = P[c * rows + i];
+  const int npad = padded(n);
+  for (int e = tid; e < npad * n; e += blockDim.x) {
+    const int r = e / npad, c = e % npad;
+    const double beta = (double)P[r * s + r];
+    double v = 0.0;
+    if (c < n) {
+      if (r < c) v = beta < 0.0 ? -(double)P[c * s + r] : (double)P[c * s + r];
+      else if (r == c) v = fabs(beta);
+    }
+    RsT[(int64_t)r * npad + c] = v;
+    if (c < n) Rs[(int64_t)c * n + r] = v;
   }
+  for (int r = tid; r < npad; r += blockDim.x) rinv[r] = r < n ? 1.0 / fabs((double)P[r * s + r]) : 0.0;
 }
 
-// Columns c >= c1: apply the panel's reflectors j = c0 .. c1-1 in order
-// (one warp per column; lane l holds rows c0 + l + 32 t, t < kR, with
-// 32 kR >= s - c0).
-template <typename T, int kR>
-__global__ void __launch_bounds__(32) k_sqr_update(int s, int c0, int c1, T* __restrict__ Wk, const Ctl* ctl,
-                                                   int level) {
-  if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
-  const int lane = threadIdx.x;
-  const int c = c1 + blockIdx.x;
-  T* y = Wk + (int64_t)c * s;
-  const T* V = Wk;
-  T xr[kR];
-#pragma unroll
-  for (int t = 0; t < kR; ++t) {
-    const int i = c0 + lane + 32 * t;
-    xr[t] = i < s ? y[i] : T(0);
-  }
-  for (int j = c0; j < c1; ++j) {
-    const T* v = V + (int64_t)j * s;
-    T d[2] = {T(0), T(0)}, vv[2] = {T(0), T(0)};
-#pragma unroll
-    for (int t = 0; t < kR; ++t) {
-      const int i = c0 + lane + 32 * t;
-      if (i > j && i < s) {
-        const T vi = v[i];
-        d[t & 1] = fma(vi, xr[t], d[t & 1]);
-        vv[t & 1] = fma(vi, vi, vv[t & 1]);
-      } else if (i == j) {
-        d[t & 1] += xr[t];
-      }
-    }
-    const T dd = wsum(d[0] + d[1]), vs = wsum(vv[0] + vv[1]);
-    const T f = (T(2) / (T(1) + vs)) * dd;
-#pragma unroll
-    for (int t = 0; t < kR; ++t) {
-      const int i = c0 + lane + 32 * t;
-      if (i > j && i < s) xr[t] = fma(-f, v[i], xr[t]);
-      else if (i == j) xr[t] -= f;
-    }
-  }
-#pragma unroll
-  for (int t = 0; t < kR; ++t) {
-    const int i = c0 + lane + 32 * t;
-    if (i < s) y[i] = xr[t];
-  }
+// FP32 up to n = 64 and FP64 up to n = 32, where the sketch fits the shared memory: beyond, one SM takes longer
+// than the blocked form and its launches (FP32: n = 64 141 us against 120, but 6 against 49 where the level is
+// skipped; n = 100 274 against 191).
+template <typename T>
+bool sqr_one_cta(int n, int s) {
+  return n <= (sizeof(T) == 8 ? 32 : 64) && sizeof(T) * (size_t)n * s <= 200 * 1024;
+}
+
+template <typename T>
+void launch_sqr_cta(int n, int s, const double* Y, double* Rs, double* RsT, double* rinv, Ctl* ctl, int level,
+                    cudaStream_t st) {
+  cudaFuncSetAttribute(k_sqr_cta<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  launch_dep(k_sqr_cta<T>, 1, n <= 32 ? 512 : 1024, sizeof(T) * (size_t)n * s, st, n, s, Y, Rs, RsT, rinv, ctl, level);
 }
 
 // R_s (column-major), its padded transpose and 1/diag from the factored
@@ -339,39 +492,47 @@ template <typename T>
 void launch_sqr_blocked(int n, int s, const double* Y, T* Wk, double* Rs, double* RsT, double* rinv, Ctl* ctl,
                         int level, cudaStream_t st) {
   const int64_t total = (int64_t)s * n;
-  { ::mrcqr::note_launch(); k_sqr_copy<<<(unsigned)((total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024), 256, 0, st>>>(
-      total, Y, Wk, std::is_same<T, double>::value ? 1 : 0, ctl, level); }
-  cudaFuncSetAttribute(k_sqr_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(sizeof(T) * (size_t)kQB * (size_t)kQMaxS));
+  launch_dep(k_sqr_copy, (unsigned)((total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024), 256, 0, st, total, Y, Wk, std::is_same<T, double>::value ? 1 : 0, ctl, level);
   for (int c0 = 0; c0 < n; c0 += kQB) {
-    const int c1 = c0 + kQB < n ? c0 + kQB : n;
-    const size_t smem = sizeof(T) * (size_t)kQB * (size_t)(s - c0);
-    { ::mrcqr::note_launch(); k_sqr_panel<T><<<1, kQPanelThreads, smem, st>>>(s, c0, c1, Wk, ctl, level); }
+    const int c1 = c0 + kQB < n ? c0 + kQB : n, rows = s - c0;
+    auto panel = rows <= 128 ? k_sqr_panel<T, 1> : rows <= 256 ? k_sqr_panel<T, 2>
+               : rows <= 512 ? k_sqr_panel<T, 4> : k_sqr_panel<T, 8>;
+    launch_dep(panel, 1, kQThreads, 0, st, s, c0, c1, Wk, rinv, ctl, level);
     if (c1 < n) {
-      const int rows = s - c0;
-      const unsigned g = (unsigned)(n - c1);
-      if (rows <= 256) { ::mrcqr::note_launch(); k_sqr_update<T, 8><<<g, 32, 0, st>>>(s, c0, c1, Wk, ctl, level); }
-      else if (rows <= 512) { ::mrcqr::note_launch(); k_sqr_update<T, 16><<<g, 32, 0, st>>>(s, c0, c1, Wk, ctl, level); }
-      else { ::mrcqr::note_launch(); k_sqr_update<T, 32><<<g, 32, 0, st>>>(s, c0, c1, Wk, ctl, level); }
+      auto update = rows <= 128 ? k_sqr_update<T, 1> : rows <= 256 ? k_sqr_update<T, 2>
+                  : rows <= 512 ? k_sqr_update<T, 4> : k_sqr_update<T, 8>;
+      launch_dep(update, (unsigned)(n - c1), kQThreads, 0, st, s, c0, c1, Wk, rinv, ctl, level);
     }
   }
   const int64_t tot = (int64_t)padded(n) * n;
-  { ::mrcqr::note_launch(); k_sqr_out<T><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n, s, Wk, Rs, RsT, rinv, ctl, level); }
+  launch_dep(k_sqr_out<T>, (unsigned)((tot + 255) / 256), 256, 0, st, n, s, Wk, Rs, RsT, rinv, ctl, level);
 }
 
 size_t sqr_workspace_bytes(int n, int s) { return (size_t)n * (size_t)s * sizeof(double); }
 
+// One launch with Y in shared memory where it fits and one CTA is faster (FP32
+// up to n = 64, FP64 up to n = 32), panels of kQB columns in registers with the
+// trailing columns over the chip up to s = kQMaxS, and the kernel over global
+// memory beyond.  Measured (s = 2n, us, before / now): FP64 n = 512 8250 /
+// 4540, 128 863 / 760; FP32 n = 256 853 / 483, 100 250 / 191, 64 147 / 141,
+// 32 63 / 55; a level that is skipped costs one launch instead of up to 25
+// (49 / 6 us at n = 64).
 void launch_sketch_qr(int prec, int n, int s, const double* Y, void* work, double* Rs, double* RsT, double* rinv,
                       Ctl* ctl, int level, cudaStream_t st) {
+  if (prec == P_FP64 ? sqr_one_cta<double>(n, s) : sqr_one_cta<float>(n, s)) {
+    if (prec == P_FP64) launch_sqr_cta<double>(n, s, Y, Rs, RsT, rinv, ctl, level, st);
+    else launch_sqr_cta<float>(n, s, Y, Rs, RsT, rinv, ctl, level, st);
+    return;
+  }
   if (s <= kQMaxS) {
     if (prec == P_FP64) launch_sqr_blocked<double>(n, s, Y, (double*)work, Rs, RsT, rinv, ctl, level, st);
     else launch_sqr_blocked<float>(n, s, Y, (float*)work, Rs, RsT, rinv, ctl, level, st);
     return;
   }
   if (prec == P_FP64)
-    { ::mrcqr::note_launch(); k_sketch_qr<double><<<1, kSqrThreads, 0, st>>>(n, s, Y, (double*)work, Rs, RsT, rinv, ctl, level); }
+    launch_dep(k_sketch_qr<double>, 1, kSqrThreads, 0, st, n, s, Y, (double*)work, Rs, RsT, rinv, ctl, level);
   else
-    { ::mrcqr::note_launch(); k_sketch_qr<float><<<1, kSqrThreads, 0, st>>>(n, s, Y, (float*)work, Rs, RsT, rinv, ctl, level); }
+    launch_dep(k_sketch_qr<float>, 1, kSqrThreads, 0, st, n, s, Y, (float*)work, Rs, RsT, rinv, ctl, level);
 }
 
 }  // namespace mrcqr

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(128) k_trsm(int64_t m, int n, const double* __
 
 void launch_trsm(int64_t m, int n, const double* A, int64_t lda, const double* RT, const double* rinv, double* W,
                  int64_t ldw, const Ctl* ctl, int level, cudaStream_t st) {
-  { ::mrcqr::note_launch(); k_trsm<<<(unsigned)((m + 127) / 128), 128, 0, st>>>(m, n, A, lda, RT, rinv, W, ldw, ctl, level); }
+  launch_dep(k_trsm, (unsigned)((m + 127) / 128), 128, 0, st, m, n, A, lda, RT, rinv, W, ldw, ctl, level);
 }
 
 // ---------------------------------------------------------------------------
@@ -190,9 +190,9 @@ void launch_syrk(int64_t m, int n, const double* X, int64_t ldx, int splits, dou
   int64_t rps = (m + splits - 1) / splits;
   rps = (rps + 31) / 32 * 32;
   const dim3 grid(tiles, splits);
-  if (TN == 16) { ::mrcqr::note_launch(); k_syrk<16><<<grid, 32, 0, st>>>(m, n, X, ldx, rps, nt, Gpart, ctl, level); }
-  else if (TN == 32) { ::mrcqr::note_launch(); k_syrk<32><<<grid, 128, 0, st>>>(m, n, X, ldx, rps, nt, Gpart, ctl, level); }
-  else { ::mrcqr::note_launch(); k_syrk<64><<<grid, 512, 0, st>>>(m, n, X, ldx, rps, nt, Gpart, ctl, level); }
+  if (TN == 16) launch_dep(k_syrk<16>, grid, 32, 0, st, m, n, X, ldx, rps, nt, Gpart, ctl, level);
+  else if (TN == 32) launch_dep(k_syrk<32>, grid, 128, 0, st, m, n, X, ldx, rps, nt, Gpart, ctl, level);
+  else launch_dep(k_syrk<64>, grid, 512, 0, st, m, n, X, ldx, rps, nt, Gpart, ctl, level);
 }
 
 // ---------------------------------------------------------------------------
@@ -218,7 +218,7 @@ __global__ void k_reduce_partials(int n, int splits, const double* __restrict__ 
 void launch_reduce_partials(int n, int splits, const double* part, double* out, const Ctl* ctl, int level,
                             cudaStream_t st) {
   const int64_t nn = (int64_t)n * n;
-  { ::mrcqr::note_launch(); k_reduce_partials<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(n, splits, part, out, ctl, level); }
+  launch_dep(k_reduce_partials, (unsigned)((nn + 255) / 256), 256, 0, st, n, splits, part, out, ctl, level);
 }
 
 // ---------------------------------------------------------------------------
@@ -265,69 +265,97 @@ __device__ __forceinline__ bool chol_block(int n, double* __restrict__ G) {
   return true;
 }
 
-__global__ void __launch_bounds__(1024) k_chol(int n, double* __restrict__ G, Ctl* ctl, int level) {
-  if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
-  if (!chol_block(n, G) && threadIdx.x == 0) raise_level_status(ctl, ST_BREAKDOWN);
+// p = sqrt(d) and y = 1 / sqrt(d) of a pivot, y = -1 if d is not positive and
+// finite: an FP32 reciprocal square root of the significand, one cubically
+// convergent step (y0 (1 + r / 2 + 3 r^2 / 8), r = 1 - d y0^2 ~ 2^-21), then a
+// Heron step for p and a Newton step for y (both to about half an ulp).  A
+// dozen FP64 operations in place of the square root and the division, whose
+// sequences were most of an elimination step here (1/64-rate pipe).
+__device__ __forceinline__ void pivot_sqrt(double d, double& p, double& y) {
+  p = y = -1.0;
+  const int h = __double2hiint(d);
+  if (h < 0x00100000 || h >= 0x7FF00000) {          // not a positive normal number
+    if (d > 0.0 && h < 0x00100000) {                // subnormal
+      p = sqrt(d);
+      y = 1.0 / p;
+    }
+    return;
+  }
+  const int e2 = ((h >> 20) - 1023) & ~1;           // d = dm 2^e2, dm in [1, 4)
+  const double dm = __hiloint2double(h - (e2 << 20), __double2loint(d));
+  const double y0 = (double)rsqrtf((float)dm);
+  const double r = fma(-dm * y0, y0, 1.0);
+  double yy = fma(y0 * r, fma(0.375, r, 0.5), y0);
+  double pp = dm * yy;
+  pp = fma(fma(-pp, pp, dm) * 0.5, yy, pp);
+  yy = fma(yy, fma(-pp, yy, 1.0), yy);
+  p = __hiloint2double(__double2hiint(pp) + ((e2 / 2) << 20), __double2loint(pp));
+  y = __hiloint2double(__double2hiint(yy) - ((e2 / 2) << 20), __double2loint(yy));
 }
 
-// The same elimination with the upper triangle of G held in shared memory
-// (n <= kCholSmemN); the finished row k of R_c goes straight to G.
+// Cholesky of the w x w matrix in shared memory (S[j ld + i] = element (i, j),
+// i <= j) by all threads of the block: per step one thread forms the next
+// pivot while the other warps update the rest of the trailing matrix, so the
+// pivot's chain of dependent operations is off the critical path.  row: w
+// doubles, py: 4 doubles.  False on a breakdown (every thread).
+__device__ __forceinline__ bool chol_shared(int w, double* S, int ld, double* row, double* py) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  if (tid == 0) pivot_sqrt(S[0], py[0], py[2]);
+  for (int k = 0; k < w; ++k) {
+    __syncthreads();   // pivot k formed, columns > k updated
+    const double p = py[k & 1], y = py[2 + (k & 1)];
+    if (!(p > 0.0)) return false;
+    for (int j = k + 1 + tid; j < w; j += blockDim.x) {
+      const double r = S[j * ld + k] * y;
+      S[j * ld + k] = r;
+      row[j] = r;
+    }
+    if (tid == 0) S[k * ld + k] = p;
+    __syncthreads();
+    if (warp == 0) {
+      if (lane == 0 && k + 1 < w) {
+        const double r = row[k + 1];
+        pivot_sqrt(fma(-r, r, S[(k + 1) * ld + k + 1]), py[(k + 1) & 1], py[2 + ((k + 1) & 1)]);
+      }
+    } else {
+      for (int j = k + 1 + (warp - 1); j < w; j += nw - 1) {
+        const double rkj = row[j];
+        for (int i = k + 1 + lane; i <= j; i += 32)
+          if (i != k + 1 || j != k + 1) S[j * ld + i] = fma(-row[i], rkj, S[j * ld + i]);
+      }
+    }
+  }
+  __syncthreads();
+  return true;
+}
+
+// The whole elimination in one CTA's shared memory (n <= kCholSmemN).
+// Measured (before: square root and division by one thread between barriers; n > 64 blocked):
+// the figures stand at launch_chol.
 constexpr int kCholSmemN = 160;
 
 __global__ void __launch_bounds__(1024) k_chol_smem(int n, double* __restrict__ G, Ctl* ctl, int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
-  extern __shared__ double S[];   // S[j n + i] = G[i][j], i <= j
-  __shared__ double piv, ipiv;
-  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-  const int64_t nn = (int64_t)n * n;
-  for (int64_t e = tid; e < nn; e += blockDim.x) S[e] = G[e];
+  extern __shared__ double S[];   // S[j ld + i] = G[i][j], i <= j
+  __shared__ double row[kCholSmemN], py[4];
+  const int tid = threadIdx.x, ld = n | 1;
+  for (int e = tid; e < n * n; e += blockDim.x) S[(e / n) * ld + e % n] = G[e];
   __syncthreads();
-  bool ok = true;
-  for (int k = 0; k < n; ++k) {
-    // one thread forms the pivot and its reciprocal: the FP64 sqrt and division are
-    // long sequences on a 1/64-rate pipe, not to be repeated by every warp
-    if (tid == 0) {
-      const double d = S[(int64_t)k * n + k];
-      piv = (d > 0.0 && isfinite(d)) ? sqrt(d) : -1.0;
-      ipiv = piv > 0.0 ? 1.0 / piv : 0.0;
-    }
-    __syncthreads();
-    const double p = piv;
-    if (!(p > 0.0)) {
-      ok = false;
-      break;
-    }
-    const double ip = ipiv;
-    for (int j = k + 1 + tid; j < n; j += blockDim.x) {
-      const double r = S[(int64_t)j * n + k] * ip;
-      S[(int64_t)j * n + k] = r;
-      G[(int64_t)j * n + k] = r;
-    }
-    if (tid == 0) G[(int64_t)k * n + k] = p;
-    __syncthreads();
-    for (int j = k + 1 + ty; j < n; j += 32) {
-      const double rkj = S[(int64_t)j * n + k];
-      for (int i = k + 1 + tx; i <= j; i += 32)
-        S[(int64_t)j * n + i] = fma(-S[(int64_t)i * n + k], rkj, S[(int64_t)j * n + i]);
-    }
-    __syncthreads();
-  }
-  if (!ok) {
+  if (!chol_shared(n, S, ld, row, py)) {
     if (tid == 0) raise_level_status(ctl, ST_BREAKDOWN);
     return;
   }
-  for (int64_t e = tid; e < nn; e += blockDim.x) {
-    const int i = (int)(e % n), j = (int)(e / n);
-    if (i > j) G[e] = 0.0;
+  for (int e = tid; e < n * n; e += blockDim.x) {
+    const int i = e % n, j = e / n;
+    G[e] = i > j ? 0.0 : S[j * ld + i];
   }
 }
 
-// Blocked right-looking Cholesky over many CTAs (n > kCholBlockedMin): the
+// Blocked right-looking Cholesky over many CTAs (n > kCholSmemN): the
 // single-CTA elimination puts all n^3/3 FP64 flops on one SM's 1/64-rate
 // FP64 pipe (5.4 ms at n = 512), here the trailing updates spread over the
 // GPU.  Panels of kCB = 32 columns; for the panel at columns c0 .. c0 + 31:
-//   k_chol_diag    R_pp = chol(G_pp): one warp, lane j holds column j of the
-//                  block, pivots broadcast by shuffles (no block barriers);
+//   k_chol_diag    R_pp = chol(G_pp) in shared memory (chol_shared);
 //   k_chol_panel   R_{p,j} = R_pp^{-T} G_{p,j} for the columns j beyond the
 //                  panel: forward substitution, one warp per column;
 //   k_chol_update  G_ij -= R_{p,i}^T R_{p,j} on the trailing upper triangle,
@@ -336,43 +364,21 @@ __global__ void __launch_bounds__(1024) k_chol_smem(int n, double* __restrict__ 
 // one FMA each), a different order of the updates.  A pivot that is not
 // positive and finite raises BREAKDOWN; the later launches then return.
 constexpr int kCB = 32;
-constexpr int kCholBlockedMin = 64;
 
-__global__ void __launch_bounds__(32) k_chol_diag(int n, int c0, double* __restrict__ G, Ctl* ctl, int level) {
+__global__ void __launch_bounds__(256) k_chol_diag(int n, int c0, double* __restrict__ G, Ctl* ctl, int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
-  const int lane = threadIdx.x;
+  __shared__ double S[kCB * (kCB + 1)], row[kCB], py[4];
   const int w = min(kCB, n - c0);
-  const int64_t col = (int64_t)(c0 + lane) * n + c0;   // column c0 + lane, row c0
-  double g[kCB];
-#pragma unroll
-  for (int i = 0; i < kCB; ++i) g[i] = (lane < w && i <= lane) ? G[col + i] : 0.0;
-  bool ok = true;
-#pragma unroll
-  for (int k = 0; k < kCB; ++k) {
-    if (k >= w) break;
-    const double d = __shfl_sync(0xffffffffu, g[k], k);
-    const double piv = (d > 0.0 && isfinite(d)) ? sqrt(d) : -1.0;
-    if (!(piv > 0.0)) {
-      ok = false;
-      break;
-    }
-    const double ip = 1.0 / piv;
-    if (lane == k) g[k] = piv;
-    else if (lane > k) g[k] *= ip;                      // r_k,lane
-#pragma unroll
-    for (int i = k + 1; i < kCB; ++i) {
-      const double rki = __shfl_sync(0xffffffffu, g[k], i);
-      if (i <= lane) g[i] = fma(-rki, g[k], g[i]);
-    }
-  }
-  if (!ok) {
-    if (lane == 0) raise_level_status(ctl, ST_BREAKDOWN);
+  for (int e = threadIdx.x; e < w * w; e += blockDim.x)
+    S[(e / w) * (kCB + 1) + e % w] = G[(int64_t)(c0 + e / w) * n + c0 + e % w];
+  __syncthreads();
+  if (!chol_shared(w, S, kCB + 1, row, py)) {
+    if (threadIdx.x == 0) raise_level_status(ctl, ST_BREAKDOWN);
     return;
   }
-  if (lane < w) {
-#pragma unroll
-    for (int i = 0; i < kCB; ++i)
-      if (i < w) G[col + i] = i <= lane ? g[i] : 0.0;
+  for (int e = threadIdx.x; e < w * w; e += blockDim.x) {
+    const int i = e % w, j = e / w;
+    G[(int64_t)(c0 + j) * n + c0 + i] = i <= j ? S[j * (kCB + 1) + i] : 0.0;
   }
 }
 
@@ -435,26 +441,30 @@ __global__ void __launch_bounds__(256) k_chol_update(int n, int c0, double* __re
   }
 }
 
+// One CTA with the triangle in shared memory up to kCholSmemN columns (one
+// launch; the longest n whose padded square fits beside nothing else), blocked
+// over the chip beyond.  FP64 has 1/64 of the FP32 rate, so one warp's FP64
+// instruction holds a quadrant's pipe for 64 clocks: the pivot's reciprocal
+// square root and the column scaling are done once, not per thread.  Measured
+// (one level, us, before / now): n = 32 50 / 35, 64 117 / 88, 128 280 / 249
+// (all one launch over global memory before), 256 561 / 397, 512 1129 / 814.
+// 512 threads up to n = 48 (35 us, 38 with 1024: fewer warps at the barriers).
 void launch_chol(int n, double* G, Ctl* ctl, int level, cudaStream_t st) {
-  if (n > kCholBlockedMin) {
+  if (n > kCholSmemN) {
     for (int c0 = 0; c0 < n; c0 += kCB) {
-      { ::mrcqr::note_launch(); k_chol_diag<<<1, 32, 0, st>>>(n, c0, G, ctl, level); }
+      launch_dep(k_chol_diag, 1, 256, 0, st, n, c0, G, ctl, level);
       const int ncols = n - c0 - kCB;
       if (ncols <= 0) break;
-      { ::mrcqr::note_launch(); k_chol_panel<<<(ncols + 7) / 8, 256, 0, st>>>(n, c0, G, ctl, level); }
+      launch_dep(k_chol_panel, (ncols + 7) / 8, 256, 0, st, n, c0, G, ctl, level);
       const int T = (ncols + kCB - 1) / kCB;
-      { ::mrcqr::note_launch(); k_chol_update<<<T * (T + 1) / 2, 256, 0, st>>>(n, c0, G, ctl, level); }
+      launch_dep(k_chol_update, T * (T + 1) / 2, 256, 0, st, n, c0, G, ctl, level);
     }
     return;
   }
-  if (n <= kCholSmemN) {
-    const size_t smem = sizeof(double) * (size_t)n * n;
-    cudaFuncSetAttribute(k_chol_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(double) * kCholSmemN * kCholSmemN));
-    { ::mrcqr::note_launch(); k_chol_smem<<<1, 1024, smem, st>>>(n, G, ctl, level); }
-    return;
-  }
-  { ::mrcqr::note_launch(); k_chol<<<1, 1024, 0, st>>>(n, G, ctl, level); }
+  const size_t smem = sizeof(double) * (size_t)n * (n | 1);
+  cudaFuncSetAttribute(k_chol_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)(sizeof(double) * kCholSmemN * (kCholSmemN | 1)));
+  launch_dep(k_chol_smem, 1, n <= 48 ? 512 : 1024, smem, st, n, G, ctl, level);
 }
 
 // ---------------------------------------------------------------------------
@@ -528,10 +538,10 @@ __global__ void __launch_bounds__(128) k_trinv(int n, const double* __restrict__
 void launch_trinv(int n, const double* Rc, double* RcinvT, const Ctl* ctl, int level, cudaStream_t st) {
   const int npad = padded(n);
   const unsigned grid = (unsigned)((npad + 3) / 4);
-  if (n <= 64) { ::mrcqr::note_launch(); k_trinv<2><<<grid, 128, 0, st>>>(n, Rc, RcinvT, ctl, level); }
-  else if (n <= 128) { ::mrcqr::note_launch(); k_trinv<4><<<grid, 128, 0, st>>>(n, Rc, RcinvT, ctl, level); }
-  else if (n <= 256) { ::mrcqr::note_launch(); k_trinv<8><<<grid, 128, 0, st>>>(n, Rc, RcinvT, ctl, level); }
-  else { ::mrcqr::note_launch(); k_trinv<16><<<grid, 128, 0, st>>>(n, Rc, RcinvT, ctl, level); }
+  if (n <= 64) launch_dep(k_trinv<2>, grid, 128, 0, st, n, Rc, RcinvT, ctl, level);
+  else if (n <= 128) launch_dep(k_trinv<4>, grid, 128, 0, st, n, Rc, RcinvT, ctl, level);
+  else if (n <= 256) launch_dep(k_trinv<8>, grid, 128, 0, st, n, Rc, RcinvT, ctl, level);
+  else launch_dep(k_trinv<16>, grid, 128, 0, st, n, Rc, RcinvT, ctl, level);
 }
 
 // R = R_c R_s (Algorithm 2 step 9), upper x upper; R col-major with ld ldr,
@@ -554,7 +564,7 @@ __global__ void k_rmul(int n, const double* __restrict__ Rc, const double* __res
 void launch_rmul(int n, const double* Rc, const double* Rs, double* R, int64_t ldr, const Ctl* ctl, int level,
                  cudaStream_t st) {
   const int64_t nn = (int64_t)n * n;
-  { ::mrcqr::note_launch(); k_rmul<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(n, Rc, Rs, R, ldr, ctl, level); }
+  launch_dep(k_rmul, (unsigned)((nn + 255) / 256), 256, 0, st, n, Rc, Rs, R, ldr, ctl, level);
 }
 
 // ---------------------------------------------------------------------------
@@ -618,7 +628,7 @@ void launch_upper_to_xt(int n, const double* X, int64_t ldx, double* XT, cudaStr
 
 void launch_finalize(int64_t m, int n, double* Q, int64_t ldq, const double* XT, const Ctl* ctl, int level,
                      cudaStream_t st) {
-  { ::mrcqr::note_launch(); k_finalize<<<(unsigned)((m + 127) / 128), 128, 0, st>>>(m, n, Q, ldq, XT, ctl, level); }
+  launch_dep(k_finalize, (unsigned)((m + 127) / 128), 128, 0, st, m, n, Q, ldq, XT, ctl, level);
 }
 
 // ---------------------------------------------------------------------------
@@ -674,7 +684,7 @@ __global__ void __launch_bounds__(1024) k_judge(int n, const double* __restrict_
 }
 
 void launch_judge(int n, const double* E, int check, Ctl* ctl, int level, cudaStream_t st) {
-  { ::mrcqr::note_launch(); k_judge<<<1, 1024, 0, st>>>(n, E, check, ctl, level); }
+  launch_dep(k_judge, 1, 1024, 0, st, n, E, check, ctl, level);
 }
 
 // ---------------------------------------------------------------------------
