@@ -98,6 +98,7 @@ T* at(void* base, size_t off) {
 }
 
 __global__ void k_init_ctl(Ctl* ctl, int nlevels, int p0, int p1, int p2, int p3, double tol) {
+  wait_prior_kernels();
   ctl->active = 0;
   ctl->lvl_status = 0;
   ctl->final_status = ST_OK;
@@ -118,6 +119,7 @@ __global__ void k_init_ctl(Ctl* ctl, int nlevels, int p0, int p1, int p2, int p3
 }
 
 __global__ void k_write_stats(const Ctl* ctl, mrcqr_stats_t* out) {
+  wait_prior_kernels();
   out->status = ctl->final_status;
   out->prec_used = ctl->prec_used;
   out->retries = ctl->retries;
@@ -404,7 +406,7 @@ int mrcqr_factor_ex(int64_t m, int64_t n, const double* A, int64_t lda, double* 
   Ctl* ctl = at<Ctl>(ws, p.off_ctl);
   uint32_t* idx = at<uint32_t>(ws, p.off_idx);
   double* tab = at<double>(ws, p.off_tab);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, nlevels, lv[0], lv[1], lv[2], lv[3], tol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, nlevels, lv[0], lv[1], lv[2], lv[3], tol); });
   launch(SG_SAMPLE, 0, st, [&] { launch_sample(m, bins, seed, idx, ctl, st, tf); });
   launch(SG_COSTAB, 0, st, [&] { launch_costab(m, tab, st); });
   for (int L = 0; L < nlevels; ++L) {
@@ -423,9 +425,9 @@ int mrcqr_factor_ex(int64_t m, int64_t n, const double* A, int64_t lda, double* 
     }
     enqueue_stage2(p, ws, A, lda, Q, ldq, R, ldr, check, ctl, L, st, fp64p);
   }
-  launch(SG_STATS, 0, st, [&] { { ::mrcqr::note_launch(); k_write_stats<<<1, 1, 0, st>>>(ctl, slot); } });
+  launch(SG_STATS, 0, st, [&] { launch_dep(k_write_stats, 1, 1, 0, st, ctl, slot); });
   if (opts && opts->stats_device)
-    launch(SG_STATS, 0, st, [&] { { ::mrcqr::note_launch(); k_write_stats<<<1, 1, 0, st>>>(ctl, (mrcqr_stats_t*)opts->stats_device); } });
+    launch(SG_STATS, 0, st, [&] { launch_dep(k_write_stats, 1, 1, 0, st, ctl, (mrcqr_stats_t*)opts->stats_device); });
   cudaFreeAsync(ws, st);
   return finish(st);
 }
@@ -501,7 +503,7 @@ int mrcqr_sketch_transform(int64_t m, int64_t n, const double* A, int64_t lda, i
   Ctl* ctl = at<Ctl>(ws, p.off_ctl);
   uint32_t* idx = at<uint32_t>(ws, p.off_idx);
   double* tab = at<double>(ws, p.off_tab);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, 1, sketch_prec, P_FP64, P_FP64, P_FP64, kDefaultTol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, sketch_prec, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   launch(SG_SAMPLE, 0, st, [&] { launch_sample(m, (int)c, seed, idx, ctl, st, transform); });
   launch(SG_COSTAB, 0, st, [&] { launch_costab(m, tab, st); });
   g_sketch_variant_last = enqueue_sketch(p, ws, sketch_prec, variant, 0, A, lda, seed, Y, ctl, 0, st,
@@ -523,7 +525,7 @@ int mrcqr_sketch_qr(int64_t n, int64_t s, const double* Y, int prec, double* Rs,
     return MRCQR_ERR_ALLOC;
   }
   Ctl* ctl = at<Ctl>(ws, o_ctl);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, 1, prec, P_FP64, P_FP64, P_FP64, kDefaultTol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, prec, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   launch(SG_SQR, 0, st, [&] {
     launch_sketch_qr(prec, (int)n, (int)s, Y, at<void>(ws, o_w), Rs, at<double>(ws, o_rst), at<double>(ws, o_rinv),
                      ctl, 0, st);
@@ -548,7 +550,7 @@ int mrcqr_cholqr2(int64_t m, int64_t n, const double* A, int64_t lda, double* Q,
   Ctl* ctl = at<Ctl>(ws, p.off_ctl);
   double* Rc = at<double>(ws, p.off_rc);
   double* Rs = at<double>(ws, p.off_rs);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   // first pass, R only: R_1 = chol(A^T A) (a breakdown ends the call with that status)
   launch(SG_SYRK, 0, st, [&] {
     launch_syrk_oz(p.m, p.n, A, lda, p.oz, at<uint32_t>(ws, p.off_colhi), at<long long>(ws, p.off_ozpart), Rc, ctl, 0, st);
@@ -558,7 +560,7 @@ int mrcqr_cholqr2(int64_t m, int64_t n, const double* A, int64_t lda, double* Q,
   cudaMemcpyAsync(Rs, Rc, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, st);
   launch(SG_PREP, 0, st, [&] { launch_rs_prepare((int)n, Rs, at<double>(ws, p.off_rst), at<double>(ws, p.off_rinv), st); });
   enqueue_stage2(p, ws, A, lda, Q, ldq, R, ldr, 1, ctl, 0, st);
-  launch(SG_STATS, 0, st, [&] { { ::mrcqr::note_launch(); k_write_stats<<<1, 1, 0, st>>>(ctl, slot); } });
+  launch(SG_STATS, 0, st, [&] { launch_dep(k_write_stats, 1, 1, 0, st, ctl, slot); });
   cudaFreeAsync(ws, st);
   return finish(st);
 }
@@ -585,7 +587,7 @@ int mrcqr_regime_estimate(int64_t m, int64_t n, const double* A, int64_t lda, in
   double* rinv = at<double>(ws, p.off_rinv);
   uint32_t* colhi = at<uint32_t>(ws, p.off_colhi);
   long long* part = at<long long>(ws, p.off_ozpart);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   // G = A^T A (emulated FP64) and its Cholesky factor (a breakdown raises the level status)
   launch(SG_SYRK, 0, st, [&] { launch_syrk_oz(p.m, p.n, A, lda, p.oz, colhi, part, Rc, ctl, 0, st); });
   if (!probe) cudaMemcpyAsync(E, Rc, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, st);
@@ -623,11 +625,11 @@ int mrcqr_cholqr_precond(int64_t m, int64_t n, const double* A, int64_t lda, con
     return MRCQR_ERR_ALLOC;
   }
   Ctl* ctl = at<Ctl>(ws, p.off_ctl);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   cudaMemcpyAsync(at<double>(ws, p.off_rs), Rs, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, st);
   launch(SG_PREP, 0, st, [&] { launch_rs_prepare((int)n, Rs, at<double>(ws, p.off_rst), at<double>(ws, p.off_rinv), st); });
   enqueue_stage2(p, ws, A, lda, Q, ldq, R, ldr, 1, ctl, 0, st);
-  launch(SG_STATS, 0, st, [&] { { ::mrcqr::note_launch(); k_write_stats<<<1, 1, 0, st>>>(ctl, slot); } });
+  launch(SG_STATS, 0, st, [&] { launch_dep(k_write_stats, 1, 1, 0, st, ctl, slot); });
   cudaFreeAsync(ws, st);
   return finish(st);
 }
@@ -652,7 +654,7 @@ int mrcqr_trsm(int64_t m, int64_t n, const double* A, int64_t lda, const double*
   double* Rp = at<double>(ws, p.off_rs);
   double* RsT = at<double>(ws, p.off_rst);
   double* rinv = at<double>(ws, p.off_rinv);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   cudaMemcpy2DAsync(Rp, sizeof(double) * n, R, sizeof(double) * ldr, sizeof(double) * n, n, cudaMemcpyDeviceToDevice, st);
   launch(SG_PREP, 0, st, [&] { launch_rs_prepare((int)n, Rp, RsT, rinv, st); });
   if (fp64_products == 0)
@@ -681,7 +683,7 @@ int mrcqr_gram(int64_t m, int64_t n, const double* W, int64_t ldw, double* G, in
     return MRCQR_ERR_ALLOC;
   }
   Ctl* ctl = at<Ctl>(ws, p.off_ctl);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   if (fp64_products == 0) {
     launch(SG_SYRK, 0, st, [&] {
       launch_syrk_oz(m, (int)n, W, ldw, p.oz, at<uint32_t>(ws, p.off_colhi), at<long long>(ws, p.off_ozpart), G, ctl,
@@ -713,7 +715,7 @@ int mrcqr_finalize_q(int64_t m, int64_t n, double* Q, int64_t ldq, const double*
   }
   Ctl* ctl = at<Ctl>(ws, p.off_ctl);
   double* XT = at<double>(ws, p.off_xt);
-  launch(SG_INIT, 0, st, [&] { { ::mrcqr::note_launch(); k_init_ctl<<<1, 1, 0, st>>>(ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); } });
+  launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   launch(SG_PREP, 0, st, [&] { launch_upper_to_xt((int)n, X, ldx, XT, st); });
   if (fp64_products == 1)
     launch(SG_FINALIZE, 0, st, [&] { launch_finalize(m, (int)n, Q, ldq, XT, ctl, 0, st); });

@@ -486,7 +486,7 @@ void launch_col_hi(int64_t m, int n, const double* X, int64_t ldx, uint32_t* col
   const int64_t max_y = (m + 4095) / 4096;
   if (ysplit > max_y) ysplit = (int)max_y;
   if (ysplit < 1) ysplit = 1;
-  { ::mrcqr::note_launch(); k_col_hi<<<dim3(n, ysplit), 256, 0, st>>>(m, n, X, ldx, (m + ysplit - 1) / ysplit, colHi, ctl, level); }
+  launch_dep(k_col_hi, dim3(n, ysplit), 256, 0, st, m, n, X, ldx, (m + ysplit - 1) / ysplit, colHi, ctl, level);
 }
 }  // namespace
 
@@ -499,7 +499,7 @@ void launch_sketch_oz_reduce(int n, int s, const uint32_t* colHi, const uint32_t
                              const long long* part, double* Y, Ctl* ctl, int level, cudaStream_t st, int tf,
                              int64_t m) {
   const int64_t total = (int64_t)s * n;
-  { ::mrcqr::note_launch(); k_sketch_oz_reduce<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(n, s, colHi, idx, P, part, Y, ctl, level, tf, m); }
+  launch_dep(k_sketch_oz_reduce, (unsigned)((total + 255) / 256), 256, 0, st, n, s, colHi, idx, P, part, Y, ctl, level, tf, m);
 }
 
 SyrkOzPlan syrk_oz_plan(int64_t m, int n, int64_t rows_per_slab) {
@@ -534,10 +534,10 @@ void launch_syrk_oz(int64_t m, int n, const double* W, int64_t ldw, const SyrkOz
   if (!colhi_ready) launch_col_hi(m, n, W, ldw, colHi, ctl, level, st);
   set_smem(k_syrk_oz);
   const int nitems = P.ntiles * P.slabs;
-  { ::mrcqr::note_launch(); k_syrk_oz<<<nitems < num_sms() ? nitems : num_sms(), kOzThreads, kSmem, st>>>(m, n, W, ldw, colHi, P, part, ctl,
-                                                                               level); }
+  launch_dep(k_syrk_oz, nitems < num_sms() ? nitems : num_sms(), kOzThreads, kSmem, st, m, n, W, ldw, colHi, P, part, ctl,
+                                                                               level);
   const int64_t nn = (int64_t)n * n;
-  { ::mrcqr::note_launch(); k_syrk_oz_reduce<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(n, colHi, P, part, out, ctl, level); }
+  launch_dep(k_syrk_oz_reduce, (unsigned)((nn + 255) / 256), 256, 0, st, n, colHi, P, part, out, ctl, level);
 }
 
 
@@ -559,8 +559,8 @@ void launch_sketch_oz(int64_t m, int n, int s, const double* A, int64_t lda, con
   launch_col_hi(m, n, A, lda, colHi, ctl, level, st);
   set_smem(k_sketch_oz);
   const int nitems = P.mblocks * P.ntiles * P.slabs;
-  { ::mrcqr::note_launch(); k_sketch_oz<<<nitems < num_sms() ? nitems : num_sms(), kOzThreads, kSmem, st>>>(m, n, s, A, lda, colHi, idx, tab,
-                                                                                 seed_key(seed), P, part, ctl, level, tf); }
+  launch_dep(k_sketch_oz, nitems < num_sms() ? nitems : num_sms(), kOzThreads, kSmem, st, m, n, s, A, lda, colHi, idx, tab,
+                                                                                 seed_key(seed), P, part, ctl, level, tf);
   launch_sketch_oz_reduce(n, s, colHi, idx, P, part, Y, ctl, level, st, tf, m);
 }
 

@@ -341,18 +341,18 @@ bool launch_sketch_ozp(int64_t m, int n, int s, const double* A, int64_t lda, co
   }
   launch_oz_col_hi(m, n, A, lda, colHi, ctl, level, st);
   const int64_t tq = (m + 2) / 2;   // table entries 0 .. m, two per thread
-  { ::mrcqr::note_launch(); k_oz_tab_digits<<<(unsigned)((tq + 255) / 256), 256, 0, st>>>(m, tab, tabd, ctl, level); }
+  launch_dep(k_oz_tab_digits, (unsigned)((tq + 255) / 256), 256, 0, st, m, tab, tabd, ctl, level);
   const uint2 key = seed_key(seed);
   const int grid = items < sm_count() ? items : sm_count();
   for (int64_t k = 0; k < nch; ++k) {
     const int64_t row0 = k * R, mc = std::min(R, m - row0);
     const int64_t pairs = (mc + 1) / 2;
     const dim3 pg((unsigned)((pairs + 255) / 256), (unsigned)((n + kPlaneCols - 1) / kPlaneCols));
-    { ::mrcqr::note_launch(); k_oz_planes_a<<<pg, 256, 0, st>>>(row0, mc, n, A, lda, colHi, key,
-                                                                static_cast<uint32_t*>(scratch), R, ctl, level); }
-    { ::mrcqr::note_launch(); k_sketch_ozp<<<grid, kOzThreads, kSmem, st>>>(maps[(size_t)k], row0, mc, n, s, idx,
+    launch_dep(k_oz_planes_a, pg, 256, 0, st, row0, mc, n, A, lda, colHi, key,
+                                                                static_cast<uint32_t*>(scratch), R, ctl, level);
+    launch_dep(k_sketch_ozp, grid, kOzThreads, kSmem, st, maps[(size_t)k], row0, mc, n, s, idx,
                                                                               tabd, Pc, part + (size_t)k * items * kPartElems,
-                                                                              ctl, level, tf, m); }
+                                                                              ctl, level, tf, m);
   }
   SketchOzPlan Pall = Pc;
   Pall.slabs = Pc.slabs * (int)nch;

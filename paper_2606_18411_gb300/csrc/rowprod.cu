@@ -869,7 +869,7 @@ void rp_launch(const RpArgs& a, Ctl* ctl, int level, cudaStream_t st) {
   const unsigned grid = (unsigned)(nblocks < slots ? nblocks : slots);
   auto kernel = a.n > kRN * kGroupChunks ? k_rowprod<kTrsm, true> : k_rowprod<kTrsm, false>;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRSmem);
-  { ::mrcqr::note_launch(); kernel<<<grid, kRThreads, kRSmem, st>>>(a, ctl, level); }
+  launch_dep(kernel, grid, kRThreads, kRSmem, st, a, ctl, level);
 }
 
 unsigned rp_grid(int nitems, int per_sm) {
@@ -892,9 +892,9 @@ void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double
   const int n32 = rp_n32(n);
   const int nhi = (int)(syrk_oz_colhi_bytes(n) / sizeof(uint32_t));
   int *colE = ints, *eR = ints + n32, *flags = ints + 2 * n32;
-  if (n > kRpOwnScale) { ::mrcqr::note_launch(); k_rp_row_scale<<<(n + 7) / 8, 256, 0, st>>>(n, n32, RT, eR, ctl, level); }
+  if (n > kRpOwnScale) launch_dep(k_rp_row_scale, (n + 7) / 8, 256, 0, st, n, n32, RT, eR, ctl, level);
   cudaFuncSetAttribute(k_rp_prep_r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RpPrep));
-  { ::mrcqr::note_launch(); k_rp_prep_r<<<n32 / kRN, 256, sizeof(RpPrep), st>>>(n, n32, RT, rinv, eR, colE, flags, Rd, colHiOut, nhi, ctl, level); }
+  launch_dep(k_rp_prep_r, n32 / kRN, 256, sizeof(RpPrep), st, n, n32, RT, rinv, eR, colE, flags, Rd, colHiOut, nhi, ctl, level);
   const RpArgs a{m, n, A, lda, W, ldw, colE, Rd, eR, flags, RT, rinv, colHiOut};
   rp_launch<true>(a, ctl, level, st);
 }
@@ -903,7 +903,7 @@ void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* 
                         Ctl* ctl, int level, cudaStream_t st, uint32_t* colHiOut) {
   const int n32 = rp_n32(n);
   const int nhi = (int)(syrk_oz_colhi_bytes(n) / sizeof(uint32_t));
-  { ::mrcqr::note_launch(); k_rp_prep_x<<<n32, 128, 0, st>>>(n, n32, XT, colE, Xs, colHiOut, nhi, ctl, level); }
+  launch_dep(k_rp_prep_x, n32, 128, 0, st, n, n32, XT, colE, Xs, colHiOut, nhi, ctl, level);
   const RpArgs a{m, n, nullptr, 0, Q, ldq, colE, Xs, nullptr, nullptr, nullptr, nullptr, colHiOut};
   rp_launch<false>(a, ctl, level, st);
 }

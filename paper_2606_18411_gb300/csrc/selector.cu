@@ -56,83 +56,156 @@ __device__ double block_max_d(double v, double* red) {
 // once: FP64 division is a long sequence on this GPU's 1/64-rate pipe, and the
 // sweeps below would otherwise divide at every step in every thread.
 
-// y = M x (M = R or R diag(R)^-1), x and y in shared memory
-__device__ void mat_vec(const double* R, const double* rd, bool unit, int n, const double* x, double* y) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    double acc = 0.0;
-    for (int j = i; j < n; ++j) acc = fma(R[(int64_t)j * n + i] * (unit ? rd[j] : 1.0), x[j], acc);
-    y[i] = acc;
-  }
-  __syncthreads();
-}
+// The power iterations: one warp each, the vector in registers (lane l holds
+// entries l + 32 t), no block barriers.  Every sweep walks the columns of R
+// or rows of R with the loads of the next kD in flight and adds a multiple of
+// each: no sums over lanes, which cost five dependent FP64 additions (64 clocks
+// of the pipe each) a step.  M = R or, unit, R diag(R)^-1.  (By the
+// whole block, with two barriers and a strided or dependent load per step, the
+// twelve triangular sweeps took 400 us at n = 100: the kernel 413 us then, 217
+// now, most of it the dependent chain of the two inverse norms.)
+template <int NT>
+struct WarpTri {
+  static constexpr int kD = NT <= 8 ? 4 : 2;
+  const double* R;
+  const double *rd, *rdg;
+  int n, lane;
+  bool unit;
 
-// y = M^T x
-__device__ void mat_t_vec(const double* R, const double* rd, bool unit, int n, const double* x, double* y) {
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    double acc = 0.0;
-    for (int i = 0; i <= j; ++i) acc = fma(R[(int64_t)j * n + i], x[i], acc);
-    y[j] = unit ? acc * rd[j] : acc;
-  }
-  __syncthreads();
-}
-
-// x <- M^{-1} x (column sweep from the last column)
-__device__ void solve(const double* R, const double* rd, const double* rdg, bool unit, int n, double* x) {
-  for (int j = n - 1; j >= 0; --j) {
-    const double xj = unit ? x[j] : x[j] * rdg[j];
-    __syncthreads();
-    for (int i = threadIdx.x; i < j; i += blockDim.x)
-      x[i] = fma(-R[(int64_t)j * n + i] * (unit ? rd[j] : 1.0), xj, x[i]);
-    if (threadIdx.x == 0) x[j] = xj;
-    __syncthreads();
-  }
-}
-
-// x <- M^{-T} x (forward sweep)
-__device__ void solve_t(const double* R, const double* rd, const double* rdg, bool unit, int n, double* x) {
-  for (int j = 0; j < n; ++j) {
-    const double xj = unit ? x[j] : x[j] * rdg[j];
-    __syncthreads();
-    for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x)
-      x[i] = fma(-R[(int64_t)i * n + j] * (unit ? rd[i] : 1.0), xj, x[i]);
-    if (threadIdx.x == 0) x[j] = xj;
-    __syncthreads();
-  }
-}
-
-__device__ double vec_norm(const double* x, int n, double* red) {
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s = fma(x[i], x[i], s);
-  return sqrt(block_sum_d(s, red));
-}
-
-// 3-step power iteration for ||M|| (inverse = false) or ||M^{-1}|| (true).
-__device__ double power_norm(const double* R, const double* rd, const double* rdg, bool unit, bool inverse, int n,
-                             double* x, double* y, double* red) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = 1.0 / sqrt((double)n);
-  __syncthreads();
-  double nrm = 0.0;
-  for (int it = 0; it < 3; ++it) {
-    if (!inverse) {
-      mat_vec(R, rd, unit, n, x, y);
-      mat_t_vec(R, rd, unit, n, y, x);
-    } else {
-      solve(R, rd, rdg, unit, n, x);
-      solve_t(R, rd, rdg, unit, n, x);
+  __device__ __forceinline__ void load(int j, double (&v)[NT]) const {
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const int i = lane + 32 * t;
+      v[t] = j >= 0 && j < n && i <= j ? __ldg(R + (int64_t)j * n + i) : 0.0;
     }
-    nrm = vec_norm(x, n, red);
-    if (!(nrm > 0.0) || !isfinite(nrm)) return nrm;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] /= nrm;
-    __syncthreads();
   }
-  return sqrt(nrm);
-}
 
+  // y = M x
+  __device__ void mul(const double (&x)[NT], double (&y)[NT]) const {
+#pragma unroll
+    for (int t = 0; t < NT; ++t) y[t] = 0.0;
+    double v[kD][NT];
+#pragma unroll
+    for (int d = 0; d < kD; ++d) load(d, v[d]);
+#pragma unroll
+    for (int tb = 0; tb < NT; ++tb)
+#pragma unroll 1
+      for (int l = 0; l < 32 && 32 * tb + l < n; l += kD)
+#pragma unroll
+        for (int d = 0; d < kD; ++d) {
+          const int j = 32 * tb + l + d;   // columns beyond n are zero
+          const double f = __shfl_sync(0xffffffffu, x[tb], l + d) * (unit && j < n ? rd[j] : 1.0);
+#pragma unroll
+          for (int t = 0; t <= tb; ++t) y[t] = fma(v[d][t], f, y[t]);
+          load(j + kD, v[d]);
+        }
+  }
+
+  // row i: entry t is R[i][lane + 32 t] (a strided load; 16 consecutive rows hit its line in L1)
+  __device__ __forceinline__ void load_row(int i, double (&v)[NT]) const {
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const int j = lane + 32 * t;
+      v[t] = j < n && i <= j ? __ldg(R + (int64_t)j * n + i) : 0.0;
+    }
+  }
+
+  // y = M^T x (solve = false) or y = M^{-T} x
+  __device__ void transposed(const double (&x)[NT], double (&y)[NT], bool solve) const {
+    double own[NT];   // this lane's reciprocal diagonals
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const int j = lane + 32 * t;
+      own[t] = j >= n ? 0.0 : unit ? rd[j] : solve ? rdg[j] : 1.0;
+      y[t] = 0.0;   // sums over the rows so far
+    }
+    double v[kD][NT];
+#pragma unroll
+    for (int d = 0; d < kD; ++d) load_row(d, v[d]);
+#pragma unroll
+    for (int tb = 0; tb < NT; ++tb) {
+#pragma unroll 1
+      for (int l = 0; l < 32 && 32 * tb + l < n; l += kD)
+#pragma unroll
+        for (int d = 0; d < kD; ++d) {
+          const int i = 32 * tb + l + d;   // rows beyond n are zero
+          double z = x[tb];
+          if (solve) z = unit ? fma(-own[tb], y[tb], z) : (z - y[tb]) * own[tb];
+          const double f = __shfl_sync(0xffffffffu, z, l + d);
+#pragma unroll
+          for (int t = tb; t < NT; ++t) {
+            if (!solve) y[t] = fma(v[d][t], f, y[t]);
+            else if (lane + 32 * t > i) y[t] = fma(v[d][t], f, y[t]);
+            else if (lane + 32 * t == i) y[t] = f;
+          }
+          load_row(i + kD, v[d]);
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+      if (!solve) y[t] *= own[t];
+  }
+
+  // x <- M^{-1} x
+  __device__ void solve(double (&x)[NT]) const {
+    const int last = (n + kD - 1) / kD * kD - 1;   // columns beyond n are zero and do nothing
+    double v[kD][NT];
+#pragma unroll
+    for (int d = 0; d < kD; ++d) load(last - d, v[d]);
+#pragma unroll
+    for (int tb = NT - 1; tb >= 0; --tb)
+#pragma unroll 1
+      for (int l = min(31, last - 32 * tb); l >= 0; l -= kD)
+#pragma unroll
+        for (int d = 0; d < kD; ++d) {
+          const int j = 32 * tb + l - d;
+          const double b = __shfl_sync(0xffffffffu, x[tb], l - d);
+          const double xj = unit ? b : b * (j < n ? rdg[j] : 0.0), f = unit ? b * (j < n ? rd[j] : 0.0) : xj;
+#pragma unroll
+          for (int t = 0; t <= tb; ++t)
+            if (lane + 32 * t < j) x[t] = fma(-v[d][t], f, x[t]);
+          if (lane == l - d) x[tb] = xj;
+          load(j - kD, v[d]);
+        }
+  }
+
+  // 3-step power iteration for ||M|| (inverse = false) or ||M^{-1}|| (true)
+  __device__ double power_norm(bool inverse) const {
+    double x[NT], y[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) x[t] = lane + 32 * t < n ? 1.0 / sqrt((double)n) : 0.0;
+    double nrm = 0.0;
+#pragma unroll 1
+    for (int it = 0; it < 3; ++it) {
+      if (!inverse) {
+        mul(x, y);
+        transposed(y, x, false);
+      } else {
+        solve(x);
+        transposed(x, y, true);
+#pragma unroll
+        for (int t = 0; t < NT; ++t) x[t] = y[t];
+      }
+      double s = 0.0;
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+        if (lane + 32 * t < n) s = fma(x[t], x[t], s);
+      nrm = sqrt(warp_sum(s));
+      if (!(nrm > 0.0) || !isfinite(nrm)) return nrm;
+#pragma unroll
+      for (int t = 0; t < NT; ++t) x[t] /= nrm;
+    }
+    return sqrt(nrm);
+  }
+};
+
+template <int NT>
 __global__ void __launch_bounds__(kFeatThreads) k_features(const double* __restrict__ R, int n, int64_t m,
                                                           float* __restrict__ out, const Ctl* ctl, int level) {
+  wait_prior_kernels();
   if (ctl && (ctl->active != level || ctl->lvl_status != 0)) return;
-  __shared__ double d[kMaxN], L[kMaxN], Ls[kMaxN], x[kMaxN], y[kMaxN], rd[kMaxN], rdg[kMaxN];
-  __shared__ double red[33];
+  __shared__ double d[kMaxN], L[kMaxN], Ls[kMaxN], rd[kMaxN], rdg[kMaxN];
+  __shared__ double red[33], norms[4];
   const double tiny = 2.2250738585072014e-308;
   const int tid = threadIdx.x;
   for (int i = tid; i < kMaxN; i += blockDim.x) {
@@ -148,9 +221,11 @@ __global__ void __launch_bounds__(kFeatThreads) k_features(const double* __restr
   }
   __syncthreads();
   // bitonic sort of Ls (ascending, padding +inf last)
-  for (int k = 2; k <= kMaxN; k <<= 1)
+  int nsort = 2;
+  while (nsort < n) nsort <<= 1;
+  for (int k = 2; k <= nsort; k <<= 1)
     for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = tid; i < kMaxN; i += blockDim.x) {
+      for (int i = tid; i < nsort; i += blockDim.x) {
         const int l = i ^ j;
         if (l > i) {
           const double a = Ls[i], b = Ls[l];
@@ -172,27 +247,30 @@ __global__ void __launch_bounds__(kFeatThreads) k_features(const double* __restr
   const double lstd = sqrt(block_sum_d(dev, red) / n);
   const double gapm = block_sum_d(gap, red) / n;
   const double dmax = pow(10.0, lmax);
-  // condition estimates of R and of R diag(R)^-1
-  const double nr = power_norm(R, rd, rdg, false, false, n, x, y, red);
-  const double ni = power_norm(R, rd, rdg, false, true, n, x, y, red);
-  const double ur = power_norm(R, rd, rdg, true, false, n, x, y, red);
-  const double ui = power_norm(R, rd, rdg, true, true, n, x, y, red);
-  // column norms, off-diagonal mass, noise-floor fractions
   double cmax = 0.0, cmin = INFINITY, off = 0.0, dsq = 0.0, f16 = 0.0, f32 = 0.0;
-  for (int j = tid; j < n; j += blockDim.x) {
-    double c = 0.0;
-    for (int i = 0; i <= j; ++i) {
-      const double v = R[(int64_t)j * n + i];
-      c = fma(v, v, c);
-      if (i < j) off = fma(v, v, off);
+  // condition estimates of R and of R diag(R)^-1
+  if (tid < 128) {   // warps 0 .. 3: ||R||, ||R^-1||, ||U||, ||U^-1||
+    const int w = tid >> 5;
+    const WarpTri<NT> M{R, rd, rdg, n, tid & 31, w >= 2};
+    const double v = M.power_norm((w & 1) != 0);
+    if ((tid & 31) == 0) norms[w] = v;
+  } else {   // the other warps: column norms, off-diagonal mass, noise-floor fractions
+    for (int j = tid - 128; j < n; j += kFeatThreads - 128) {
+      double c = 0.0;
+      const double* col = R + (int64_t)j * n;
+#pragma unroll 8
+      for (int i = 0; i < j; ++i) c = fma(col[i], col[i], c);
+      off += c;
+      c = sqrt(fma(col[j], col[j], c));
+      cmax = fmax(cmax, c);
+      cmin = fmin(cmin, c);
+      dsq = fma(d[j], d[j], dsq);
+      f16 += d[j] < ldexp(dmax, -11) ? 1.0 : 0.0;
+      f32 += d[j] < ldexp(dmax, -20) ? 1.0 : 0.0;
     }
-    c = sqrt(c);
-    cmax = fmax(cmax, c);
-    cmin = fmin(cmin, c);
-    dsq = fma(d[j], d[j], dsq);
-    f16 += d[j] < ldexp(dmax, -11) ? 1.0 : 0.0;
-    f32 += d[j] < ldexp(dmax, -20) ? 1.0 : 0.0;
   }
+  __syncthreads();
+  const double nr = norms[0], ni = norms[1], ur = norms[2], ui = norms[3];
   cmax = block_max_d(cmax, red);
   cmin = -block_max_d(-cmin, red);
   off = block_sum_d(off, red);
@@ -291,6 +369,7 @@ __device__ int expected_cost_choice(const float* z, const float* costs) {
 
 // AUTO: choose the start of the ladder (levels 0/1/2 = fp16/fp32/fp64).
 __global__ void __launch_bounds__(64) k_mlp_select(Sel S, const float* __restrict__ feat, Ctl* ctl) {
+  wait_prior_kernels();
   if (ctl->active != 0 || ctl->lvl_status != 0) return;
   __shared__ float xs[kF], h1[kH], h2[kH], a1[kH], a2[kH], z[kC];
   mlp_forward64(S, feat, xs, h1, h2, a1, a2, z);
@@ -450,7 +529,8 @@ int selector_set(const float* params, const float* mu, const float* sd, const fl
 }
 
 void launch_features(const double* Rs, int n, int64_t m, float* out, const Ctl* ctl, int level, cudaStream_t st) {
-  { ::mrcqr::note_launch(); k_features<<<1, kFeatThreads, 0, st>>>(Rs, n, m, out, ctl, level); }
+  auto kernel = n <= 64 ? k_features<2> : n <= 128 ? k_features<4> : n <= 256 ? k_features<8> : k_features<16>;
+  launch_dep(kernel, dim3(1), kFeatThreads, 0, st, Rs, n, m, out, ctl, level);
 }
 
 bool launch_mlp_select(const float* feat, Ctl* ctl, cudaStream_t st) {
@@ -462,7 +542,7 @@ bool launch_mlp_select(const float* feat, Ctl* ctl, cudaStream_t st) {
     if (dev >= (int)g_sel.size() || !g_sel[dev].w) return false;
     S = Sel{g_sel[dev].w, g_sel[dev].aux, g_sel[dev].aux + 16, g_sel[dev].aux + 32};
   }
-  { ::mrcqr::note_launch(); k_mlp_select<<<1, 64, 0, st>>>(S, feat, ctl); }
+  launch_dep(k_mlp_select, dim3(1), 64, 0, st, S, feat, ctl);
   return true;
 }
 

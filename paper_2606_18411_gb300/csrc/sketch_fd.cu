@@ -593,10 +593,10 @@ void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, con
   uint32_t* sgn = reinterpret_cast<uint32_t*>(slots + kFdTile * p.max_tiles);
   cudaMemsetAsync(colHi, 0, syrk_oz_colhi_bytes(n), st);
   cudaMemsetAsync(colU, 0, sizeof(int) * 512, st);
-  { ::mrcqr::note_launch(); k_fd_bounds<<<dim3((unsigned)((p.J + 255) / 256), (unsigned)n), 256, 0, st>>>(p.J, A, lda, colHi, colU, ctl, level); }
-  { ::mrcqr::note_launch(); k_fd_table<<<(unsigned)((m + 256) / 256), 256, 0, st>>>(m, tabd, ctl, level); }
-  { ::mrcqr::note_launch(); k_fd_signs<<<(unsigned)((p.J + 31) / 32), 256, 0, st>>>(p.J, seed_key(seed), sgn, ctl, level); }
-  { ::mrcqr::note_launch(); k_fd_classes<<<1, 1024, 0, st>>>(s, idx, ntiles, cls, slots, ctl, level); }
+  launch_dep(k_fd_bounds, dim3((unsigned)((p.J + 255) / 256), (unsigned)n), 256, 0, st, p.J, A, lda, colHi, colU, ctl, level);
+  launch_dep(k_fd_table, (unsigned)((m + 256) / 256), 256, 0, st, m, tabd, ctl, level);
+  launch_dep(k_fd_signs, (unsigned)((p.J + 31) / 32), 256, 0, st, p.J, seed_key(seed), sgn, ctl, level);
+  launch_dep(k_fd_classes, 1, 1024, 0, st, s, idx, ntiles, cls, slots, ctl, level);
   cudaFuncSetAttribute(k_fd_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFdSmem);
   cudaFuncSetAttribute(k_fd_pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFdSmem);
   uint64_t* U = static_cast<uint64_t*>(scratch);
@@ -604,15 +604,14 @@ void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, con
     const int64_t j0 = (int64_t)k * p.Jc;
     const int nblocks = (int)(p.Jc / kM);   // rows j1 >= J give zero words
     const int64_t items = (int64_t)nblocks * n;
-    { ::mrcqr::note_launch(); k_fd_pass1<<<(unsigned)std::min<int64_t>(items, 2 * fd_sms()), kRThreads, kFdSmem, st>>>(
-        p.J, j0, p.Jc, nblocks, n, A, lda, colHi, colU, sgn, U, ctl, level); }
+    launch_dep(k_fd_pass1, (unsigned)std::min<int64_t>(items, 2 * fd_sms()), kRThreads, kFdSmem, st, p.J, j0, p.Jc, nblocks, n, A, lda, colHi, colU, sgn, U, ctl, level);
     const Fd2Args a{m, p.J, j0, p.Jc, p.rows, n, p.cblocks, p.slabs, U, idx, tabd, ntiles, cls, slots, part,
                     k * p.slabs, p.slabs * p.chunks};
     const int64_t most = (int64_t)p.max_tiles * p.cblocks * p.slabs;
-    { ::mrcqr::note_launch(); k_fd_pass2<<<(unsigned)std::min<int64_t>(most, 2 * fd_sms()), kRThreads, kFdSmem, st>>>(a, ctl, level); }
+    launch_dep(k_fd_pass2, (unsigned)std::min<int64_t>(most, 2 * fd_sms()), kRThreads, kFdSmem, st, a, ctl, level);
   }
   const dim3 rg((unsigned)(kFdTile * p.max_tiles / 2), (unsigned)p.cblocks);
-  { ::mrcqr::note_launch(); k_fd_reduce<<<rg, 256, 0, st>>>(n, s, p.cblocks, p.slabs * p.chunks, ntiles, slots, colHi, colU, idx, part, Y, ctl, level); }
+  launch_dep(k_fd_reduce, rg, 256, 0, st, n, s, p.cblocks, p.slabs * p.chunks, ntiles, slots, colHi, colU, idx, part, Y, ctl, level);
 }
 
 }  // namespace mrcqr
