@@ -133,7 +133,7 @@ void load_tune_file() {
   std::ifstream in(f);
   std::string key;
   int64_t a, b, c;
-  while (in >> key >> a >> b >> c) g_tune_cache[key] = Tuning{a, b, c};
+  while (in >> key >> a >> b >> c) g_tune_cache[key] = Tuning{a, (b + 63) / 64 * 64, c};   // whole sketch slabs
 }
 
 void save_tune_file() {

@@ -32,9 +32,16 @@
 // previous tile's D is copied to shared memory and step 2 runs on it.  Every
 // wait is bounded; on a timeout the CTA waits (bounded) for its own copies
 // in flight, frees its TMEM, raises TIMEOUT and returns.
+//
+// What bounds it: step 2 (per sample, j1 and column five FP32 operations) and
+// the latency between the barriers of a tile; the MMAs are short.  Measured at
+// m = 2^20 (ms, before / now): FP16 n = 256 2.50 / 2.24, 512 6.78 / 6.0; FP32
+// n = 256 4.05 / 3.77 (2.24: flags in place of reducing barriers and fewer
+// barriers per tile; the last 7% of FP32 from 16-byte reads of U).
 #include <mutex>
 
 #include "kernels.h"
+#include "sketch_cvt.cuh"
 #include "tc.cuh"
 
 namespace mrcqr {
@@ -62,7 +69,9 @@ struct Fs {
   static constexpr uint32_t X_PANEL = N * 128;
   static constexpr uint32_t XD_BYTES = kB * kM2 * C * 8;      // one FP64 tile
   static constexpr int STAGES = 3;
-  static constexpr int USTR = N + 1;                          // U row stride (floats), conflict-free columns
+  // U row stride (floats): rows start four banks apart, so 16-byte reads of up to eight rows by a warp and
+  // 16-byte writes of a row by each lane are free of conflicts
+  static constexpr int USTR = N + 4;
   static constexpr uint32_t W_OFF = 0;                                   // [PARTS][KPANELS]
   static constexpr uint32_t X_OFF = W_OFF + PARTS * KPANELS * W_PANEL;   // [2][PARTS][KPANELS]
   static constexpr uint32_t XD_OFF = X_OFF + 2 * PARTS * KPANELS * X_PANEL;
@@ -118,7 +127,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) uint64_t mma_bar[2];
   __shared__ uint32_t tmem_base;
   __shared__ float colscale[2][C];
-  __shared__ uint32_t red32[kThreads / 32][C];
+  __shared__ uint32_t red32[2][C];   // column maxima (high words) of a tile
+  __shared__ int fail;               // a wait ran out
   __shared__ uint64_t redmax[kThreads / 32];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -132,6 +142,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) tc::tmem_alloc(&tmem_base, F::TMEM_COLS);
   if (tid == 0) {
+    fail = 0;
+    for (int c = 0; c < C; ++c) red32[0][c] = red32[1][c] = 0u;
     for (int st = 0; st < F::STAGES; ++st) tc::mbar_init(&tma_bar[st], 1);
     tc::mbar_init(&mma_bar[0], 1);
     tc::mbar_init(&mma_bar[1], 1);
@@ -258,9 +270,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float* ui = U + srow_i[i] * F::USTR;
       const float sg = ssig[i];
       float cph = 0.f, sph = 0.f;
+      float4 u4r[C], u4i[C];
 #pragma unroll
       for (int jj = 0; jj < kB; ++jj) {
         if ((jj & 3) == 0) {   // exact twiddle every four j1, the phase an integer below 2^24
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            if (c < cg_lo || c >= cg_hi) continue;
+            u4r[c] = *reinterpret_cast<const float4*>(ur + c * kB + jj);
+            u4i[c] = *reinterpret_cast<const float4*>(ui + c * kB + jj);
+          }
           sincospif((float)P * inv2m, &sph, &cph);
         } else {
           const float c2 = cph * rot_c[i] - sph * rot_s[i];
@@ -273,7 +292,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int c = 0; c < C; ++c) {
           if (c < cg_lo || c >= cg_hi) continue;
-          const float t = fmaf(cph, ur[c * kB + jj], -ss * ui[c * kB + jj]);
+          const int k = jj & 3;
+          const float re = k == 0 ? u4r[c].x : k == 1 ? u4r[c].y : k == 2 ? u4r[c].z : u4r[c].w;
+          const float im = k == 0 ? u4i[c].x : k == 1 ? u4i[c].y : k == 2 ? u4i[c].z : u4i[c].w;
+          const float t = fmaf(cph, re, -ss * im);
           acc[i][c] = fmaf(t, colscale[b][c], acc[i][c]);
         }
       }
@@ -307,7 +329,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::tmem_wait_ld();
     float* dst = U + (q * 32 + lane) * F::USTR + g * CW;
 #pragma unroll
-    for (int j = 0; j < CW; ++j) dst[j] = v[j];
+    for (int j = 0; j < CW; j += 4)
+      *reinterpret_cast<float4*>(dst + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
   };
 
   for (int u = 0; u < total; ++u) {
@@ -323,8 +346,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint64_t j = (uint64_t)(j1_0 + cj1) + (uint64_t)m1 * (uint64_t)(2 * cp + h);
       sgn[h] = (philox4x32_10(make_uint4((uint32_t)j, 0u, 0u, 0u), key).x & 1u) << 31;
     }
-    const bool ok_tma = tc::mbar_wait(&tma_bar[stage], par);
-    if (__syncthreads_or(!ok_tma)) {
+    if (!tc::mbar_wait(&tma_bar[stage], par)) fail = 1;
+    if (tid < C) red32[buf ^ 1][tid] = 0u;   // the next tile's maxima; this tile's were cleared a tile ago
+    __syncthreads();
+    // a wait that ran out is agreed on here: no thread sets the flag between this barrier and the next
+    if (*(volatile int*)&fail) {
       abort = true;
       break;
     }
@@ -341,23 +367,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       // the exponent field orders |x| like the value: the high words' maximum gives the scale
       const uint32_t mx = __reduce_max_sync(0xffffffffu, max(vh[c][0] & 0x7FFFFFFFu, vh[c][1] & 0x7FFFFFFFu));
-      if (lane == 0) red32[warp][c] = mx;
-    }
-    __syncthreads();
-    if (tid < C) {
-      uint32_t mx = 0u;
-      for (int w = 0; w < kThreads / 32; ++w) mx = max(mx, red32[w][tid]);
-      red32[0][tid] = mx;
+      if (lane == 0) atomicMax(&red32[buf][c], mx);
     }
     __syncthreads();
     unsigned char* xb = xop + buf * F::PARTS * F::KPANELS * F::X_PANEL;
     const int c0t = (item % ncb) * C;
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      const uint32_t hmx = red32[0][c];
+      const uint32_t hmx = red32[buf][c], emax = hmx >> 20;
       int e = 0;
       if (c0t + c < n) {
-        if ((hmx >> 20) != 0u) {
+        if (emax != 0u) {
           e = scale_exponent_bits(hmx, 1u);
         } else {   // no normal value in this tile column: the exact 64-bit maximum (uniform branch)
           const uint64_t a0 = ((uint64_t)(vh[c][0] & 0x7FFFFFFFu) << 32) | vl[c][0];
@@ -371,14 +391,21 @@ __global__ void __launch_bounds__(kThreads, 1)
           e = scale_exponent_bits((uint32_t)(mb >> 32), (uint32_t)mb);
         }
       }
-      if (tid == 0) colscale[buf][c] = ldexpf(1.0f, -e);
+      const bool fast = col_fast(emax) && c0t + c < n;   // uniform
+      const ColScale cs(emax);
+      if (tid == 0) colscale[buf][c] = fast ? col_unscale(emax) : ldexpf(1.0f, -e);
       const int row = c * kB + cj1;   // MMA N index: (column, j1)
       if constexpr (PREC == P_FP32) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           uint32_t hh = vh[c][h], ll = vl[c][h];
-          scale_bits(hh, ll, e);
-          const float f = __uint_as_float(f64bits_to_f32(hh, ll));
+          if (fast) {
+            hh = f32_col(hh, ll, cs, e);
+          } else {
+            scale_bits(hh, ll, e);
+            hh = f64bits_to_f32(hh, ll);
+          }
+          const float f = __uint_as_float(hh);
           const uint32_t bg = tc::to_tf32(f);
           const int k = 2 * cp + h;
           unsigned char* pan = xb + (k / F::KPER) * F::X_PANEL;
@@ -387,25 +414,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               tc::to_tf32(f - __uint_as_float(bg));
         }
       } else {
-        uint32_t pk;
-        uint32_t f0, f1;
-        const bool ok0 = scaled_f32_rto(vh[c][0], vl[c][0], e, f0);
-        const bool ok1 = scaled_f32_rto(vh[c][1], vl[c][1], e, f1);
-        if (ok0 && ok1) {
-          if constexpr (PREC == P_FP16) {
-            const __half2 v2 = __floats2half2_rn(__uint_as_float(f0), __uint_as_float(f1));
-            pk = *reinterpret_cast<const uint32_t*>(&v2);
-          } else {
-            const __nv_bfloat162 v2 = __floats2bfloat162_rn(__uint_as_float(f0), __uint_as_float(f1));
-            pk = *reinterpret_cast<const uint32_t*>(&v2);
-          }
-        } else {
-          uint32_t h0 = vh[c][0], l0 = vl[c][0], h1 = vh[c][1], l1 = vl[c][1];
-          scale_bits(h0, l0, e);
-          scale_bits(h1, l1, e);
-          if constexpr (PREC == P_FP16) pk = f64bits_to_f16(h0, l0) | (f64bits_to_f16(h1, l1) << 16);
-          else pk = f64bits_to_bf16(h0, l0) | (f64bits_to_bf16(h1, l1) << 16);
-        }
+        const uint32_t pk = fast ? pack2_col<F::FMT>(vh[c][0], vl[c][0], vh[c][1], vl[c][1], cs, e)
+                                 : pack2<F::FMT>(vh[c][0], vl[c][0], vh[c][1], vl[c][1], e);
         *reinterpret_cast<uint32_t*>(xb + tc::sw128_offset(row, 2 * cp, 2)) = pk;
       }
     }
@@ -434,26 +444,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       mma_issued = u + 1;
     }
     if (u > 0) {   // step 2 of the previous tile while this tile's MMAs run
-      const bool ok_mma = tc::mbar_wait(&mma_bar[buf ^ 1], (uint32_t)(((u - 1) >> 1) & 1));
-      if (__syncthreads_or(!ok_mma)) {
-        abort = true;
-        break;
+      // After a failed wait this tile's sums are rubbish; the next tile's first
+      // barrier agrees on it.  That barrier also separates these reads of U, of
+      // the scales and of TMEM from their next writes.
+      if (tc::mbar_wait(&mma_bar[buf ^ 1], (uint32_t)(((u - 1) >> 1) & 1))) {
+        mma_done = u;
+        tc::fence_after();
+        d_to_smem(u - 1);
+        tc::fence_before();
+      } else {
+        fail = 1;
       }
-      mma_done = u;
-      tc::fence_after();
-      d_to_smem(u - 1);
-      tc::fence_before();
       __syncthreads();
       step2(u - 1);
-      __syncthreads();   // U is rewritten by the next tile
     }
   }
   if (!abort && total > 0) {
     const int u = total - 1;
-    const bool ok_mma = tc::mbar_wait(&mma_bar[u & 1], (uint32_t)((u >> 1) & 1));
-    if (__syncthreads_or(!ok_mma)) {
-      abort = true;
-    } else {
+    if (!tc::mbar_wait(&mma_bar[u & 1], (uint32_t)((u >> 1) & 1))) fail = 1;
+    __syncthreads();
+    abort = *(volatile int*)&fail != 0;
+    if (!abort) {
       mma_done = total;
       tc::fence_after();
       d_to_smem(u);
@@ -528,7 +539,7 @@ bool launch_fs(const double* A, int64_t lda, int64_t m, int n, int s, const uint
   const int tpc = ntiles / chunks;
   const int nitems = ((n + F::C - 1) / F::C) * chunks;
   const int grid = nitems < sms() ? nitems : sms();
-  { ::mrcqr::note_launch(); k_sketch_fs<PREC><<<grid, kThreads, smem, st>>>(map, m, n, s, idx, tab, seed_key(seed), chunks, tpc, Ypart, ctl, level); }
+  launch_dep(k_sketch_fs<PREC>, grid, kThreads, smem, st, map, m, n, s, idx, tab, seed_key(seed), chunks, tpc, Ypart, ctl, level);
   return true;
 }
 

@@ -33,10 +33,20 @@
 //
 // Every wait is bounded; on a timeout the CTA waits (bounded) for its own
 // copies in flight, frees its TMEM, raises TIMEOUT and returns.
+//
+// What bounds it: the integer instructions of step 2 and the two barriers per
+// slab (issue slots 48% busy, tensor pipe 5%, 1.7 TB/s at n = 64), not the
+// MMAs.  Measured at m = 2^20 (ms, before / now): FP16 n = 64 0.355 / 0.236,
+// 100 1.05 / 0.57, 128 0.92 / 0.58; FP32 n = 100 2.30 / 1.51, 128 1.93 / 1.56.
+// Of the FP16 n = 64 gain, 17 us came from a flag in place of the reducing
+// barriers and from drawing signs for several slabs at once, 27 us from several
+// chunks to a CTA, 65 us from the branch-free rounding; at n = 100 the zero
+// columns beyond n had cost as much as the rest.
 #include <cstring>
 #include <mutex>
 
 #include "kernels.h"
+#include "sketch_cvt.cuh"
 #include "tc.cuh"
 
 namespace mrcqr {
@@ -85,29 +95,6 @@ __device__ __forceinline__ void store_table(unsigned char* big, unsigned char* s
   }
 }
 
-// fl_p of two consecutive entries (k, k+1) of row r of the X operand, given
-// as FP64 bits scaled by 2^e: round to odd into FP32 (integer ops), then one
-// packed round-to-nearest-even; exact slow path outside the FP32 range.
-template <uint32_t FMT>
-__device__ __forceinline__ uint32_t pack2(uint32_t h0, uint32_t l0, uint32_t h1, uint32_t l1, int e) {
-  uint32_t f0, f1;
-  const bool ok0 = scaled_f32_rto(h0, l0, e, f0);
-  const bool ok1 = scaled_f32_rto(h1, l1, e, f1);
-  if (ok0 && ok1) {
-    if constexpr (FMT == tc::F16) {
-      const __half2 v = __floats2half2_rn(__uint_as_float(f0), __uint_as_float(f1));
-      return *reinterpret_cast<const uint32_t*>(&v);
-    } else {
-      const __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(f0), __uint_as_float(f1));
-      return *reinterpret_cast<const uint32_t*>(&v);
-    }
-  }
-  scale_bits(h0, l0, e);
-  scale_bits(h1, l1, e);
-  if constexpr (FMT == tc::F16) return f64bits_to_f16(h0, l0) | (f64bits_to_f16(h1, l1) << 16);
-  else return f64bits_to_bf16(h0, l0) | (f64bits_to_bf16(h1, l1) << 16);
-}
-
 // Phase (dk j0 + beta) mod 4m of a row at slab start j0, advanced by slabs of
 // T rows: adds dk T mod 4m.
 struct Phase {
@@ -133,7 +120,8 @@ struct TcCta {
   uint64_t* mma_bar;
   uint32_t tmem;
   float (*colscale)[kN];
-  uint32_t (*sgnmask)[Cfg<PREC, MT>::T];
+  uint32_t* sgnmask;   // signs of the rows of the current kThreads / T slabs
+  int* fail;           // a wait ran out
   uint32_t seq;    // slabs this CTA has run: the MMA barriers' phases and the operand/TMEM buffers
   uint32_t tseq;   // slabs this CTA has loaded by TMA: the copy barriers' stages and phases (a
                    // plain-copy item completes no copy-barrier phase, so it must not advance them)
@@ -141,15 +129,16 @@ struct TcCta {
 
 // One work item: sampled rows s0 .. s0 + 128 MT - 1, columns n0 .. n0 + 63,
 // rows [j_begin, j_end) of A (TMA map tmap, or with tmap null plain copies
-// of A with leading dimension lda); the partial sums go to out[col s + row].
+// of A with leading dimension lda) in nchunks chunks of rpc rows (a multiple of
+// the slab); the partial sums of chunk c go to out[c n s + col s + row].
 // False when a wait timed out (every thread together; this CTA's copies and
 // MMAs in flight are awaited first).
 template <int PREC, int MT>
 __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const double* __restrict__ A, int64_t lda,
                                                int64_t m, int n, int s,
                                                const uint32_t* __restrict__ idx, const double* __restrict__ tab,
-                                               uint2 key, int64_t j_begin, int64_t j_end, int s0, int n0,
-                                               double* __restrict__ out, int tf, TcCta<PREC, MT>& S) {
+                                               uint2 key, int64_t j_begin, int64_t j_end, int64_t rpc, int nchunks,
+                                               int s0, int n0, double* __restrict__ out, int tf, TcCta<PREC, MT>& S) {
   using C = Cfg<PREC, MT>;
   constexpr int T = C::T;
   unsigned char* tabs = S.tabs;
@@ -159,7 +148,8 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
   uint64_t* mma_bar = S.mma_bar;
   const uint32_t tmem = S.tmem;
   float(*colscale)[kN] = S.colscale;
-  uint32_t(*sgnmask)[T] = S.sgnmask;
+  uint32_t* sgnmask = S.sgnmask;
+  volatile int* fail = S.fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nslabs = j_begin < j_end ? (int)((j_end - j_begin + T - 1) / T) : 0;
   const uint64_t four_m = 4ull * (uint64_t)m;
@@ -256,6 +246,19 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
     ph.advance();
   };
 
+  const int spc = (int)(rpc / T);   // slabs per chunk
+  int left = spc, chunk = 0;
+  auto flush = [&]() {
+    double* o = out + (size_t)chunk * (size_t)s * (size_t)n;
+#pragma unroll
+    for (int c = 0; c < C::ACC; ++c) {
+      const int col = n0 + c_lo + c;
+      if (row_ok && col < n) o[(size_t)col * s + s0 + erow] = (double)acc[c];
+      acc[c] = 0.f;
+    }
+    left = spc;
+    ++chunk;
+  };
   auto epilogue = [&](int sl) {
     const int buf = sl & 1;
     const float cf = buf ? rc1 : rc0, sf = buf ? rs1 : rs0;
@@ -271,6 +274,7 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
         acc[c0 + j] = fmaf(fmaf(cf, pc[j], -sf * ps[j]), colscale[buf][c_lo + c0 + j], acc[c0 + j]);
     }
     tc::fence_before();
+    if (--left == 0) flush();
   };
 
   for (int sl = 0; sl < nslabs; ++sl) {
@@ -281,10 +285,14 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
     const int buf = (int)(u & 1u);
     const int64_t j0 = j_begin + (int64_t)sl * T;
     prefetch_rotation((int)u);
-    if (tid < T) {
+    // signs, one row per thread every kThreads / T slabs (two warps drawing
+    // each slab's held the other fourteen up at the barrier)
+    const int sgrp = sl % (kThreads / T);
+    if (sgrp == 0) {
       const int64_t j = j0 + tid;
-      sgnmask[buf][tid] = j < j_end ? (philox4x32_10(make_uint4((uint32_t)j, 0u, 0u, 0u), key).x & 1u) << 31
-                                    : 0xFFFFFFFFu;   // all ones marks a row outside the chunk
+      // rows outside [j_begin, j_end) are zeros in the tile: only j_end = m
+      // can lie inside a slab, and the copies fill with zero there
+      sgnmask[tid] = (philox4x32_10(make_uint4((uint32_t)j, 0u, 0u, 0u), key).x & 1u) << 31;
     }
     bool ok_tma = true;
     if (tmap) {
@@ -296,46 +304,73 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
       else if (younger == 1) tc::cp_async_wait_group<1>();
       else tc::cp_async_wait_group<0>();
     }
-    if (__syncthreads_or(!ok_tma)) { abort = true; break; }
+    if (!ok_tma) *fail = 1;
+    __syncthreads();
+    // a wait that ran out is agreed on here, between this barrier and the next,
+    // where no thread sets the flag (a reducing barrier costs 250 clocks more)
+    if (*fail) { abort = true; break; }
     consumed = sl + 1;
     // convert the FP64 tile: warp w owns columns 4w..4w+3
     const uint2* X = reinterpret_cast<const uint2*>(xd + stage * (C::XD_BYTES / 8));
     unsigned char* xb = xt + buf * C::PARTS * C::XT_BYTES;
     if constexpr (PREC == P_FP32) {
-      const uint32_t sm = sgnmask[buf][lane];
+      const uint32_t sm = sgnmask[sgrp * T + lane];
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc) {
         const int col = warp * 4 + cc;
         const uint2 w = X[col * T + lane];
-        const uint32_t hi = sm == 0xFFFFFFFFu ? 0u : (w.y ^ sm), lo = sm == 0xFFFFFFFFu ? 0u : w.x;
-        uint32_t amax = __reduce_max_sync(0xffffffffu, hi & 0x7FFFFFFFu);
-        int e;
-        if ((amax >> 20) != 0u) e = scale_exponent_bits(amax, 1u);
-        else e = scale_exponent(warp_max(fabs(__hiloint2double((int)hi, (int)lo))));
-        if (lane == 0) colscale[buf][col] = ldexpf(1.0f, -e);
-        uint32_t h = hi, l = lo;
-        scale_bits(h, l, e);
-        const float f = __uint_as_float(f64bits_to_f32(h, l));   // fl_32
+        const uint32_t hi = w.y ^ sm, lo = w.x, ha = hi & 0x7FFFFFFFu;
+        const uint32_t amax = __reduce_max_sync(0xffffffffu, ha), emax = amax >> 20;
+        uint32_t fb;   // fl_32
+        if (col_fast(emax)) {
+          const ColScale c(emax);
+          if (lane == 0) colscale[buf][col] = col_unscale(emax);
+          fb = f32_col(hi, lo, c, 1036 - (int)emax);
+        } else if (amax == 0u && !__any_sync(0xffffffffu, lo != 0u)) {   // a zero column, or one beyond n
+          if (lane == 0) colscale[buf][col] = 1.f;
+          fb = hi;
+        } else {
+          int e;
+          if (emax != 0u) e = scale_exponent_bits(amax, 1u);
+          else e = scale_exponent(warp_max(fabs(__hiloint2double((int)hi, (int)lo))));
+          if (lane == 0) colscale[buf][col] = ldexpf(1.0f, -e);
+          uint32_t h = hi, l = lo;
+          scale_bits(h, l, e);
+          fb = f64bits_to_f32(h, l);
+        }
+        const float f = __uint_as_float(fb);
         const uint32_t b = tc::to_tf32(f);
         *reinterpret_cast<uint32_t*>(xb + tc::sw128_offset(col, lane, 4)) = b;
         *reinterpret_cast<uint32_t*>(xb + C::XT_BYTES + tc::sw128_offset(col, lane, 4)) =
             tc::to_tf32(f - __uint_as_float(b));
       }
     } else {
-      const uint32_t sm0 = sgnmask[buf][2 * lane], sm1 = sgnmask[buf][2 * lane + 1];
+      const uint32_t sm0 = sgnmask[sgrp * T + 2 * lane], sm1 = sgnmask[sgrp * T + 2 * lane + 1];
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc) {
         const int col = warp * 4 + cc;
         const uint4 w = reinterpret_cast<const uint4*>(X)[(col * T) / 2 + lane];   // rows 2 lane, 2 lane + 1
-        const uint32_t h0 = sm0 == 0xFFFFFFFFu ? 0u : (w.y ^ sm0), l0 = sm0 == 0xFFFFFFFFu ? 0u : w.x;
-        const uint32_t h1 = sm1 == 0xFFFFFFFFu ? 0u : (w.w ^ sm1), l1 = sm1 == 0xFFFFFFFFu ? 0u : w.z;
-        uint32_t amax = __reduce_max_sync(0xffffffffu, max(h0 & 0x7FFFFFFFu, h1 & 0x7FFFFFFFu));
-        int e;
-        if ((amax >> 20) != 0u) e = scale_exponent_bits(amax, 1u);
-        else e = scale_exponent(warp_max(fmax(fabs(__hiloint2double((int)h0, (int)l0)),
-                                              fabs(__hiloint2double((int)h1, (int)l1)))));
-        if (lane == 0) colscale[buf][col] = ldexpf(1.0f, -e);
-        *reinterpret_cast<uint32_t*>(xb + tc::sw128_offset(col, 2 * lane, 2)) = pack2<C::FMT>(h0, l0, h1, l1, e);
+        const uint32_t h0 = w.y ^ sm0, h1 = w.w ^ sm1;
+        const uint32_t amax = __reduce_max_sync(0xffffffffu, max(h0 & 0x7FFFFFFFu, h1 & 0x7FFFFFFFu));
+        const uint32_t emax = amax >> 20;
+        uint32_t pk;
+        if (col_fast(emax)) {
+          if (lane == 0) colscale[buf][col] = col_unscale(emax);
+          pk = pack2_col<C::FMT>(h0, w.x, h1, w.z, ColScale(emax), 1036 - (int)emax);
+        } else if (amax == 0u && !__any_sync(0xffffffffu, (w.x | w.z) != 0u)) {
+          // a zero column, or one beyond n (the exact maximum below, in FP64
+          // instructions, doubled the kernel's time at n = 100)
+          if (lane == 0) colscale[buf][col] = 1.f;
+          pk = (h0 >> 16) | (h1 & 0x80000000u);
+        } else {
+          int e;
+          if (emax != 0u) e = scale_exponent_bits(amax, 1u);
+          else e = scale_exponent(warp_max(fmax(fabs(__hiloint2double((int)h0, (int)w.x)),
+                                                fabs(__hiloint2double((int)h1, (int)w.z)))));
+          if (lane == 0) colscale[buf][col] = ldexpf(1.0f, -e);
+          pk = pack2<C::FMT>(h0, w.x, h1, w.z, e);
+        }
+        *reinterpret_cast<uint32_t*>(xb + tc::sw128_offset(col, 2 * lane, 2)) = pk;
       }
     }
     tc::fence_proxy_async();
@@ -377,18 +412,23 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
     }
     // the previous slab's products are read while this slab's MMAs run
     if (sl > 0) {
-      const bool ok_mma = tc::mbar_wait(&mma_bar[buf ^ 1], ((u - 1) >> 1) & 1u);
-      if (__syncthreads_or(!ok_mma)) { abort = true; break; }
-      mma_done = sl;
-      tc::fence_after();
-      epilogue((int)(u - 1));
+      // no barrier: the next slab's first one separates these reads from the
+      // next writes to this accumulator, operand and scale buffer
+      if (tc::mbar_wait(&mma_bar[buf ^ 1], ((u - 1) >> 1) & 1u)) {
+        mma_done = sl;
+        tc::fence_after();
+        epilogue((int)(u - 1));
+      } else {
+        *fail = 1;
+      }
     }
   }
   if (!abort && nslabs > 0) {
     const uint32_t u = S.seq + (uint32_t)(nslabs - 1);
-    const bool ok_mma = tc::mbar_wait(&mma_bar[u & 1u], (u >> 1) & 1u);
-    if (__syncthreads_or(!ok_mma)) abort = true;
-    else {
+    if (!tc::mbar_wait(&mma_bar[u & 1u], (u >> 1) & 1u)) *fail = 1;
+    __syncthreads();
+    abort = *fail != 0;
+    if (!abort) {
       mma_done = nslabs;
       tc::fence_after();
       epilogue((int)u);
@@ -411,11 +451,7 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
   }
   S.seq += (uint32_t)nslabs;
   if (tmap) S.tseq += (uint32_t)nslabs;
-#pragma unroll
-  for (int c = 0; c < C::ACC; ++c) {
-    const int col = n0 + c_lo + c;
-    if (row_ok && col < n) out[(size_t)col * s + s0 + erow] = (double)acc[c];
-  }
+  while (chunk < nchunks) flush();   // a short last chunk; chunks beyond the rows are zero
   return true;
 }
 
@@ -430,9 +466,11 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
   __shared__ __align__(8) uint64_t mma_bar_s[2];                                                      \
   __shared__ uint32_t tmem_base;                                                                      \
   __shared__ float colscale_s[2][kN];                                                                 \
-  __shared__ uint32_t sgnmask_s[2][C::T];                                                             \
+  __shared__ uint32_t sgnmask_s[kThreads];                                                            \
+  __shared__ int fail_s;                                                                              \
   if ((threadIdx.x >> 5) == 0) tc::tmem_alloc(&tmem_base, C::TMEM_COLS);                              \
   if (threadIdx.x == 0) {                                                                             \
+    fail_s = 0;                                                                                       \
     for (int st = 0; st < C::STAGES; ++st) tc::mbar_init(&tma_bar_s[st], 1);                          \
     tc::mbar_init(&mma_bar_s[0], 1);                                                                  \
     tc::mbar_init(&mma_bar_s[1], 1);                                                                  \
@@ -442,7 +480,7 @@ __device__ __forceinline__ bool sketch_tc_item(const CUtensorMap* tmap, const do
   __syncthreads();                                                                                    \
   tc::fence_after();                                                                                  \
   TcCta<PREC, MT> S{smem + C::TAB_OFF, smem + C::XT_OFF, reinterpret_cast<double*>(smem + C::XD_OFF), \
-                    tma_bar_s,          mma_bar_s,         tmem_base, colscale_s, sgnmask_s, 0u, 0u};
+                    tma_bar_s,          mma_bar_s,         tmem_base, colscale_s, sgnmask_s, &fail_s, 0u, 0u};
 
 template <int PREC, int MT>
 __device__ __forceinline__ void sketch_tc_cta_end(TcCta<PREC, MT>& S, bool abort, Ctl* ctl) {
@@ -457,14 +495,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     k_sketch_tc(const __grid_constant__ CUtensorMap tmapA, int use_map, const double* __restrict__ A, int64_t lda,
                 int64_t m, int n, int s, const uint32_t* __restrict__ idx,
                 const double* __restrict__ tab, uint2 key, int64_t rows_per_chunk,
-                double* __restrict__ Ypart, Ctl* ctl, int level, int tf) {
+                double* __restrict__ Ypart, Ctl* ctl, int level, int tf, int chunks, int per_cta) {
   if (level_inactive(ctl, level)) return;
   MRCQR_SKETCH_TC_CTA(S)
-  const int64_t j_begin = (int64_t)blockIdx.z * rows_per_chunk;
+  const int c0 = blockIdx.z * per_cta, nc = min(per_cta, chunks - c0);
+  const int64_t j_begin = (int64_t)c0 * rows_per_chunk;
   const bool ok = sketch_tc_item<PREC, MT>(use_map ? &tmapA : nullptr, A, lda, m, n, s, idx, tab, key, j_begin,
-                                           min(m, j_begin + rows_per_chunk),
+                                           min(m, j_begin + nc * rows_per_chunk), rows_per_chunk, nc,
                                            blockIdx.x * (kM * MT), blockIdx.y * kN,
-                                           Ypart + (size_t)blockIdx.z * (size_t)s * (size_t)n, tf, S);
+                                           Ypart + (size_t)c0 * (size_t)s * (size_t)n, tf, S);
   sketch_tc_cta_end(S, !ok, ctl);
 }
 
@@ -483,7 +522,7 @@ __global__ void __launch_bounds__(kThreads, 1) kg_sketch_tc(Group g, int level) 
     const CUtensorMap* map = reinterpret_cast<const CUtensorMap*>(PREC == P_FP32 ? P.tmap32 : P.tmap64);
     const int64_t j_begin = (int64_t)w.y * P.rows_per_chunk;
     if (!sketch_tc_item<PREC, MT>(map, P.A, P.lda, P.m, P.n, P.s, P.idx, P.tab, P.key, j_begin,
-                                  min(P.m, j_begin + P.rows_per_chunk),
+                                  min(P.m, j_begin + P.rows_per_chunk), P.rows_per_chunk, 1,
                                   w.z * (kM * MT), w.w * kN, P.ypart + (size_t)w.y * (size_t)P.s * (size_t)P.n, P.tf,
                                   S)) {
       abort = true;
@@ -524,9 +563,21 @@ bool launch_tc(const CUtensorMap& map, bool use_map, const double* A, int64_t ld
     return false;
   int64_t rpc = (m + chunks - 1) / chunks;
   rpc = (rpc + 63) / 64 * 64;
-  const dim3 grid((s + kM * MT - 1) / (kM * MT), (n + kN - 1) / kN, chunks);
-  { ::mrcqr::note_launch(); k_sketch_tc<PREC, MT><<<grid, kThreads, smem, st>>>(map, use_map ? 1 : 0, A, lda, m, n, s, idx, tab,
-                                                                               seed_key(seed), rpc, Ypart, ctl, level, tf); }
+  // Consecutive chunks per CTA: the transform tables, TMEM and the pipeline's
+  // start are worth about kSetupRows rows of a CTA's work, paid once per CTA;
+  // the count that makes the waves shortest.  Sums by chunk either way.
+  constexpr int kSetupRows = 512;
+  const int tiles = ((s + kM * MT - 1) / (kM * MT)) * ((n + kN - 1) / kN);
+  int per_cta = 1;
+  int64_t best = INT64_MAX;
+  for (int k = 1; k <= chunks && k <= 16; ++k) {
+    const int64_t ctas = (int64_t)tiles * ((chunks + k - 1) / k);
+    const int64_t cost = (ctas + 151) / 152 * (k * rpc + kSetupRows);
+    if (cost < best) { best = cost; per_cta = k; }
+  }
+  const dim3 grid((s + kM * MT - 1) / (kM * MT), (n + kN - 1) / kN, (chunks + per_cta - 1) / per_cta);
+  launch_dep(k_sketch_tc<PREC, MT>, grid, kThreads, smem, st, map, use_map ? 1 : 0, A, lda, m, n, s, idx, tab,
+                                                                               seed_key(seed), rpc, Ypart, ctl, level, tf, chunks, per_cta);
   return true;
 }
 
