@@ -35,8 +35,8 @@
 // copies in flight, frees its TMEM, raises TIMEOUT and returns.
 //
 // What bounds it: the integer instructions of step 2 and the two barriers per
-// slab (issue slots 48% busy, tensor pipe 5%, 1.7 TB/s at n = 64), not the
-// MMAs.  Measured at m = 2^20 (ms, before / now): FP16 n = 64 0.355 / 0.236,
+// slab (2.3 TB/s at n = 64; tensor pipe 5% busy before the last of the changes
+// below), not the MMAs.  Measured at m = 2^20 (ms, before / now): FP16 n = 64 0.355 / 0.236,
 // 100 1.05 / 0.57, 128 0.92 / 0.58; FP32 n = 100 2.30 / 1.51, 128 1.93 / 1.56.
 // Of the FP16 n = 64 gain, 17 us came from a flag in place of the reducing
 // barriers and from drawing signs for several slabs at once, 27 us from several
