@@ -166,16 +166,17 @@ __device__ __forceinline__ void rp_end(const RpArgs& a, RpCta& S) {
   __syncthreads();
 }
 
-// Solves the 32 x 32 diagonal block of a panel that keeps its substitution:
-// sb[c][row] holds B = A_t - W_{<t} R_{<t,t} and receives B R_tt^{-1}.
+// Solves the w x w diagonal block (w = 32, less in the last panel: R has n rows)
+// of a panel that keeps its substitution: sb[c][row] holds B = A_t - W_{<t} R_{<t,t}
+// and receives B R_tt^{-1} in its first w columns.
 __device__ __noinline__ void rp_substitute(const RpArgs& a, double* sb, int c0, int row) {
-  const int npad = (a.n + 31) / 32 * 32;
-  for (int c = 0; c < kRN; ++c) {
+  const int npad = (a.n + 31) / 32 * 32, w = min(kRN, a.n - c0);
+  for (int c = 0; c < w; ++c) {
     const double x = sb[c * kM + row] * a.rinv[c0 + c];
     sb[c * kM + row] = x;
     const double* r = a.RT + (int64_t)(c0 + c) * npad + c0;
 #pragma unroll 4
-    for (int c2 = c + 1; c2 < kRN; ++c2) sb[c2 * kM + row] = fma(-x, r[c2], sb[c2 * kM + row]);
+    for (int c2 = c + 1; c2 < w; ++c2) sb[c2 * kM + row] = fma(-x, r[c2], sb[c2 * kM + row]);
   }
 }
 

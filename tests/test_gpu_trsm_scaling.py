@@ -1,0 +1,44 @@
+"""W = A R^{-1} where its fast path needs care: panels that keep the substitution
+at a ragged edge.  References are correctly rounded products
+(``oracle.product_rounded``) and the solve in FP64 arithmetic."""
+import numpy as np
+import pytest
+
+from oracle import mrcqr_oracle as O
+
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2606_18411_gb300 import mrcqr as M
+    return torch, M
+
+
+def _triangle(n, rng):
+    return np.triu(rng.standard_normal((n, n)) * 0.3) + np.diag(1.0 + rng.random(n))
+
+
+def _column_residuals(A, W, R):
+    """||A_j - (W R)_j|| against ||(|W| |R|)_j|| per column."""
+    res = np.linalg.norm(A - O.product_rounded(W, R), axis=0)
+    return res, np.linalg.norm(np.abs(W) @ np.abs(R), axis=0)
+
+
+# A tiny diagonal entry just before the last column: the last panel, of 2, 8, 18 and 31 columns, would amplify and
+# keeps the substitution, whose triangle ends at column n.
+@pytest.mark.parametrize("n", [34, 40, 50, 63, 512 - 1])
+def test_ragged_last_panel_keeps_its_substitution(env, n):
+    torch, M = env
+    rng = np.random.default_rng(n)
+    R = _triangle(n, rng)
+    R[n - 2, n - 2] = 1e-9
+    A = rng.standard_normal((200, n))
+    W = M.trsm(M.to_colmajor(A), M.to_colmajor(R)).cpu().numpy()
+    assert np.isfinite(W).all()
+    res, scale = _column_residuals(A, W, R)
+    assert (res <= 4 * n * U * scale).all(), float((res / scale).max())
