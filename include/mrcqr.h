@@ -98,8 +98,11 @@ typedef struct mrcqr_opts {
                              rows -- else as 2; 3: FP64 only, the emulated sketch sliced per work
                              item; 5: FP64 only, from digit planes.  The digit planes and the
                              words of the four-step form take 16 bytes per entry of A: a
-                             factorization writes them into its Q buffer (Q is overwritten before
-                             stage 2 of the level), in row chunks of at most half of Q;
+                             factorization writes them into the m x n entries of its Q buffer (Q is
+                             overwritten before stage 2 of the level; the rows m .. ldq - 1 are not
+                             touched), in row chunks of at most half of Q; with ldq > m the planes,
+                             and the words if ldq is odd, go to its workspace instead (sliced per
+                             work item if there is no room, or in a retry after a lower precision);
                              mrcqr_sketch and mrcqr_sketch_ex hold them in their workspace. */
   double ortho_tol;   /* acceptance threshold on ||I - Q^T Q||_F (default 1e-13) */
   void* stats_device; /* optional DEVICE pointer to an mrcqr_stats_t written at the end */

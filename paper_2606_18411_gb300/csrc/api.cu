@@ -36,7 +36,8 @@ struct Plan {
 };
 
 // planes: reserve the digit planes of the FP64 sketch in the workspace (the step-level sketch call,
-// which has no Q buffer to lend them); a factorization lends them its Q buffer.
+// which has no Q buffer to lend them, and a factorization whose Q has ldq > m and no four-step form);
+// else a factorization lends them its Q buffer.
 Plan make_plan(int64_t m, int n, int s, int tf = T_DCT, bool planes = false) {
   Plan p;
   p.tf = tf;
@@ -257,7 +258,7 @@ int g_sketch_variant_last = 0;
 // FP64 sliced per item, 4 four-step, 5 emulated FP64 from digit planes, 6 four-step emulated FP64).
 int enqueue_sketch(const Plan& p, void* ws, int prec, int variant, int fp64_products, const double* A, int64_t lda,
                    uint64_t seed, double* Y, Ctl* ctl, int lvl, cudaStream_t st, void* scratch = nullptr,
-                   size_t scratch_bytes = 0) {
+                   size_t scratch_bytes = 0, size_t scratch_stride = 0) {
   const uint32_t* idx = at<uint32_t>(ws, p.off_idx);
   const double* tab = at<double>(ws, p.off_tab);
   int used = 0;
@@ -265,14 +266,14 @@ int enqueue_sketch(const Plan& p, void* ws, int prec, int variant, int fp64_prod
     uint32_t* colhi = at<uint32_t>(ws, p.off_colhi);
     long long* part = at<long long>(ws, p.off_ozpart);
     if ((variant == 0 || variant == 6) && scratch_bytes >= p.fd_scratch &&
-        sketch_fd_eligible(p.m, p.n, p.s, p.tf, scratch, p.fd_scratch)) {
+        sketch_fd_eligible(p.m, p.n, p.s, p.tf, scratch, p.fd_scratch, scratch_stride)) {
       launch(SG_SKETCH, lvl, st, [&] {
         launch_sketch_fd(p.m, p.n, p.s, A, lda, idx, at<uint4>(ws, p.off_tabd), seed, colhi, part, at<void>(ws, p.off_fd),
-                         Y, scratch, p.fd_scratch, ctl, lvl, st);
+                         Y, scratch, p.fd_scratch, scratch_stride, ctl, lvl, st);
       });
       return 6;
     }
-    const bool planes = variant != 3 && sketch_ozp_eligible(p.m, p.n, scratch, scratch_bytes) &&
+    const bool planes = variant != 3 && scratch_stride == 0 && sketch_ozp_eligible(p.m, p.n, scratch, scratch_bytes) &&
                         sketch_ozp_part_bytes(p.m, p.n, p.s, scratch_bytes) <= p.ozpart_bytes;
     used = 3;
     launch(SG_SKETCH, lvl, st, [&] {
@@ -392,17 +393,34 @@ int mrcqr_factor_ex(int64_t m, int64_t n, const double* A, int64_t lda, double* 
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int bins = s_factor * (int)n;                 // sampled rows (DCT) or bins (real FFT)
   const int s = (int)sketch_rows(m, bins, tf);        // rows of Y
-  const Plan p = make_plan(m, (int)n, s, tf);
   int lv[kMaxLevels] = {P_FP64, P_FP64, P_FP64, P_FP64};
   // AUTO: the ladder fp16 -> fp32 -> fp64 always; the selector picks where it starts
   const int nlevels = make_ladder(autosel ? (int)P_FP16 : sketch_prec, autosel || escalate, lv);
+  // Scratch of the FP64 sketch: the m x n entries of Q (stage 2 of the level writes W there later).  With ldq > m
+  // the words of the four-step form keep to the columns of Q; digit planes, whose copies want them packed, go to
+  // the workspace where FP64 may be the first level (a retry in FP64 slices per work item: reserving 16 bytes per
+  // entry on every low-precision call would cost more).
+  const size_t q_bytes = sizeof(double) * (size_t)m * (size_t)n;
+  const size_t q_stride = ldq == m || n == 1 ? 0 : sizeof(double) * (size_t)ldq;
+  bool own = q_stride != 0 && (lv[0] == P_FP64 || autosel) && variant != 1 && variant != 3 && fp64p == 0 &&
+             !((variant == 0 || variant == 6) && sketch_fd_eligible(m, (int)n, s, tf, Q, q_bytes, q_stride));
+  Plan p = make_plan(m, (int)n, s, tf, own);
   mrcqr_stats_t* slot = status_slot(st);
   if (!slot) return MRCQR_ERR_ALLOC;
   void* ws = nullptr;
-  if (cudaMallocAsync(&ws, p.total, st) != cudaSuccess) {
+  cudaError_t got = cudaMallocAsync(&ws, p.total, st);
+  if (got != cudaSuccess && own) {   // no room for planes of its own: the FP64 sketch slices per work item
+    cudaGetLastError();
+    own = false;
+    p = make_plan(m, (int)n, s, tf);
+    got = cudaMallocAsync(&ws, p.total, st);
+  }
+  if (got != cudaSuccess) {
     cudaGetLastError();
     return MRCQR_ERR_ALLOC;
   }
+  void* scratch = own ? at<void>(ws, p.off_planes) : static_cast<void*>(Q);
+  const size_t scratch_bytes = own ? p.planes_bytes : q_bytes, scratch_stride = own ? 0 : q_stride;
   Ctl* ctl = at<Ctl>(ws, p.off_ctl);
   uint32_t* idx = at<uint32_t>(ws, p.off_idx);
   double* tab = at<double>(ws, p.off_tab);
@@ -411,9 +429,8 @@ int mrcqr_factor_ex(int64_t m, int64_t n, const double* A, int64_t lda, double* 
   launch(SG_COSTAB, 0, st, [&] { launch_costab(m, tab, st); });
   for (int L = 0; L < nlevels; ++L) {
     double* y = at<double>(ws, p.off_y);
-    // the FP64 sketch borrows the Q buffer for its digit planes (stage 2 of the level writes W there later)
-    g_sketch_variant_last = enqueue_sketch(p, ws, lv[L], variant, fp64p, A, lda, seed, y, ctl, L, st, Q,
-                                           sizeof(double) * (size_t)((n - 1) * ldq + m));
+    g_sketch_variant_last = enqueue_sketch(p, ws, lv[L], variant, fp64p, A, lda, seed, y, ctl, L, st, scratch,
+                                           scratch_bytes, scratch_stride);
     launch(SG_SQR, L, st, [&] {
       launch_sketch_qr(lv[L], (int)n, s, y, at<void>(ws, p.off_sqr), at<double>(ws, p.off_rs),
                        at<double>(ws, p.off_rst), at<double>(ws, p.off_rinv), ctl, L, st);

@@ -216,13 +216,16 @@ void launch_sketch_oz_reduce(int n, int s, const uint32_t* colHi, const uint32_t
 // --- FP64 sketch as a four-step transform (sketch_fd.cu) --------------------------
 // From this many sampled rows on (with n, m and the alignment as sketch_fd_eligible says) it is the faster
 // form; the words of the first step go to `scratch`, ints holds sketch_fd_ints_bytes.
+// The scratch is scratch_bytes / n bytes of each of n columns that are scratch_stride bytes apart (0: packed), so
+// that a Q with ldq > m can be lent without the rows between its columns.
 constexpr int kFdMinRows = 160;
-bool sketch_fd_eligible(int64_t m, int n, int s, int tf, const void* scratch, size_t scratch_bytes);
+bool sketch_fd_eligible(int64_t m, int n, int s, int tf, const void* scratch, size_t scratch_bytes,
+                        size_t scratch_stride);
 size_t sketch_fd_part_bytes(int64_t m, int n, int s, size_t scratch_bytes);
 size_t sketch_fd_ints_bytes(int64_t m, int s);
 void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, const uint32_t* idx, uint4* tabd,
                       uint64_t seed, uint32_t* colHi, long long* part, void* ints, double* Y, void* scratch,
-                      size_t scratch_bytes, Ctl* ctl, int level, cudaStream_t st);
+                      size_t scratch_bytes, size_t scratch_stride, Ctl* ctl, int level, cudaStream_t st);
 
 // --- W = A R^{-1} and Q = W X in emulated FP64 (rowprod.cu) -----------------------
 // Workspace: digit panels of the multiplier (each product), the TRSM's integers (column exponents, row

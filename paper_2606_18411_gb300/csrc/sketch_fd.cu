@@ -20,7 +20,8 @@
 // and both cosine tables are evaluated to about 2^-61 by their Taylor series in
 // 64-bit integers (the dense form takes FP64 cosines), so the sketch is as
 // accurate as the dense form's.  The words take twice the space of A; a
-// factorization lends the Q buffer and works in two ranges of j1.
+// factorization lends the Q buffer, each column's words in that column, and
+// works in two ranges of j1.
 //
 // Measured (Y; dense form before): m = 2^20, n = 512, s = 1024 55.0 -> 12.7 ms; n = 128, s = 256 4.03 -> 2.63;
 // m = 2^18, n = 160, s = 320 2.35 -> 0.98. Pass 1 (0.85 of 2.63 ms at n = 128) is bound by the integer pipe
@@ -223,11 +224,11 @@ __device__ __forceinline__ void fd_end(FdCta& S, bool abort, Ctl* ctl) {
 // ---------------------------------------------------------------------------
 // Pass 1.  Item = (128 rows j1 from jb, column c): A operand = rows j1, K =
 // j2 (loads contiguous in j1); B operand = the 64 x 32 transform digits, kept
-// in shared memory by the CTA.  Output words U[(c 64 + row) Jc + j1 - j0].
+// in shared memory by the CTA.  Output words U[c cs + row Jc + j1 - j0].
 __global__ void __launch_bounds__(kRThreads, 2)
     k_fd_pass1(int64_t J, int64_t j0, int64_t Jc, int nblocks, int n, const double* __restrict__ A, int64_t lda,
                const uint32_t* __restrict__ colHi, const int* __restrict__ colU, const uint32_t* __restrict__ sgn,
-               uint64_t* __restrict__ U, Ctl* ctl, int level) {
+               uint64_t* __restrict__ U, int64_t cs, Ctl* ctl, int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
   MRCQR_FD_CTA(S)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(kRThreads, 2)
     tc::fence_proxy_async();
     tc::fence_before();
     __syncthreads();
-    uint64_t* out = U + (int64_t)(c * kRows + g * 16) * Jc + kM * (item - c * nblocks) + q * 32 + lane;
+    uint64_t* out = U + c * cs + g * 16 * Jc + kM * (item - c * nblocks) + q * 32 + lane;
 #pragma unroll 1
     for (int t = 0; t < 2; ++t) {
       if (tid == 0) {
@@ -335,6 +336,7 @@ struct Fd2Args {
   int64_t m, J, j0, Jc, rows;   // rows: j1 per slab (multiple of 32)
   int n, cblocks, slabs;
   const uint64_t* U;
+  int64_t cs;                   // words between columns
   const uint32_t* idx;
   const uint4* tabd;
   const int* ntiles;
@@ -388,7 +390,7 @@ __global__ void __launch_bounds__(kRThreads, 2) k_fd_pass2(Fd2Args a, Ctl* ctl, 
     };
     int64_t coff[4];   // the four columns' words (column 0 beyond n: its digits are dropped)
 #pragma unroll
-    for (int it = 0; it < 4; ++it) coff[it] = (int64_t)(cbase + 4 * it < a.n ? cbase + 4 * it : 0) * kRows * a.Jc;
+    for (int it = 0; it < 4; ++it) coff[it] = (cbase + 4 * it < a.n ? cbase + 4 * it : 0) * a.cs;
     auto gather = [&] {
       uint64_t r = ph;
 #pragma unroll
@@ -562,9 +564,10 @@ constexpr size_t kFdSmem = (size_t)kRABytes + 2 * (size_t)kRBBytes + 1024;
 }  // namespace
 
 // m a multiple of 32 (the radix) and at least 2^15, DCT, s >= kFdMinRows.
-bool sketch_fd_eligible(int64_t m, int n, int s, int tf, const void* scratch, size_t scratch_bytes) {
+bool sketch_fd_eligible(int64_t m, int n, int s, int tf, const void* scratch, size_t scratch_bytes,
+                        size_t scratch_stride) {
   if (tf != T_DCT || m % kR != 0 || m < (1 << 15) || s < kFdMinRows) return false;
-  if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 15) != 0) return false;
+  if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 15) != 0 || scratch_stride % 16 != 0) return false;
   const FdPlan p = fd_plan(m, n, s, scratch_bytes);
   return p.Jc > 0 && p.chunks <= 4;
 }
@@ -584,7 +587,7 @@ size_t sketch_fd_ints_bytes(int64_t m, int s) {
 
 void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, const uint32_t* idx, uint4* tabd,
                       uint64_t seed, uint32_t* colHi, long long* part, void* ints, double* Y, void* scratch,
-                      size_t scratch_bytes, Ctl* ctl, int level, cudaStream_t st) {
+                      size_t scratch_bytes, size_t scratch_stride, Ctl* ctl, int level, cudaStream_t st) {
   const FdPlan p = fd_plan(m, n, s, scratch_bytes);
   int* ntiles = static_cast<int*>(ints);
   int* colU = ntiles + 64;
@@ -600,12 +603,13 @@ void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, con
   cudaFuncSetAttribute(k_fd_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFdSmem);
   cudaFuncSetAttribute(k_fd_pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFdSmem);
   uint64_t* U = static_cast<uint64_t*>(scratch);
+  const int64_t cs = scratch_stride ? (int64_t)(scratch_stride / 8) : kRows * p.Jc;
   for (int k = 0; k < p.chunks; ++k) {
     const int64_t j0 = (int64_t)k * p.Jc;
     const int nblocks = (int)(p.Jc / kM);   // rows j1 >= J give zero words
     const int64_t items = (int64_t)nblocks * n;
-    launch_dep(k_fd_pass1, (unsigned)std::min<int64_t>(items, 2 * fd_sms()), kRThreads, kFdSmem, st, p.J, j0, p.Jc, nblocks, n, A, lda, colHi, colU, sgn, U, ctl, level);
-    const Fd2Args a{m, p.J, j0, p.Jc, p.rows, n, p.cblocks, p.slabs, U, idx, tabd, ntiles, cls, slots, part,
+    launch_dep(k_fd_pass1, (unsigned)std::min<int64_t>(items, 2 * fd_sms()), kRThreads, kFdSmem, st, p.J, j0, p.Jc, nblocks, n, A, lda, colHi, colU, sgn, U, cs, ctl, level);
+    const Fd2Args a{m, p.J, j0, p.Jc, p.rows, n, p.cblocks, p.slabs, U, cs, idx, tabd, ntiles, cls, slots, part,
                     k * p.slabs, p.slabs * p.chunks};
     const int64_t most = (int64_t)p.max_tiles * p.cblocks * p.slabs;
     launch_dep(k_fd_pass2, (unsigned)std::min<int64_t>(most, 2 * fd_sms()), kRThreads, kFdSmem, st, a, ctl, level);

@@ -80,6 +80,27 @@ def test_factorization_takes_it_with_q_as_scratch(env, ldq):
     assert O.residual_error(A, Q[:m].cpu().numpy(), R.cpu().numpy())[0] <= 1e-13
 
 
+# Q as the leading rows of a taller array: the FP64 sketch's scratch leaves the rows between its columns alone, in
+# the columns of Q (the four-step form, 6, even ldq) or in the workspace (odd ldq; digit planes, 5).  Q and R are
+# those of a packed Q bit for bit.
+@pytest.mark.parametrize("m,n,pad,variant", [(1 << 15, 96, 2, 6), (1 << 15, 80, 1, 6), (9000, 100, 64, 5),
+                                             (4099, 30, 1, 5), (1 << 15, 1, 6, 5), (32 * 2048, 128, 128, 6)])
+def test_rows_between_the_columns_of_q_are_kept(env, m, n, pad, variant):
+    torch, M = env
+    from paper_2606_18411_gb300 import inputs
+    A = M.to_colmajor(inputs.make_matrix(m, n, 1e10 if n > 1 else 1.0, seed=m + n))
+    outs = []
+    for ld in (m, m + pad):
+        full = torch.full((n, ld), 7.25, dtype=torch.float64, device="cuda")
+        Q, R = full.t()[:m], M.empty_colmajor(n, n)
+        M.factor_ex(A, Q, R, prec="fp64", seed=4, escalate=False)
+        assert M.last_status()["status"] == "OK" and M.last_sketch_variant() == variant
+        assert bool((full[:, m:] == 7.25).all())
+        outs.append((Q.cpu().numpy(), R.cpu().numpy()))
+    np.testing.assert_array_equal(outs[0][0], outs[1][0])
+    np.testing.assert_array_equal(outs[0][1], outs[1][1])
+
+
 def test_sizes_the_four_step_form_does_not_take(env):
     torch, M = env
     A = np.random.default_rng(1).standard_normal((1 << 15, 4))
