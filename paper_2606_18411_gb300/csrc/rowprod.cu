@@ -369,13 +369,13 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
           if (h > cm[c]) atomicMax(cm + c, h);
           if (kTrsm) {
             mxh = max(mxh, h);
-            mxE = max(mxE, (int)h + er[c] * (1 << 20));
+            if (h != 0u) mxE = max(mxE, (int)(h >> 2) + er[c] * (1 << 18));   // >> 2: room for both exponents
           }
         }
         wp += a.ldw;
       }
-      // a zero counts as exponent 0 + e_k: below every normal entry's unless the whole row is zero
-      if (kTrsm && mxh != 0u) atomicMax(&S.rowX[rr], mxh >= 0x7FF00000u ? kNonfinite : mxE >> 20);
+      // zeros do not count: with e_k over more than 2^1000 a zero's 0 + e_k could pass every entry's exponent
+      if (kTrsm && mxh != 0u) atomicMax(&S.rowX[rr], mxh >= 0x7FF00000u ? kNonfinite : mxE >> 18);
     }
     if (__syncthreads_or(*(volatile int*)S.dead)) return false;   // the tile's W is visible to the next tile's loads
   }

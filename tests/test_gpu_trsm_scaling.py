@@ -42,3 +42,21 @@ def test_ragged_last_panel_keeps_its_substitution(env, n):
     assert np.isfinite(W).all()
     res, scale = _column_residuals(A, W, R)
     assert (res <= 4 * n * U * scale).all(), float((res / scale).max())
+
+
+# R's first 32 rows 2^1200 above the others: zeros of W in those columns say nothing about the rows' size.
+@pytest.mark.parametrize("n", [33, 64, 130])
+def test_zeros_do_not_raise_a_row_reference(env, n):
+    torch, M = env
+    rng = np.random.default_rng(n)
+    R = _triangle(n, rng)
+    R[:32, :32] *= 2.0 ** 600
+    R[:, 32:] *= 2.0 ** -600
+    A = rng.standard_normal((150, n))
+    A[:, :32] *= 2.0 ** 600
+    A[:, 32:] *= 2.0 ** -600
+    A[::2, :32] = 0.0
+    W = M.trsm(M.to_colmajor(A), M.to_colmajor(R)).cpu().numpy()
+    assert (W[::2, :32] == 0.0).all()
+    res, scale = _column_residuals(A[::2, 32:] * 2.0 ** 600, W[::2, 32:], R[32:, 32:] * 2.0 ** 600)
+    assert (res <= 4 * n * U * scale).all(), float((res / scale).max())
