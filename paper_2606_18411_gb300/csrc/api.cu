@@ -86,7 +86,7 @@ Plan make_plan(int64_t m, int n, int s, int tf = T_DCT, bool planes = false) {
   }
   p.off_ozpart = take(p.ozpart_bytes);   // the Gram, the check and the FP64 sketch use it one after the other
   p.off_tcole = take(rp_trsm_ints_bytes(n));
-  p.off_trd = take(rp_digit_bytes(n));
+  p.off_trd = take(rp_trsm_digit_bytes(n));
   p.off_tabd = take(16ull * (size_t)(m + 1));   // FP16 digits of the quarter-wave table
   if (planes) p.off_planes = take(p.planes_bytes);
   p.total = o;

@@ -47,7 +47,7 @@ enum Kind {
   // emulated-FP64 phases of one problem (param = problem) between a fork and a join of the side streams
   K_FORK, K_JOIN, K_OZ_SKETCH, K_OZ_STAGE2A, K_OZ_STAGE2B,
   // grouped emulated-FP64 kernels (param = 1: the check's Gram)
-  KG_OZ_COLHI, KG_OZ_SKETCH, KG_OZ_SKREDUCE, KG_OZ_ROWSCALE, KG_OZ_PREPR, KG_OZ_TRSM, KG_OZ_SYRK, KG_OZ_SYREDUCE,
+  KG_OZ_COLHI, KG_OZ_SKETCH, KG_OZ_SKREDUCE, KG_OZ_COLSCALE, KG_OZ_ROWSCALE, KG_OZ_PREPR, KG_OZ_TRSM, KG_OZ_SYRK, KG_OZ_SYREDUCE,
   KG_OZ_PREPX, KG_OZ_FINALIZE,
   // grouped tensor-core sketch, param = 2 precision + (MT - 1)
   KG_TC_SKETCH
@@ -227,7 +227,7 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
     g[0] = take(syrk_oz_colhi_bytes(P.n));
     g[1] = take(std::max(syrk_oz_part_bytes(z.sp), sketch_oz_part_bytes(z.kp)));
     g[2] = take(rp_trsm_ints_bytes(P.n));
-    g[3] = take(rp_digit_bytes(P.n));
+    g[3] = take(rp_trsm_digit_bytes(P.n));
     g[4] = take(rp_fin_ints_bytes(P.n));
     g[5] = take(rp_digit_bytes(P.n));
   }
@@ -329,11 +329,13 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
     add(K_SQR, L, 0, q32);
     add(K_SQR, L, 1, q64);
     // emulated-FP64 stage 2 work lists (grouped form)
-    std::vector<int4> z_rs, z_pr, z_tr, z_sy, z_gr, z_px, z_fi;
+    std::vector<int4> z_cs, z_rs, z_pr, z_tr, z_sy, z_gr, z_px, z_fi;
     if (pl.emu && pl.oz_grouped)
       for (int i : live) {
         const Prob& P = pl.probs[i];
         const OzWs& z = pl.oz[i];
+        if (P.n > kRpOwnScale)
+          for (int b = 0; b < rp_panels(P.n); ++b) z_cs.push_back(make_int4(i, b, 0, 0));
         if (P.n > kRpOwnScale)
           for (int b = 0; b < blocks(P.n, 8); ++b) z_rs.push_back(make_int4(i, b, 0, 0));
         for (int c = 0; c < rp_panels(P.n); ++c) z_pr.push_back(make_int4(i, c, 0, 0));
@@ -344,6 +346,7 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
         for (int b = 0; b < blocks(P.m, 128); ++b) z_fi.push_back(make_int4(i, b, 0, 0));
       }
     if (pl.emu && pl.oz_grouped) {   // W = A R_s^{-1} (folding W's column maxima), G = W^T W
+      add(KG_OZ_COLSCALE, L, 0, z_cs);
       add(KG_OZ_ROWSCALE, L, 0, z_rs);
       add(KG_OZ_PREPR, L, 0, z_pr);
       add(KG_OZ_TRSM, L, 0, z_tr);
@@ -513,6 +516,7 @@ void enqueue(mrcqr_batched_plan_s& pl, cudaStream_t st) {
       case KG_OZ_COLHI: launch_g_oz_colhi(g, L.level, st); break;
       case KG_OZ_SKETCH: launch_g_oz_sketch(g, L.level, st); break;
       case KG_OZ_SKREDUCE: launch_g_oz_sketch_reduce(g, L.level, st); break;
+      case KG_OZ_COLSCALE: launch_g_oz_col_scale(g, L.level, st); break;
       case KG_OZ_ROWSCALE: launch_g_oz_row_scale(g, L.level, st); break;
       case KG_OZ_PREPR: launch_g_oz_prep_r(g, L.level, st); break;
       case KG_OZ_TRSM: launch_g_oz_trsm(g, L.level, st); break;
@@ -527,14 +531,14 @@ void enqueue(mrcqr_batched_plan_s& pl, cudaStream_t st) {
 }
 
 // Kernels one execute launches (each emulated heavy phase of a problem is
-// several kernels: sketch 3; TRSM 2 or 3 + Gram 3; finalize 2 + check 3).
+// several kernels: sketch 3; TRSM 2 or 4 + Gram 3; finalize 2 + check 3).
 int count_kernels(const mrcqr_batched_plan_s& pl) {
   int k = 0;
   for (const Launch& L : pl.launches) {
     switch (L.kind) {
       case K_FORK: case K_JOIN: break;
       case K_OZ_SKETCH: k += 3; break;
-      case K_OZ_STAGE2A: k += pl.probs[L.param].n > kRpOwnScale ? 6 : 5; break;
+      case K_OZ_STAGE2A: k += pl.probs[L.param].n > kRpOwnScale ? 7 : 5; break;
       case K_OZ_STAGE2B: k += pl.probs[L.param].check ? 5 : 2; break;
       default: k += 1;
     }

@@ -74,8 +74,8 @@ struct Prob {
   SketchOzPlan oz_kp;
   uint32_t* oz_colhi;     // column maxima of A, W or Q (high words)
   long long* oz_part;     // Gram / check / FP64-sketch partials
-  int* oz_cole;           // TRSM: multiplier column exponents, e_k (n32 ints each), panel flags
-  unsigned char* oz_rd;   // TRSM: digit panels of the multiplier
+  int* oz_cole;           // TRSM: its integers (RpInts in rowprod.cu)
+  unsigned char* oz_rd;   // TRSM: digit panels of the two multipliers
   int* oz_xe;             // finalize: column exponents of R_c^-1
   unsigned char* oz_xs;   // finalize: digit panels of R_c^-1
   // tensor-core sketch (grouped): TMA maps of A with slabs of 64 rows (FP16/BF16) and 32 rows (FP32);
@@ -112,7 +112,8 @@ void launch_g_publish(const Group& g, cudaStream_t st);
 // grouped emulated-FP64 heavy phases (ozaki.cu, rowprod.cu): one persistent launch per kernel over the work list
 //   colhi        items {i, column}: column maxima of A (FP64 sketch)
 //   sketch_oz    items {i, item of the problem's SketchOzPlan}   sketch_oz_reduce {i, 256-entry block}
-//   row_scale    items {i, 8-row block of R_s}                   prep_r {i, 32-column panel}
+//   col_scale    items {i, 32-column panel of R_s}               row_scale {i, 8-row block of R_s}
+//   prep_r       items {i, 32-column panel}
 //   trsm_oz      items {i, 128-row block}
 //   syrk_oz      items {i, item of the problem's SyrkOzPlan}     syrk_oz_reduce {i, 256-entry block}
 //   prep_x       items {i, column < n32}                         finalize_oz {i, 128-row block}
@@ -121,6 +122,7 @@ void prepare_g_oz_kernels();   // kernel attributes; call outside stream capture
 void launch_g_oz_colhi(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_sketch(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_sketch_reduce(const Group& g, int level, cudaStream_t st);
+void launch_g_oz_col_scale(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_row_scale(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_prep_r(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_trsm(const Group& g, int level, cudaStream_t st);
@@ -228,10 +230,11 @@ void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, con
                       size_t scratch_bytes, size_t scratch_stride, Ctl* ctl, int level, cudaStream_t st);
 
 // --- W = A R^{-1} and Q = W X in emulated FP64 (rowprod.cu) -----------------------
-// Workspace: digit panels of the multiplier (each product), the TRSM's integers (column exponents, row
-// scalings, panel flags), the finalize's column exponents; columns and 32-column panels of n.
-constexpr int kRpOwnScale = 128;   // up to this n the TRSM's preparation finds the row scalings itself (no launch)
+// Workspace: digit panels of the multiplier (two sets for the TRSM), the TRSM's integers (column exponents,
+// row and column scalings, panel flags), the finalize's column exponents; columns and 32-column panels of n.
+constexpr int kRpOwnScale = 128;   // up to this n the TRSM's preparation finds the scalings itself (no launches)
 size_t rp_digit_bytes(int n);
+size_t rp_trsm_digit_bytes(int n);
 size_t rp_trsm_ints_bytes(int n);
 size_t rp_fin_ints_bytes(int n);
 int rp_cols(int n);

@@ -13,22 +13,28 @@
 //    No FP64 arithmetic is left: this GPU issues FP64 at 1/64 rate, and the
 //    16 x 16 substitutions that were here before kept its pipe busy for 55% of
 //    the kernel at n = 64, while W was sliced again for every 16 columns.
-//    X_t and Z_t are formed by k_rp_prep_r to 2^-61 of their column maxima
-//    (an FP64 substitution corrected once with the residual I - R_tt X_t in
-//    128-bit integers), so the product's error is that of the digits, about
-//    2^-60 max|row| max|column| per entry.  Seen as a backward error of A it is
-//    amplified by at most
-//      amp = max_j sum_c max|column c of (Z_t; X_t)| |R_tt[c][j]|,
+//    Columns enter equilibrated: with F = diag(2^f_c), f_c the exponent of the
+//    largest entry of column c of R, the kernel solves W (R F^{-1}) = A F^{-1},
+//    the same W (powers of two are exact), so the digits of a row of A cover every
+//    column whatever the columns' sizes.  The rows k of W enter scaled by 2^e_k, the
+//    binade of the largest entry of row k of R F^{-1}, and Z_t by 2^-e_k, so a
+//    graded R pairs balanced operands.
+//    X_t = (R F^{-1})_tt^{-1} and Z_t are formed by k_rp_prep_r to 2^-61 of their
+//    column maxima (an FP64 substitution corrected once with the residual
+//    I - R_tt X_t in 128-bit integers), so the product's error is that of the
+//    digits, about 2^-60 max|row| max|column| per entry.  Seen as a backward error
+//    of A F^{-1} it is amplified by at most
+//      amp = max_j sum_c max|column c of (Z_t; X_t)| |(R F^{-1})_tt[c][j]|,
 //    and a panel whose amp exceeds 512 (measured: below 400 for the R of sketched
 //    matrices with kappa up to 1e16, four spectra, n = 32 .. 512) keeps the
-//    substitution: its multiplier is (-R_{<t,t}; I), and the kernel solves
-//    with R_tt in FP64 afterwards.
-// The rows k of W enter scaled by 2^e_k, the binade of the largest entry of
-// row k of R, and Z_t by 2^-e_k, so a graded R pairs balanced operands.
+//    substitution: the product is W_{<t} (-R_{<t,t}) alone (A's digits are
+//    zeros in it), A_t is added and R_tt solved with in FP64.
 //
 // Measured at m = 2^20 (before: substitution blocks of 16 columns; Q = W X in
 // 128 x 64 tiles by one CTA per SM): W = A R^{-1} 1.78 -> 0.75 ms at n = 64,
-// 4.53 -> 1.80 at 128, 12.7 -> 5.9 at 256, 41.3 -> 20.5 at 512; Q = W X
+// 4.53 -> 1.80 at 128, 12.7 -> 5.9 at 256, 41.3 -> 20.5 at 512 (the column scales cost
+// nothing there: m = 300001, n = 320 2.94 ms without and 2.93 with them; 3 us of the 280 at
+// m = 4096, n = 32); Q = W X
 // 0.99 -> 0.63, 2.19 -> 1.61, 5.67 -> 5.39, 17.3 -> 18.6.  What bounds them is
 // integer-pipe work around the products (slicing about 1100 cycles per SM and
 // chunk, conversion of the results about 2400 per tile, against 1340 of MMAs
@@ -58,6 +64,16 @@ __host__ __device__ __forceinline__ size_t rp_block_offset(int t, int kc) {
   return ((size_t)t * (t + 1) / 2 + kc) * kRBBytes;
 }
 
+__host__ __device__ __forceinline__ int rp_n32(int n) { return (n + kRN - 1) / kRN * kRN; }
+__host__ __device__ __forceinline__ size_t rp_digit_size(int n) { return rp_block_offset(rp_n32(n) / kRN, 0); }
+
+// The TRSM's integers: column exponents of the two multipliers, e_k, -f_c (n32 each) and the panel flags (16).
+struct RpInts {
+  int *colE, *colE2, *eR, *fN, *flags;
+  __host__ __device__ __forceinline__ RpInts(int* p, int n)
+      : colE(p), colE2(p + rp_n32(n)), eR(p + 2 * rp_n32(n)), fN(p + 3 * rp_n32(n)), flags(p + 4 * rp_n32(n)) {}
+};
+
 struct RpArgs {
   int64_t m;
   int n;
@@ -67,7 +83,10 @@ struct RpArgs {
   int64_t ldw;
   const int* colE;              // reference exponent of each multiplier column
   const unsigned char* Md;      // digit panels of the multiplier blocks
+  const int* colE2;             // TRSM: the same for the panels that keep their substitution
+  const unsigned char* Md2;
   const int* eR;                // TRSM: row scaling e_k
+  const int* fN;                // TRSM: column scaling -f_c
   const int* flags;             // TRSM: 1 = the panel keeps its substitution
   const double* RT;             // TRSM: R transposed, row stride npad
   const double* rinv;
@@ -84,11 +103,13 @@ struct RpCta {
   int* dead;                    // a bounded wait gave up
   int* rowX;                    // TRSM: running maximum exponent of W D per row
   int* rowRef;                  // reference exponent of each row for the current tile
-  uint32_t (*red)[kM];          // [2][128]
+  int (*red)[kM];               // [2][128]
   int* eRs;                     // e_k, padded to 512
+  int* fNs;                     // -f_c, padded to 512
   uint32_t* cmax;               // column maxima of the result over this CTA's rows
   int* colE;                    // reference exponents of the multiplier columns
-  int* emax;                    // largest e_k (at least 0)
+  int* emax;                    // largest of the scalings e_k, -f_c and 0
+  uint32_t* keep;               // bit t: panel t keeps its substitution
 };
 
 __device__ __forceinline__ void rp_wait(RpCta& S, uint64_t* bar, uint32_t parity) {
@@ -96,11 +117,11 @@ __device__ __forceinline__ void rp_wait(RpCta& S, uint64_t* bar, uint32_t parity
   if (!tc::mbar_wait(bar, parity, 1u << 20)) *(volatile int*)S.dead = 1;
 }
 
-// Starts the copy of multiplier block (t, kc) into stage seq & 1.
-__device__ __forceinline__ void rp_fetch_b(const RpArgs& a, RpCta& S, uint32_t seq, int t, int kc) {
+// Starts the copy of multiplier block (t, kc) from Md into stage seq & 1.
+__device__ __forceinline__ void rp_fetch_b(const unsigned char* Md, RpCta& S, uint32_t seq, int t, int kc) {
   uint64_t* bar = &S.bar[1 + (seq & 1u)];
   tc::mbar_expect_tx(bar, kRBBytes);
-  tc::bulk_load(S.bs + (seq & 1u) * kRBBytes, a.Md + rp_block_offset(t, kc), kRBBytes, bar);
+  tc::bulk_load(S.bs + (seq & 1u) * kRBBytes, Md + rp_block_offset(t, kc), kRBBytes, bar);
 }
 
 // Slicing of sixteen values of one row into digits: four groups of four
@@ -142,18 +163,27 @@ __device__ __forceinline__ void rp_slice(const double (&v)[4][4], const int* es,
   }
 }
 
-// Per-problem state of a CTA: e_k, the column maxima.
+// Per-problem state of a CTA: the scalings, the kept panels, the column maxima.
 template <bool kTrsm>
 __device__ __forceinline__ void rp_begin(const RpArgs& a, RpCta& S) {
   __syncthreads();
-  if (threadIdx.x == 0) *S.emax = 0;
+  if (threadIdx.x == 0) {
+    *S.emax = 0;
+    *S.keep = 0u;
+  }
   __syncthreads();
   for (int k = threadIdx.x; k < 512; k += kRThreads) {
-    const int e = (kTrsm && k < a.n) ? a.eR[k] : 0;
-    S.eRs[k] = e;
     S.cmax[k] = 0u;
-    S.colE[k] = k < a.n ? a.colE[k] : 0;
-    if (kTrsm && e > 0) atomicMax(S.emax, e);
+    if (!kTrsm) S.colE[k] = k < a.n ? a.colE[k] : 0;
+    if (kTrsm) {
+      const int e = k < a.n ? a.eR[k] : 0, f = k < a.n ? a.fN[k] : 0;
+      const bool keep = k < a.n && a.flags[k / kRN] != 0;
+      S.colE[k] = k < a.n ? (keep ? a.colE2 : a.colE)[k] : 0;
+      S.eRs[k] = e;
+      S.fNs[k] = f;
+      if (max(e, f) > 0) atomicMax(S.emax, max(e, f));
+      if (keep && k % kRN == 0) atomicOr(S.keep, 1u << (k / kRN));
+    }
   }
   __syncthreads();
 }
@@ -244,10 +274,10 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
       mx = max(mx, (uint32_t)__double2hiint(*p) & 0x7FFFFFFFu);
       p += 2 * a.ldw;
     }
-    S.red[ph][pr] = mx;
+    S.red[ph][pr] = (int)mx;
     __syncthreads();
     if (tid < kM) {
-      const int E = (int)oz::exp_field(max(S.red[0][tid], S.red[1][tid]));
+      const int E = (int)oz::exp_field((uint32_t)max(S.red[0][tid], S.red[1][tid]));
       S.rowRef[tid] = E == 2047 ? kNonfinite : E == 0 ? kNoEntry : E;
     }
   } else if (tid < kM) {
@@ -256,23 +286,30 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   __syncthreads();
   const uint32_t tbase = S.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * 16);
   bool pending = false;
-  if (tid == 0) rp_fetch_b(a, S, S.bseq, kTrsm ? 0 : nt - 1, 0);
+  if (tid == 0) rp_fetch_b(a.Md, S, S.bseq, kTrsm ? 0 : nt - 1, 0);
   for (int ti = 0; ti < nt; ++ti) {
     const int t = kTrsm ? ti : nt - 1 - ti;
     const int c0 = t * kRN;
-    if (kTrsm) {   // the rows' reference exponents: W D so far and A_t
+    const bool keep = kTrsm && ((*S.keep >> t) & 1u) != 0u;
+    if (kTrsm) {   // the rows' reference exponents: W D so far and A_t F^{-1} (W D alone in a kept panel)
       load(a.A, a.lda, c0);
       uint32_t mx = 0u;
+      int me = INT_MIN;
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < 4; ++j) {
+        const int4 f4 = *reinterpret_cast<const int4*>(S.fNs + c0 + gcol[j]);
+        const int f[4] = {f4.x, f4.y, f4.z, f4.w};
 #pragma unroll
-        for (int c = 0; c < 4; ++c) mx = max(mx, (uint32_t)__double2hiint(v[j][c]) & 0x7FFFFFFFu);
-      S.red[ph][pr] = mx;
-      __syncthreads();
-      if (tid < kM) {
-        const int E = (int)oz::exp_field(max(S.red[0][tid], S.red[1][tid]));
-        S.rowRef[tid] = max(S.rowX[tid], E == 2047 ? kNonfinite : E == 0 ? kNoEntry : E);
+        for (int c = 0; c < 4; ++c) {
+          const uint32_t h = (uint32_t)__double2hiint(v[j][c]) & 0x7FFFFFFFu;
+          mx = max(mx, h);
+          if (h != 0u) me = max(me, (int)(h >> 2) + f[c] * (1 << 18));   // >> 2: room for both exponents
+          if (keep) v[j][c] = 0.0;
+        }
       }
+      S.red[ph][pr] = keep || mx == 0u ? kNoEntry : mx >= 0x7FF00000u ? kNonfinite : me >> 18;
+      __syncthreads();
+      if (tid < kM) S.rowRef[tid] = max(S.rowX[tid], max(S.red[0][tid], S.red[1][tid]));
       __syncthreads();
     } else {
       load(a.W, a.ldw, 0);
@@ -291,11 +328,11 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
       pending = false;
       const uint32_t stage = S.bseq & 1u, bpar = (S.bseq >> 1) & 1u;
       if (tid == 0) {   // the next multiplier block, into the stage that the finished batch read
-        if (i < t) rp_fetch_b(a, S, S.bseq + 1, t, kTrsm ? i : i + 1);
-        else if (ti + 1 < nt) rp_fetch_b(a, S, S.bseq + 1, kTrsm ? t + 1 : t - 1, kTrsm ? t + 1 : 0);
+        if (i < t) rp_fetch_b(keep ? a.Md2 : a.Md, S, S.bseq + 1, t, kTrsm ? i : i + 1);
+        else if (ti + 1 < nt) rp_fetch_b(a.Md, S, S.bseq + 1, kTrsm ? t + 1 : t - 1, kTrsm ? t + 1 : 0);
       }
       const int kW = kTrsm ? i - 1 : i;   // W chunk (TRSM: -1 is A_t)
-      rp_slice(v, kTrsm && i > 0 ? S.eRs + kRN * kW : nullptr, gcol, Eref, cr, tc::smem_u32(S.as), off);
+      rp_slice(v, !kTrsm ? nullptr : i > 0 ? S.eRs + kRN * kW : S.fNs + c0, gcol, Eref, cr, tc::smem_u32(S.as), off);
       tc::fence_proxy_async();
       tc::fence_before();
       __syncthreads();
@@ -330,7 +367,6 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
     tc::fence_before();
     // the tile: one rounding per entry
     const int Erow = S.rowRef[rr];
-    const bool keep = kTrsm && a.flags[t] != 0;
     double out[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
@@ -346,7 +382,9 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
     if (keep) {
       double* sb = reinterpret_cast<double*>(S.as);   // the chunk's panels are free
 #pragma unroll
-      for (int c = 0; c < 16; ++c) sb[(16 * g + c) * kM + rr] = out[c];
+      for (int c = 0; c < 16; ++c)
+        if (c0 + 16 * g + c < n)
+          sb[(16 * g + c) * kM + rr] = a.A[min(r0 + rr, a.m - 1) + (int64_t)(c0 + 16 * g + c) * a.lda] + out[c];
       __syncthreads();
       if (tid < kM) rp_substitute(a, sb, c0, tid);
       __syncthreads();
@@ -387,10 +425,12 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   __shared__ __align__(8) uint64_t bars_s[3];                                  \
   __shared__ uint32_t tmem_slot;                                               \
   __shared__ int dead_s, emax_s;                                               \
+  __shared__ uint32_t keep_s;                                                  \
   __shared__ int rowX_s[kM];                                                   \
   __shared__ int rowRef_s[kM];                                                 \
-  __shared__ uint32_t red_s[2][kM];                                            \
+  __shared__ int red_s[2][kM];                                                 \
   __shared__ __align__(16) int eRs_s[512];                                     \
+  __shared__ __align__(16) int fNs_s[512];                                     \
   __shared__ __align__(16) uint32_t cmax_s[512];                               \
   __shared__ __align__(16) int colE_s[512];                                             \
   if ((threadIdx.x >> 5) == 0) tc::tmem_alloc(&tmem_slot, kRTmem);             \
@@ -414,9 +454,11 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   S.rowRef = rowRef_s;                                                         \
   S.red = red_s;                                                               \
   S.eRs = eRs_s;                                                               \
+  S.fNs = fNs_s;                                                               \
   S.cmax = cmax_s;                                                             \
   S.colE = colE_s;                                                             \
-  S.emax = &emax_s;
+  S.emax = &emax_s;                                                            \
+  S.keep = &keep_s;
 
 // Every batch and every copy has been waited for unless a wait gave up; then
 // the outstanding ones get one more bounded wait before the TMEM is freed.
@@ -487,25 +529,55 @@ __global__ void __launch_bounds__(128) k_rp_prep_x(int n, int npad, const double
 }
 
 // ---------------------------------------------------------------------------
-// e_k = unbiased exponent of max_c |R[k][c]| (0 for a zero or non-finite row).
-// One warp per row.
-__device__ __forceinline__ void rp_row_scale_block(int n, int npad, const double* __restrict__ RT, int* __restrict__ eR,
+// -f_c = minus the unbiased exponent of max_k |R[k][c]| (0 for a zero or
+// non-finite column), 32 columns by the block's 256 threads; red: [8][32].
+__device__ __forceinline__ void rp_col_scale_block(int n, int npad, const double* __restrict__ RT, int* fN, int blk,
+                                                   int (*red)[kRN]) {
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, c = kRN * blk + lane;
+  uint32_t mx = 0u;
+  if (c < n)
+#pragma unroll 4
+    for (int k = g; k <= c; k += 8) mx = max(mx, (uint32_t)__double2hiint(RT[(int64_t)k * npad + c]) & 0x7FFFFFFFu);
+  __syncthreads();
+  red[g][lane] = (int)mx;
+  __syncthreads();
+  if (g == 0 && c < n) {
+    int all = 0;
+    for (int w = 0; w < 8; ++w) all = max(all, red[w][lane]);
+    const int E = (int)oz::exp_field((uint32_t)all);
+    fN[c] = (E == 0 || E == 2047) ? 0 : 1023 - E;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_rp_col_scale(int n, int npad, const double* __restrict__ RT, int* fN,
+                                                      const Ctl* ctl, int level) {
+  if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
+  __shared__ int red[8][kRN];
+  rp_col_scale_block(n, npad, RT, fN, blockIdx.x, red);
+}
+
+// e_k = unbiased exponent of max_c |R[k][c]| 2^-f_c (0 for a zero or non-finite
+// row).  One warp per row.
+__device__ __forceinline__ void rp_row_scale_block(int n, int npad, const double* __restrict__ RT, const int* fN, int* eR,
                                                    int blk) {
   const int k = blk * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (k >= n) return;
   uint32_t mx = 0u;
-  for (int c = lane; c < n; c += 32) mx = max(mx, (uint32_t)__double2hiint(RT[(int64_t)k * npad + c]) & 0x7FFFFFFFu);
-  mx = __reduce_max_sync(0xffffffffu, mx);
-  if (lane == 0) {
-    const int E = (int)oz::exp_field(mx);
-    eR[k] = (E == 0 || E == 2047) ? 0 : E - 1023;
+  int me = INT_MIN;
+  for (int c = lane; c < n; c += 32) {
+    const uint32_t h = (uint32_t)__double2hiint(RT[(int64_t)k * npad + c]) & 0x7FFFFFFFu;
+    mx = max(mx, h);
+    if (h >= 0x00100000u) me = max(me, (int)(h >> 20) + fN[c]);
   }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  me = __reduce_max_sync(0xffffffffu, me);
+  if (lane == 0) eR[k] = (mx >= 0x7FF00000u || me == INT_MIN) ? 0 : me - 1023;
 }
 
-__global__ void __launch_bounds__(256) k_rp_row_scale(int n, int npad, const double* __restrict__ RT,
-                                                      int* __restrict__ eR, const Ctl* ctl, int level) {
+__global__ void __launch_bounds__(256) k_rp_row_scale(int n, int npad, const double* __restrict__ RT, const int* fN,
+                                                      int* eR, const Ctl* ctl, int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
-  rp_row_scale_block(n, npad, RT, eR, blockIdx.x);
+  rp_row_scale_block(n, npad, RT, fN, eR, blockIdx.x);
 }
 
 // Multiplier digits of a 32-column panel t of W = A R^{-1} (top of the file);
@@ -514,7 +586,7 @@ __global__ void __launch_bounds__(256) k_rp_row_scale(int n, int npad, const dou
 // same in double-double would be eight times the instructions of the 1/64-rate
 // FP64 pipe).
 struct RpPrep {
-  double R[kRN][kRN + 1];       // R_tt (identity beyond column n)
+  double R[kRN][kRN + 1];       // (R F^{-1})_tt (identity beyond column n)
   double X[kRN][kRN + 1];       // its inverse in FP64
   float F[kRN][kRN + 1];        // I - R_tt X (scaled)
   long long Ri[kRN][kRN + 1];   // a block of R in fixed point, row k against er[k]
@@ -523,12 +595,17 @@ struct RpPrep {
   int red[8][kRN];
 };
 
-// Signed 63-bit fixed point of x against the exponent E: x 2^(1085 - E).
-__device__ __forceinline__ long long rp_fix(double x, int E) {
+// Signed 63-bit fixed point of x 2^eoff against the exponent E: x 2^(eoff + 1085 - E).
+__device__ __forceinline__ long long rp_fix(double x, int E, int eoff = 0) {
   const uint32_t h = (uint32_t)__double2hiint(x);
   const long long v =
-      (long long)(oz::biased_fixed63(h, (uint32_t)__double2loint(x), E, 0) - 0x0080808080808080ull);
+      (long long)(oz::biased_fixed63(h, (uint32_t)__double2loint(x), E, eoff) - 0x0080808080808080ull);
   return (h >> 31) ? -v : v;
+}
+
+// 2^e for -1023 <= e <= 1022.
+__device__ __forceinline__ double rp_pow2(int e) {
+  return e > -1023 ? __hiloint2double((e + 1023) << 20, 0) : __hiloint2double(0x00080000, 0);
 }
 
 // Index of the leading bit of |v|, -1 for zero.
@@ -538,9 +615,11 @@ __device__ __forceinline__ int rp_msb(__int128 v) {
   return h ? 127 - __clzll((long long)h) : l ? 63 - __clzll((long long)l) : -1;
 }
 
-// The block of R at (rows 32 kc .., columns of panel t) in fixed point, its
-// row references in er (over finite entries).  True if an entry is not finite.
-__device__ __forceinline__ bool rp_load_fixed(RpPrep& P, int n, int npad, const double* __restrict__ RT, int kc, int c0) {
+// The block of R F^{-1} at (rows 32 kc .., columns of panel t; f: -f_c of this
+// thread's column) in fixed point, its row references in er (over finite
+// entries).  True if an entry is not finite.
+__device__ __forceinline__ bool rp_load_fixed(RpPrep& P, int n, int npad, const double* __restrict__ RT, int kc, int c0,
+                                              int f) {
   const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
   bool bad = false;
 #pragma unroll
@@ -553,8 +632,9 @@ __device__ __forceinline__ bool rp_load_fixed(RpPrep& P, int n, int npad, const 
       x = 0.0;
       E = 0;
     }
-    const int Er = (int)__reduce_max_sync(0xffffffffu, (uint32_t)E);
-    P.Ri[k][c] = rp_fix(x, Er);
+    int Er = __reduce_max_sync(0xffffffffu, E ? E + f : kNoEntry);
+    if (Er == kNoEntry) Er = 0;
+    P.Ri[k][c] = rp_fix(x, Er, f);
     if (c == 0) P.er[k] = Er;
   }
   return bad;
@@ -567,31 +647,74 @@ __device__ __forceinline__ __int128 rp_dot(const RpPrep& P, int k, int c, int j0
   return acc;
 }
 
+// Multiplier of a panel that keeps its substitution: the digits of -D^{-1} R_{<t,t}
+// against the columns' largest entries (no X_t, no F: each column has its own reference).
+__device__ __forceinline__ void rp_prep_kept(RpPrep& P, int n, int npad, const double* __restrict__ RT, const RpInts& I,
+                                             unsigned char* __restrict__ Md2, int t) {
+  const int c = threadIdx.x & 31, g = threadIdx.x >> 5, c0 = kRN * t;
+  const bool live = c0 + c < n;
+  int mE = kNoEntry;
+  for (int k = g; k < c0; k += 8) {
+    const int E = live ? (int)oz::exp_field((uint32_t)__double2hiint(RT[(int64_t)k * npad + c0 + c])) : 0;
+    if (E != 0) mE = max(mE, E == 2047 ? kNonfinite : E - I.eR[k]);
+  }
+  __syncthreads();
+  P.red[g][c] = mE;
+  __syncthreads();
+  for (int k = 0; k < 8; ++k) mE = max(mE, P.red[k][c]);
+  if (g == 0) I.colE2[c0 + c] = mE;
+  for (int kc = 0; kc < t; ++kc) {
+    uint64_t J[4];
+    uint32_t neg[4], d[oz::kSlices][2], o[oz::kSlices];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int k = kRN * kc + 4 * g + r;
+      const double x = live && mE != kNonfinite ? RT[(int64_t)k * npad + c0 + c] : 0.0;
+      const uint32_t h = (uint32_t)__double2hiint(x);
+      J[r] = oz::biased_fixed63(h, (uint32_t)__double2loint(x), mE, -I.eR[k]);
+      neg[r] = (h >> 31) ^ 1u;
+    }
+    oz::digits8_pack(J[0], J[1], neg[0], neg[1], o);
+#pragma unroll
+    for (int b = 0; b < oz::kSlices; ++b) d[b][0] = o[b];
+    oz::digits8_pack(J[2], J[3], neg[2], neg[3], o);
+#pragma unroll
+    for (int b = 0; b < oz::kSlices; ++b) d[b][1] = o[b];
+    unsigned char* panel = Md2 + rp_block_offset(t, kc) + tc::sw64_offset(c, 4 * g, 2);
+#pragma unroll
+    for (int b = 0; b < oz::kSlices; ++b) *reinterpret_cast<uint2*>(panel + b * kRBPanel) = make_uint2(d[b][0], d[b][1]);
+  }
+}
+
 __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, const double* __restrict__ RT,
-                                                const double* __restrict__ rinv, int* eR, int* __restrict__ colE,
-                                                int* __restrict__ flags,
+                                                const double* __restrict__ rinv, const RpInts& I,
                                                 unsigned char* __restrict__ Md, uint32_t* __restrict__ colHiOut,
                                                 int nhi, int t) {
+  int *eR = I.eR, *fN = I.fN;
   const int tid = threadIdx.x, c = tid & 31, g = tid >> 5;   // this thread: column c, rows 4 g .. 4 g + 3
   const int c0 = kRN * t, w = min(kRN, n - c0);
   if (colHiOut && t == 0)     // the product folds the column maxima of W into these
     for (int i = tid; i < nhi; i += blockDim.x) colHiOut[i] = 0u;
-  if (n <= kRpOwnScale) {     // no launch for e_k: every panel finds its own rows' (they agree)
-    for (int blk = 0; blk < (min(n, c0 + kRN) + 7) / 8; ++blk) rp_row_scale_block(n, npad, RT, eR, blk);
+  if (n <= kRpOwnScale) {     // no launches for f_c and e_k: every panel finds them (they agree)
+    for (int blk = 0; blk < (n + kRN - 1) / kRN; ++blk) rp_col_scale_block(n, npad, RT, fN, blk, P.red);
+    __syncthreads();
+    for (int blk = 0; blk < (min(n, c0 + kRN) + 7) / 8; ++blk) rp_row_scale_block(n, npad, RT, fN, eR, blk);
   }
   __syncthreads();
-  // X = R_tt^{-1} by FP64 back substitution, column c in the lanes, rows over the warps
+  const int f = c < w ? fN[c0 + c] : 0;
+  // X = (R F^{-1})_tt^{-1} by FP64 back substitution, column c in the lanes, rows over the warps
+  const double scale = rp_pow2(f);
   double b[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int i = 4 * g + r;
-    P.R[i][c] = (i < w && c < w) ? (i <= c ? RT[(int64_t)(c0 + i) * npad + c0 + c] : 0.0) : (i == c ? 1.0 : 0.0);
+    P.R[i][c] = (i < w && c < w) ? (i <= c ? RT[(int64_t)(c0 + i) * npad + c0 + c] * scale : 0.0) : (i == c ? 1.0 : 0.0);
     b[r] = i == c ? 1.0 : 0.0;
   }
   __syncthreads();
 #pragma unroll
   for (int k = kRN - 1; k >= 0; --k) {
-    if ((k >> 2) == g) P.X[k][c] = k >= w ? b[k & 3] : c < k ? 0.0 : b[k & 3] * rinv[c0 + k];
+    if ((k >> 2) == g) P.X[k][c] = k >= w ? b[k & 3] : c < k ? 0.0 : b[k & 3] * (rinv[c0 + k] * rp_pow2(-fN[c0 + k]));
     if (k >= w) continue;   // identity beyond column n
     __syncthreads();
     const double x = P.X[k][c];
@@ -654,20 +777,12 @@ __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, cons
 #pragma unroll
     for (int r = 0; r < 4; ++r) P.Xi[4 * g + r][c] += add[r];
   }
-  bool keep = false;
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    if (attempt == 1) {   // the panel keeps its substitution: X = I
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < 4; ++r) P.Xi[4 * g + r][c] = 4 * g + r == c ? 1ll << 61 : 0;
-      if (g == 0) P.Ex[c] = 1024;
-      keep = true;
-    }
+  // column references over (D^-1 Z; X)
+  bool nf = false;
+  {
     __syncthreads();
-    // column references over (D^-1 Z; X)
     const int Ex = P.Ex[c];
     int mE = kNoEntry;
-    bool nf = false;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int p = rp_msb(P.Xi[4 * g + r][c]);
@@ -675,12 +790,12 @@ __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, cons
     }
     for (int kc = 0; kc < t; ++kc) {
       __syncthreads();
-      nf |= rp_load_fixed(P, n, npad, RT, kc, c0);
+      nf |= rp_load_fixed(P, n, npad, RT, kc, c0, f);
       __syncthreads();
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const int k = 4 * g + r;
-        const int p = rp_msb(rp_dot(P, k, c, keep ? c : 0));
+        const int p = rp_msb(rp_dot(P, k, c, 0));
         if (p >= 0) mE = max(mE, p + P.er[k] + Ex - 1141 - eR[kRN * kc + k]);
       }
     }
@@ -692,31 +807,30 @@ __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, cons
       P.cE[c] = mE;
     }
     __syncthreads();
-    if (attempt == 0) {
-      float amp = 0.0f;   // sum_i 2^(cE_i - 1022) |R[i][c]|: four rows a thread, then over the warps
+    float amp = 0.0f;   // sum_i 2^(cE_i - 1022) |R[i][c]|: four rows a thread, then over the warps
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const uint32_t h = (uint32_t)__double2hiint(P.R[4 * g + r][c]) & 0x7FFFFFFFu;
-        const float f = __uint_as_float(0x3F800000u | ((h & 0xFFFFFu) << 3) | 7u);   // significand, rounded up
-        if (h) amp += ldexpf(f, (int)oz::exp_field(h) - 1023 + P.cE[4 * g + r] - 1022);
-      }
-      P.red[g][c] = __float_as_int(amp);
-      __syncthreads();
-      if (g == 0) {
-        for (int k = 1; k < 8; ++k) amp += __int_as_float(P.red[k][c]);
-        if (!(amp <= kAmpLimit)) bad = true;
-      }
-      if (!__syncthreads_or(bad || nf)) break;
+    for (int r = 0; r < 4; ++r) {
+      const uint32_t h = (uint32_t)__double2hiint(P.R[4 * g + r][c]) & 0x7FFFFFFFu;
+      const float s = __uint_as_float(0x3F800000u | ((h & 0xFFFFFu) << 3) | 7u);   // significand, rounded up
+      if (h) amp += ldexpf(s, (int)oz::exp_field(h) - 1023 + P.cE[4 * g + r] - 1022);
+    }
+    P.red[g][c] = __float_as_int(amp);
+    __syncthreads();
+    if (g == 0) {
+      for (int k = 1; k < 8; ++k) amp += __int_as_float(P.red[k][c]);
+      if (!(amp <= kAmpLimit)) bad = true;
     }
   }
-  // digits
-  if (g == 0 && c < w) colE[c0 + c] = P.cE[c];
-  if (tid == 0) flags[t] = keep ? 1 : 0;
+  const bool keep = __syncthreads_or(bad || nf) != 0;
+  if (tid == 0) I.flags[t] = keep ? 1 : 0;
+  if (keep) rp_prep_kept(P, n, npad, RT, I, Md + rp_digit_size(n), t);
+  // digits (of a kept panel only the block of X is copied, and multiplied by zeros)
+  if (g == 0 && c < w) I.colE[c0 + c] = P.cE[c];
   const int Ex = P.Ex[c], cE = P.cE[c];
   for (int kc = 0; kc <= t; ++kc) {
     if (kc < t) {
       __syncthreads();
-      rp_load_fixed(P, n, npad, RT, kc, c0);
+      rp_load_fixed(P, n, npad, RT, kc, c0, f);
       __syncthreads();
     }
     uint32_t d[oz::kSlices][2];
@@ -728,7 +842,7 @@ __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, cons
       __int128 acc;
       int sh;   // I = |acc| 2^-sh
       if (kc < t) {
-        acc = -rp_dot(P, k, c, keep ? c : 0);
+        acc = -rp_dot(P, k, c, 0);
         sh = cE - P.er[k] - Ex + eR[kRN * kc + k] + 1079;
       } else {
         acc = P.Xi[k][c];
@@ -758,14 +872,12 @@ __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, cons
 }
 
 __global__ void __launch_bounds__(256) k_rp_prep_r(int n, int npad, const double* __restrict__ RT,
-                                                   const double* __restrict__ rinv, int* eR, int* __restrict__ colE,
-                                                   int* __restrict__ flags,
+                                                   const double* __restrict__ rinv, RpInts I,
                                                    unsigned char* __restrict__ Md, uint32_t* __restrict__ colHiOut,
                                                    int nhi, const Ctl* ctl, int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
   extern __shared__ unsigned char prep_raw[];
-  rp_prep_r_panel(*reinterpret_cast<RpPrep*>(prep_raw), n, npad, RT, rinv, eR, colE, flags, Md, colHiOut, nhi,
-                  blockIdx.x);
+  rp_prep_r_panel(*reinterpret_cast<RpPrep*>(prep_raw), n, npad, RT, rinv, I, Md, colHiOut, nhi, blockIdx.x);
 }
 
 int rp_sms() {
@@ -779,8 +891,6 @@ int rp_sms() {
   return cached;
 }
 
-int rp_n32(int n) { return (n + kRN - 1) / kRN * kRN; }
-
 // ---------------------------------------------------------------------------
 // Grouped forms for batched plans: persistent launches over {problem, block}
 // items; an item whose problem is not active at this level, or has raised a
@@ -792,14 +902,21 @@ __device__ __forceinline__ bool rp_live(const Prob& P, int level) {
 
 __device__ __forceinline__ int rp_nhi(int n) { return (n + kM - 1) / kM * kM; }
 
-// oz_cole: column exponents (n32 ints), e_k (n32 ints), panel flags (16 ints).
+__host__ __device__ __forceinline__ RpArgs rp_trsm_args(int64_t m, int n, const double* A, int64_t lda, double* W,
+                                                        int64_t ldw, int* ints, const unsigned char* Rd,
+                                                        const double* RT, const double* rinv, uint32_t* colHiOut) {
+  const RpInts I(ints, n);
+  return RpArgs{m, n, A, lda, W, ldw, I.colE, Rd, I.colE2, Rd + rp_digit_size(n), I.eR, I.fN, I.flags, RT, rinv, colHiOut};
+}
+
+__host__ __device__ __forceinline__ RpArgs rp_fin_args(int64_t m, int n, double* Q, int64_t ldq, const int* colE,
+                                                       const unsigned char* Xs, uint32_t* colHiOut) {
+  return RpArgs{m, n, nullptr, 0, Q, ldq, colE, Xs, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, colHiOut};
+}
+
 __device__ __forceinline__ RpArgs rp_args_of(const Prob& P, bool trsm) {
-  const int n32 = (P.n + kRN - 1) / kRN * kRN;
-  if (trsm)
-    return RpArgs{P.m, P.n, P.A, P.lda, P.Q, P.ldq, P.oz_cole, P.oz_rd, P.oz_cole + n32, P.oz_cole + 2 * n32, P.rst,
-                  P.rinv, P.oz_colhi};
-  return RpArgs{P.m, P.n, nullptr, 0, P.Q, P.ldq, P.oz_xe, P.oz_xs, nullptr, nullptr, nullptr, nullptr,
-                P.check ? P.oz_colhi : nullptr};
+  if (trsm) return rp_trsm_args(P.m, P.n, P.A, P.lda, P.Q, P.ldq, P.oz_cole, P.oz_rd, P.rst, P.rinv, P.oz_colhi);
+  return rp_fin_args(P.m, P.n, P.Q, P.ldq, P.oz_xe, P.oz_xs, P.check ? P.oz_colhi : nullptr);
 }
 
 template <bool kTrsm>
@@ -842,12 +959,23 @@ __global__ void __launch_bounds__(128) kg_rp_prep_x(Group g, int level) {
   }
 }
 
+__global__ void __launch_bounds__(256) kg_rp_col_scale(Group g, int level) {
+  __shared__ int red[8][kRN];
+  for (int it = blockIdx.x; it < g.nitems; it += gridDim.x) {
+    const int4 w = g.items[it];
+    const Prob& P = g.probs[w.x];
+    if (!rp_live(P, level)) continue;
+    rp_col_scale_block(P.n, P.npad, P.rst, RpInts(P.oz_cole, P.n).fN, w.y, red);
+  }
+}
+
 __global__ void __launch_bounds__(256) kg_rp_row_scale(Group g, int level) {
   for (int it = blockIdx.x; it < g.nitems; it += gridDim.x) {
     const int4 w = g.items[it];
     const Prob& P = g.probs[w.x];
     if (!rp_live(P, level)) continue;
-    rp_row_scale_block(P.n, P.npad, P.rst, P.oz_cole + (P.n + kRN - 1) / kRN * kRN, w.y);
+    const RpInts I(P.oz_cole, P.n);
+    rp_row_scale_block(P.n, P.npad, P.rst, I.fN, I.eR, w.y);
   }
 }
 
@@ -857,10 +985,9 @@ __global__ void __launch_bounds__(256) kg_rp_prep_r(Group g, int level) {
     const int4 w = g.items[it];
     const Prob& P = g.probs[w.x];
     if (!rp_live(P, level)) continue;
-    const int n32 = (P.n + kRN - 1) / kRN * kRN;
     __syncthreads();
-    rp_prep_r_panel(*reinterpret_cast<RpPrep*>(prep_raw), P.n, P.npad, P.rst, P.rinv, P.oz_cole + n32, P.oz_cole,
-                    P.oz_cole + 2 * n32, P.oz_rd, P.oz_colhi, rp_nhi(P.n), w.y);
+    rp_prep_r_panel(*reinterpret_cast<RpPrep*>(prep_raw), P.n, P.npad, P.rst, P.rinv, RpInts(P.oz_cole, P.n), P.oz_rd,
+                    P.oz_colhi, rp_nhi(P.n), w.y);
   }
 }
 
@@ -880,9 +1007,10 @@ unsigned rp_grid(int nitems, int per_sm) {
 
 }  // namespace
 
-// Workspace sizes: digit panels of the multiplier blocks, and the exponents.
-size_t rp_digit_bytes(int n) { return rp_block_offset(rp_n32(n) / kRN, 0); }
-size_t rp_trsm_ints_bytes(int n) { return sizeof(int) * (size_t)(2 * rp_n32(n) + 16); }
+// Workspace sizes: digit panels of the multiplier blocks (the TRSM has two sets), and the exponents.
+size_t rp_digit_bytes(int n) { return rp_digit_size(n); }
+size_t rp_trsm_digit_bytes(int n) { return 2 * rp_digit_size(n); }
+size_t rp_trsm_ints_bytes(int n) { return sizeof(int) * (size_t)(4 * rp_n32(n) + 16); }
 size_t rp_fin_ints_bytes(int n) { return sizeof(int) * (size_t)rp_n32(n); }
 int rp_cols(int n) { return rp_n32(n); }
 int rp_panels(int n) { return rp_n32(n) / kRN; }
@@ -892,12 +1020,14 @@ void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double
                     uint32_t* colHiOut) {
   const int n32 = rp_n32(n);
   const int nhi = (int)(syrk_oz_colhi_bytes(n) / sizeof(uint32_t));
-  int *colE = ints, *eR = ints + n32, *flags = ints + 2 * n32;
-  if (n > kRpOwnScale) launch_dep(k_rp_row_scale, (n + 7) / 8, 256, 0, st, n, n32, RT, eR, ctl, level);
+  const RpInts I(ints, n);
+  if (n > kRpOwnScale) {
+    launch_dep(k_rp_col_scale, n32 / kRN, 256, 0, st, n, n32, RT, I.fN, ctl, level);
+    launch_dep(k_rp_row_scale, (n + 7) / 8, 256, 0, st, n, n32, RT, I.fN, I.eR, ctl, level);
+  }
   cudaFuncSetAttribute(k_rp_prep_r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RpPrep));
-  launch_dep(k_rp_prep_r, n32 / kRN, 256, sizeof(RpPrep), st, n, n32, RT, rinv, eR, colE, flags, Rd, colHiOut, nhi, ctl, level);
-  const RpArgs a{m, n, A, lda, W, ldw, colE, Rd, eR, flags, RT, rinv, colHiOut};
-  rp_launch<true>(a, ctl, level, st);
+  launch_dep(k_rp_prep_r, n32 / kRN, 256, sizeof(RpPrep), st, n, n32, RT, rinv, I, Rd, colHiOut, nhi, ctl, level);
+  rp_launch<true>(rp_trsm_args(m, n, A, lda, W, ldw, ints, Rd, RT, rinv, colHiOut), ctl, level, st);
 }
 
 void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* XT, int* colE, unsigned char* Xs,
@@ -905,8 +1035,7 @@ void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* 
   const int n32 = rp_n32(n);
   const int nhi = (int)(syrk_oz_colhi_bytes(n) / sizeof(uint32_t));
   launch_dep(k_rp_prep_x, n32, 128, 0, st, n, n32, XT, colE, Xs, colHiOut, nhi, ctl, level);
-  const RpArgs a{m, n, nullptr, 0, Q, ldq, colE, Xs, nullptr, nullptr, nullptr, nullptr, colHiOut};
-  rp_launch<false>(a, ctl, level, st);
+  rp_launch<false>(rp_fin_args(m, n, Q, ldq, colE, Xs, colHiOut), ctl, level, st);
 }
 
 void prepare_g_rowprod() {
@@ -915,6 +1044,9 @@ void prepare_g_rowprod() {
   cudaFuncSetAttribute(kg_rp_prep_r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RpPrep));
 }
 
+void launch_g_oz_col_scale(const Group& g, int level, cudaStream_t st) {
+  if (g.nitems) { ::mrcqr::note_launch(); kg_rp_col_scale<<<rp_grid(g.nitems, 8), 256, 0, st>>>(g, level); }
+}
 void launch_g_oz_row_scale(const Group& g, int level, cudaStream_t st) {
   if (g.nitems) { ::mrcqr::note_launch(); kg_rp_row_scale<<<rp_grid(g.nitems, 16), 256, 0, st>>>(g, level); }
 }
