@@ -298,7 +298,8 @@ int enqueue_sketch(const Plan& p, void* ws, int prec, int variant, int fp64_prod
 }
 
 void enqueue_stage2(const Plan& p, void* ws, const double* A, int64_t lda, double* Q, int64_t ldq, double* R,
-                    int64_t ldr, int check, Ctl* ctl, int lvl, cudaStream_t st, int fp64_products = 0) {
+                    int64_t ldr, int check, Ctl* ctl, int lvl, cudaStream_t st, int fp64_products = 0,
+                    bool rs_given = false) {
   double* RsT = at<double>(ws, p.off_rst);
   double* rinv = at<double>(ws, p.off_rinv);
   double* Gpart = at<double>(ws, p.off_gpart);
@@ -311,7 +312,7 @@ void enqueue_stage2(const Plan& p, void* ws, const double* A, int64_t lda, doubl
   if (emu)
     launch(SG_TRSM, lvl, st, [&] {
       launch_trsm_oz(p.m, p.n, A, lda, RsT, rinv, at<int>(ws, p.off_tcole), at<unsigned char>(ws, p.off_trd), Q,
-                     ldq, ctl, lvl, st, colhi);
+                     ldq, ctl, lvl, st, colhi, rs_given);
     });
   else
     launch(SG_TRSM, lvl, st, [&] { launch_trsm(p.m, p.n, A, lda, RsT, rinv, Q, ldq, ctl, lvl, st); });
@@ -645,7 +646,7 @@ int mrcqr_cholqr_precond(int64_t m, int64_t n, const double* A, int64_t lda, con
   launch(SG_INIT, 0, st, [&] { launch_dep(k_init_ctl, 1, 1, 0, st, ctl, 1, P_FP64, P_FP64, P_FP64, P_FP64, kDefaultTol); });
   cudaMemcpyAsync(at<double>(ws, p.off_rs), Rs, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, st);
   launch(SG_PREP, 0, st, [&] { launch_rs_prepare((int)n, Rs, at<double>(ws, p.off_rst), at<double>(ws, p.off_rinv), st); });
-  enqueue_stage2(p, ws, A, lda, Q, ldq, R, ldr, 1, ctl, 0, st);
+  enqueue_stage2(p, ws, A, lda, Q, ldq, R, ldr, 1, ctl, 0, st, 0, true);
   launch(SG_STATS, 0, st, [&] { launch_dep(k_write_stats, 1, 1, 0, st, ctl, slot); });
   cudaFreeAsync(ws, st);
   return finish(st);
@@ -677,7 +678,7 @@ int mrcqr_trsm(int64_t m, int64_t n, const double* A, int64_t lda, const double*
   if (fp64_products == 0)
     launch(SG_TRSM, 0, st, [&] {
       launch_trsm_oz(m, (int)n, A, lda, RsT, rinv, at<int>(ws, p.off_tcole), at<unsigned char>(ws, p.off_trd), W,
-                     ldw, ctl, 0, st);
+                     ldw, ctl, 0, st, nullptr, true);
     });
   else
     launch(SG_TRSM, 0, st, [&] { launch_trsm(m, (int)n, A, lda, RsT, rinv, W, ldw, ctl, 0, st); });

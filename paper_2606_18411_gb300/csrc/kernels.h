@@ -233,6 +233,7 @@ void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, con
 // Workspace: digit panels of the multiplier (two sets for the TRSM), the TRSM's integers (column exponents,
 // row and column scalings, panel flags), the finalize's column exponents; columns and 32-column panels of n.
 constexpr int kRpOwnScale = 128;   // up to this n the TRSM's preparation finds the scalings itself (no launches)
+// check: R need not be a factor of A (its column sizes may say nothing about A's or W's); the row blocks look.
 size_t rp_digit_bytes(int n);
 size_t rp_trsm_digit_bytes(int n);
 size_t rp_trsm_ints_bytes(int n);
@@ -241,7 +242,7 @@ int rp_cols(int n);
 int rp_panels(int n);
 void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double* RT, const double* rinv, int* ints,
                     unsigned char* Rd, double* W, int64_t ldw, Ctl* ctl, int level, cudaStream_t st,
-                    uint32_t* colHiOut = nullptr);
+                    uint32_t* colHiOut = nullptr, bool check = false);
 void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* XT, int* colE, unsigned char* Xs,
                         Ctl* ctl, int level, cudaStream_t st, uint32_t* colHiOut = nullptr);
 

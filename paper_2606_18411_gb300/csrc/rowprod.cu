@@ -29,12 +29,16 @@
 //    matrices with kappa up to 1e16, four spectra, n = 32 .. 512) keeps the
 //    substitution: the product is W_{<t} (-R_{<t,t}) alone (A's digits are
 //    zeros in it), A_t is added and R_tt solved with in FP64.
+//    F fits A where W's columns are of one size, as for a factor R of A.  Where R is
+//    the caller's (mrcqr_trsm, mrcqr_cholqr_precond) a row block checks it: a panel with a
+//    column of A F^{-1} below 2^-10 of the largest entry of the block's A F^{-1} or W D
+//    would lose that column's digits, and is solved by substitution as well.
 //
 // Measured at m = 2^20 (before: substitution blocks of 16 columns; Q = W X in
 // 128 x 64 tiles by one CTA per SM): W = A R^{-1} 1.78 -> 0.75 ms at n = 64,
-// 4.53 -> 1.80 at 128, 12.7 -> 5.9 at 256, 41.3 -> 20.5 at 512 (the column scales cost
-// nothing there: m = 300001, n = 320 2.94 ms without and 2.93 with them; 3 us of the 280 at
-// m = 4096, n = 32); Q = W X
+// 4.53 -> 1.80 at 128, 12.7 -> 5.9 at 256, 41.3 -> 20.5 at 512 (m = 300001, n = 320: 2.94 ms
+// with one reference for all columns, 2.93 with the column scales, 2.99 with the check of
+// an R of the caller's); Q = W X
 // 0.99 -> 0.63, 2.19 -> 1.61, 5.67 -> 5.39, 17.3 -> 18.6.  What bounds them is
 // integer-pipe work around the products (slicing about 1100 cycles per SM and
 // chunk, conversion of the results about 2400 per tile, against 1340 of MMAs
@@ -58,6 +62,9 @@ namespace {
 constexpr size_t kRSmem = (size_t)kRABytes + 2 * (size_t)kRBBytes + 1024;
 constexpr int kNoEntry = -100000, kNonfinite = 100000;
 constexpr float kAmpLimit = 512.0f;
+// Binades a column of A F^{-1} may lie below the block's largest entry: 2^-62 2^10 amp sqrt(n) stays at the n u of a
+// triangular solve, and a matched R reaches 2^7 (largest of 128 n Gaussians times sqrt(n) against a column's largest).
+constexpr int kBalance = 10;
 
 // Multiplier block (t, kc), kc <= t.
 __host__ __device__ __forceinline__ size_t rp_block_offset(int t, int kc) {
@@ -110,6 +117,8 @@ struct RpCta {
   int* colE;                    // reference exponents of the multiplier columns
   int* emax;                    // largest of the scalings e_k, -f_c and 0
   uint32_t* keep;               // bit t: panel t keeps its substitution
+  int* rho;                     // checked solve: largest rowRef of each 32 rows
+  uint32_t* mask;               // columns 16 h .. of the panel with an entry near them [h]; with any entry [2 + h]
 };
 
 __device__ __forceinline__ void rp_wait(RpCta& S, uint64_t* bar, uint32_t parity) {
@@ -177,8 +186,9 @@ __device__ __forceinline__ void rp_begin(const RpArgs& a, RpCta& S) {
     if (!kTrsm) S.colE[k] = k < a.n ? a.colE[k] : 0;
     if (kTrsm) {
       const int e = k < a.n ? a.eR[k] : 0, f = k < a.n ? a.fN[k] : 0;
+      const int E1 = k < a.n ? a.colE[k] : 0, E2 = k < a.n ? a.colE2[k] : 0;   // loads side by side
       const bool keep = k < a.n && a.flags[k / kRN] != 0;
-      S.colE[k] = k < a.n ? (keep ? a.colE2 : a.colE)[k] : 0;
+      S.colE[k] = keep ? E2 : E1;
       S.eRs[k] = e;
       S.fNs[k] = f;
       if (max(e, f) > 0) atomicMax(S.emax, max(e, f));
@@ -210,11 +220,50 @@ __device__ __noinline__ void rp_substitute(const RpArgs& a, double* sb, int c0, 
   }
 }
 
+// Checked solve: the exponent that every column of A F^{-1} in the panel should reach in the row block.
+__device__ __forceinline__ int rp_threshold(const RpCta& S) {
+  return max(max(max(S.rho[0], S.rho[1]), max(S.rho[2], S.rho[3])) - kBalance, -4000);
+}
+
+// Whether every column of the panel at c0 that has an entry in the row block
+// has one near the block's largest (every thread).  The full look, for panels
+// where the first 32 rows do not show it.
+__device__ __noinline__ bool rp_balanced_full(const RpArgs& a, const int* fNs, uint32_t* mask, int thr, int64_t r0,
+                                              int c0) {
+  const int tid = threadIdx.x, pr = tid & (kM - 1), ph = tid >> 7;
+  __syncthreads();
+  if (tid < 4) mask[tid] = 0u;
+  __syncthreads();
+  const double* p = a.A + min(r0 + pr, a.m - 1) + (int64_t)(c0 + 16 * ph) * a.lda;
+  uint32_t near = 0u, any = 0u;
+  for (int c = 0; c < 16 && c0 + 16 * ph + c < a.n; ++c, p += a.lda) {
+    const uint32_t h = (uint32_t)__double2hiint(*p) & 0x7FFFFFFFu;
+    if (h == 0u || h >= 0x7FF00000u) continue;
+    any |= 1u << c;
+    if ((int)(h >> 2) + fNs[c0 + 16 * ph + c] * (1 << 18) >= thr) near |= 1u << c;
+  }
+  near = __reduce_or_sync(0xffffffffu, near);
+  any = __reduce_or_sync(0xffffffffu, any);
+  if ((tid & 31) == 0) {
+    atomicOr(&mask[ph], near);
+    atomicOr(&mask[2 + ph], any);
+  }
+  __syncthreads();
+  return ((mask[2] & ~mask[0]) | (mask[3] & ~mask[1])) == 0u;
+}
+
+__device__ __forceinline__ bool rp_balanced(const RpArgs& a, const RpCta& S, int64_t r0, int c0) {
+  const uint32_t all = min(kRN, a.n - c0) == kRN ? 0xFFFFFFFFu : (1u << (a.n - c0)) - 1u;
+  return ((S.mask[0] | S.mask[1] << 16) & all) == all ||
+         rp_balanced_full(a, S.fNs, S.mask, rp_threshold(S) * (1 << 18), r0, c0);
+}
+
 // One block of 128 rows from r0; the CTA's next block is `next` blocks further (0: unknown).  False when a wait
 // gave up (every thread).
 // kMulti: K may exceed 128 (n > 128), so the level sums are read out and added up several times per tile; else the
 // sums of a tile are live only after its last chunk, which leaves the slicing their 64 registers.
-template <bool kTrsm, bool kMulti>
+// kCheck: the row block decides by its own A whether a panel keeps its substitution (top of the file).
+template <bool kTrsm, bool kMulti, bool kCheck>
 __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, int next) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n = a.n, nt = (n + kRN - 1) / kRN;
@@ -290,7 +339,7 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   for (int ti = 0; ti < nt; ++ti) {
     const int t = kTrsm ? ti : nt - 1 - ti;
     const int c0 = t * kRN;
-    const bool keep = kTrsm && ((*S.keep >> t) & 1u) != 0u;
+    bool keep = kTrsm && ((*S.keep >> t) & 1u) != 0u;
     if (kTrsm) {   // the rows' reference exponents: W D so far and A_t F^{-1} (W D alone in a kept panel)
       load(a.A, a.lda, c0);
       uint32_t mx = 0u;
@@ -304,20 +353,49 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
           const uint32_t h = (uint32_t)__double2hiint(v[j][c]) & 0x7FFFFFFFu;
           mx = max(mx, h);
           if (h != 0u) me = max(me, (int)(h >> 2) + f[c] * (1 << 18));   // >> 2: room for both exponents
-          if (keep) v[j][c] = 0.0;
         }
       }
       S.red[ph][pr] = keep || mx == 0u ? kNoEntry : mx >= 0x7FF00000u ? kNonfinite : me >> 18;
       __syncthreads();
-      if (tid < kM) S.rowRef[tid] = max(S.rowX[tid], max(S.red[0][tid], S.red[1][tid]));
+      if (tid < kM) {
+        const int E = max(S.rowX[tid], max(S.red[0][tid], S.red[1][tid]));
+        S.rowRef[tid] = E;
+        if (kCheck) {
+          const int rho = __reduce_max_sync(0xffffffffu, E != kNonfinite ? E : kNoEntry);
+          if (lane == 0) S.rho[warp] = rho;
+        }
+      }
       __syncthreads();
+      if (kCheck && (warp & 3) == 0) {   // do 32 rows show every column near the block's largest entry?
+        const int thr = rp_threshold(S) * (1 << 18);
+        uint32_t mask = 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int4 f4 = *reinterpret_cast<const int4*>(S.fNs + c0 + gcol[j]);
+          const int f[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const uint32_t h = (uint32_t)__double2hiint(v[j][c]) & 0x7FFFFFFFu;
+            if (h < 0x7FF00000u && (int)(h >> 2) + f[c] * (1 << 18) >= thr) mask |= 1u << (4 * j + c);
+          }
+        }
+        if (rot) mask = (mask & 0x0F0Fu) << 4 | ((mask >> 4) & 0x0F0Fu);   // from the lane's order to the columns'
+        mask = __reduce_or_sync(0xffffffffu, mask);
+        if (lane == 0) S.mask[ph] = mask;
+      }
+      if (keep) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) v[j][c] = 0.0;
+      }
     } else {
       load(a.W, a.ldw, 0);
     }
-    const int Eref = S.rowRef[pr];
+    int Eref = S.rowRef[pr];
     // constant of the fast slicing; a reference so small that a zero's exponent field could pass for a
     // value's takes the general form throughout
-    const int cr = Eref - *S.emax > 31 ? 31 - Eref : -(1 << 30);
+    int cr = Eref - *S.emax > 31 ? 31 - Eref : -(1 << 30);
     long long hi[16], lo[16];
     if (kMulti) {
 #pragma unroll
@@ -328,15 +406,34 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
       pending = false;
       const uint32_t stage = S.bseq & 1u, bpar = (S.bseq >> 1) & 1u;
       if (tid == 0) {   // the next multiplier block, into the stage that the finished batch read
-        if (i < t) rp_fetch_b(keep ? a.Md2 : a.Md, S, S.bseq + 1, t, kTrsm ? i : i + 1);
-        else if (ti + 1 < nt) rp_fetch_b(a.Md, S, S.bseq + 1, kTrsm ? t + 1 : t - 1, kTrsm ? t + 1 : 0);
+        if (i < t) {
+          if (!(kCheck && i == 0)) rp_fetch_b(keep ? a.Md2 : a.Md, S, S.bseq + 1, t, kTrsm ? i : i + 1);
+        } else if (ti + 1 < nt) {
+          rp_fetch_b(a.Md, S, S.bseq + 1, kTrsm ? t + 1 : t - 1, kTrsm ? t + 1 : 0);
+        }
       }
       const int kW = kTrsm ? i - 1 : i;   // W chunk (TRSM: -1 is A_t)
       rp_slice(v, !kTrsm ? nullptr : i > 0 ? S.eRs + kRN * kW : S.fNs + c0, gcol, Eref, cr, tc::smem_u32(S.as), off);
       tc::fence_proxy_async();
       tc::fence_before();
       __syncthreads();
+      if (kCheck && i == 0 && !keep && !rp_balanced(a, S, r0, c0)) {   // uniform: A's digits are zeros after all
+        keep = true;
+        if (tid < kM) S.rowRef[tid] = S.rowX[tid];
+        if (tid < kRN && c0 + tid < n) S.colE[c0 + tid] = a.colE2[c0 + tid];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) v[j][c] = 0.0;
+        __syncthreads();
+        Eref = S.rowRef[pr];
+        cr = Eref - *S.emax > 31 ? 31 - Eref : -(1 << 30);
+        rp_slice(v, nullptr, gcol, Eref, cr, tc::smem_u32(S.as), off);
+        tc::fence_proxy_async();
+        __syncthreads();
+      }
       if (tid == 0) {
+        if (kCheck && i == 0 && t > 0) rp_fetch_b(keep ? a.Md2 : a.Md, S, S.bseq + 1, t, 0);   // the panel's way is known
         rp_wait(S, &S.bar[1 + stage], bpar);
         tc::fence_after();
         rp_issue(S.tmem, tc::smem_u32(S.as), tc::smem_u32(S.bs + stage * kRBBytes), kMulti ? i % kGroupChunks == 0 : i == 0);
@@ -416,6 +513,7 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
       if (kTrsm && mxh != 0u) atomicMax(&S.rowX[rr], mxh >= 0x7FF00000u ? kNonfinite : mxE >> 18);
     }
     if (__syncthreads_or(*(volatile int*)S.dead)) return false;   // the tile's W is visible to the next tile's loads
+    if (kCheck && keep && ((*S.keep >> t) & 1u) == 0u && tid < kRN && c0 + tid < n) S.colE[c0 + tid] = a.colE[c0 + tid];
   }
   return true;
 }
@@ -426,6 +524,8 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   __shared__ uint32_t tmem_slot;                                               \
   __shared__ int dead_s, emax_s;                                               \
   __shared__ uint32_t keep_s;                                                  \
+  __shared__ int rho_s[kM / 32];                                               \
+  __shared__ uint32_t mask_s[4];                                               \
   __shared__ int rowX_s[kM];                                                   \
   __shared__ int rowRef_s[kM];                                                 \
   __shared__ int red_s[2][kM];                                                 \
@@ -458,7 +558,9 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   S.cmax = cmax_s;                                                             \
   S.colE = colE_s;                                                             \
   S.emax = &emax_s;                                                            \
-  S.keep = &keep_s;
+  S.keep = &keep_s;                                                            \
+  S.rho = rho_s;                                                               \
+  S.mask = mask_s;
 
 // Every batch and every copy has been waited for unless a wait gave up; then
 // the outstanding ones get one more bounded wait before the TMEM is freed.
@@ -473,7 +575,7 @@ __device__ __forceinline__ void rp_cta_end(RpCta& S, bool abort, Ctl* ctl) {
   if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(S.tmem, kRTmem);
 }
 
-template <bool kTrsm, bool kMulti>
+template <bool kTrsm, bool kMulti, bool kCheck>
 __global__ void __launch_bounds__(kRThreads, 2) k_rowprod(RpArgs a, Ctl* ctl, int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
   MRCQR_RP_CTA(S)
@@ -481,7 +583,7 @@ __global__ void __launch_bounds__(kRThreads, 2) k_rowprod(RpArgs a, Ctl* ctl, in
   bool abort = false;
   const int64_t nblocks = (a.m + kM - 1) / kM;
   for (int64_t rb = blockIdx.x; rb < nblocks; rb += gridDim.x)
-    if (!rp_block<kTrsm, kMulti>(a, S, rb * kM, (int)gridDim.x)) {
+    if (!rp_block<kTrsm, kMulti, kCheck>(a, S, rb * kM, (int)gridDim.x)) {
       abort = true;
       break;
     }
@@ -536,7 +638,7 @@ __device__ __forceinline__ void rp_col_scale_block(int n, int npad, const double
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, c = kRN * blk + lane;
   uint32_t mx = 0u;
   if (c < n)
-#pragma unroll 4
+#pragma unroll 8
     for (int k = g; k <= c; k += 8) mx = max(mx, (uint32_t)__double2hiint(RT[(int64_t)k * npad + c]) & 0x7FFFFFFFu);
   __syncthreads();
   red[g][lane] = (int)mx;
@@ -592,6 +694,8 @@ struct RpPrep {
   long long Ri[kRN][kRN + 1];   // a block of R in fixed point, row k against er[k]
   long long Xi[kRN][kRN + 1];   // X in fixed point, column c against Ex[c]
   int er[kRN], Ex[kRN], cE[kRN];
+  int fN[kRpOwnScale];
+  double rinv[kRN];             // 1 / diagonal of the scaled panel
   int red[8][kRN];
 };
 
@@ -647,6 +751,16 @@ __device__ __forceinline__ __int128 rp_dot(const RpPrep& P, int k, int c, int j0
   return acc;
 }
 
+// f_c of every column and e_k of the rows below `rows` without launches of their own: every block of the preparation
+// finds them (they agree).
+__device__ __forceinline__ void rp_own_scales(RpPrep& P, int n, int npad, const double* __restrict__ RT, const RpInts& I,
+                                              int rows) {
+  for (int blk = 0; blk < (n + kRN - 1) / kRN; ++blk) rp_col_scale_block(n, npad, RT, P.fN, blk, P.red);
+  __syncthreads();
+  for (int c = threadIdx.x; c < n; c += 256) I.fN[c] = P.fN[c];
+  for (int blk = 0; blk < (rows + 7) / 8; ++blk) rp_row_scale_block(n, npad, RT, P.fN, I.eR, blk);
+}
+
 // Multiplier of a panel that keeps its substitution: the digits of -D^{-1} R_{<t,t}
 // against the columns' largest entries (no X_t, no F: each column has its own reference).
 __device__ __forceinline__ void rp_prep_kept(RpPrep& P, int n, int npad, const double* __restrict__ RT, const RpInts& I,
@@ -689,21 +803,19 @@ __device__ __forceinline__ void rp_prep_kept(RpPrep& P, int n, int npad, const d
 __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, const double* __restrict__ RT,
                                                 const double* __restrict__ rinv, const RpInts& I,
                                                 unsigned char* __restrict__ Md, uint32_t* __restrict__ colHiOut,
-                                                int nhi, int t) {
-  int *eR = I.eR, *fN = I.fN;
+                                                int nhi, int t, int check) {
+  int* eR = I.eR;
   const int tid = threadIdx.x, c = tid & 31, g = tid >> 5;   // this thread: column c, rows 4 g .. 4 g + 3
   const int c0 = kRN * t, w = min(kRN, n - c0);
   if (colHiOut && t == 0)     // the product folds the column maxima of W into these
     for (int i = tid; i < nhi; i += blockDim.x) colHiOut[i] = 0u;
-  if (n <= kRpOwnScale) {     // no launches for f_c and e_k: every panel finds them (they agree)
-    for (int blk = 0; blk < (n + kRN - 1) / kRN; ++blk) rp_col_scale_block(n, npad, RT, fN, blk, P.red);
-    __syncthreads();
-    for (int blk = 0; blk < (min(n, c0 + kRN) + 7) / 8; ++blk) rp_row_scale_block(n, npad, RT, fN, eR, blk);
-  }
+  if (n <= kRpOwnScale) rp_own_scales(P, n, npad, RT, I, min(n, c0 + kRN));
   __syncthreads();
+  const int* fN = n <= kRpOwnScale ? P.fN : I.fN;
   const int f = c < w ? fN[c0 + c] : 0;
   // X = (R F^{-1})_tt^{-1} by FP64 back substitution, column c in the lanes, rows over the warps
   const double scale = rp_pow2(f);
+  if (g == 0) P.rinv[c] = c < w ? rinv[c0 + c] * rp_pow2(-f) : 1.0;
   double b[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
@@ -714,7 +826,7 @@ __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, cons
   __syncthreads();
 #pragma unroll
   for (int k = kRN - 1; k >= 0; --k) {
-    if ((k >> 2) == g) P.X[k][c] = k >= w ? b[k & 3] : c < k ? 0.0 : b[k & 3] * (rinv[c0 + k] * rp_pow2(-fN[c0 + k]));
+    if ((k >> 2) == g) P.X[k][c] = k >= w ? b[k & 3] : c < k ? 0.0 : b[k & 3] * P.rinv[k];
     if (k >= w) continue;   // identity beyond column n
     __syncthreads();
     const double x = P.X[k][c];
@@ -823,7 +935,7 @@ __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, cons
   }
   const bool keep = __syncthreads_or(bad || nf) != 0;
   if (tid == 0) I.flags[t] = keep ? 1 : 0;
-  if (keep) rp_prep_kept(P, n, npad, RT, I, Md + rp_digit_size(n), t);
+  if (keep && !check) rp_prep_kept(P, n, npad, RT, I, Md + rp_digit_size(n), t);
   // digits (of a kept panel only the block of X is copied, and multiplied by zeros)
   if (g == 0 && c < w) I.colE[c0 + c] = P.cE[c];
   const int Ex = P.Ex[c], cE = P.cE[c];
@@ -874,10 +986,18 @@ __device__ __forceinline__ void rp_prep_r_panel(RpPrep& P, int n, int npad, cons
 __global__ void __launch_bounds__(256) k_rp_prep_r(int n, int npad, const double* __restrict__ RT,
                                                    const double* __restrict__ rinv, RpInts I,
                                                    unsigned char* __restrict__ Md, uint32_t* __restrict__ colHiOut,
-                                                   int nhi, const Ctl* ctl, int level) {
+                                                   int nhi, int check, const Ctl* ctl, int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
   extern __shared__ unsigned char prep_raw[];
-  rp_prep_r_panel(*reinterpret_cast<RpPrep*>(prep_raw), n, npad, RT, rinv, I, Md, colHiOut, nhi, blockIdx.x);
+  RpPrep& P = *reinterpret_cast<RpPrep*>(prep_raw);
+  const int t = (int)blockIdx.x % (npad / kRN);
+  if ((int)blockIdx.x == t) {
+    rp_prep_r_panel(P, n, npad, RT, rinv, I, Md, colHiOut, nhi, t, check);
+  } else {   // checked solve: a second block per panel prepares its substitution
+    if (n <= kRpOwnScale) rp_own_scales(P, n, npad, RT, I, kRN * t);
+    __syncthreads();
+    rp_prep_kept(P, n, npad, RT, I, Md + rp_digit_size(n), t);
+  }
 }
 
 int rp_sms() {
@@ -938,7 +1058,7 @@ __global__ void __launch_bounds__(kRThreads, 2) kg_rowprod(Group g, int level) {
       rp_begin<kTrsm>(a, S);
       cur = w.x;
     }
-    if (!rp_block<kTrsm, true>(a, S, (int64_t)w.y * kM, 0)) {
+    if (!rp_block<kTrsm, true, false>(a, S, (int64_t)w.y * kM, 0)) {
       abort = true;
       actl = P.ctl;
       break;
@@ -987,15 +1107,15 @@ __global__ void __launch_bounds__(256) kg_rp_prep_r(Group g, int level) {
     if (!rp_live(P, level)) continue;
     __syncthreads();
     rp_prep_r_panel(*reinterpret_cast<RpPrep*>(prep_raw), P.n, P.npad, P.rst, P.rinv, RpInts(P.oz_cole, P.n), P.oz_rd,
-                    P.oz_colhi, rp_nhi(P.n), w.y);
+                    P.oz_colhi, rp_nhi(P.n), w.y, 0);
   }
 }
 
-template <bool kTrsm>
+template <bool kTrsm, bool kCheck>
 void rp_launch(const RpArgs& a, Ctl* ctl, int level, cudaStream_t st) {
   const int64_t nblocks = (a.m + kM - 1) / kM, slots = 2 * (int64_t)rp_sms();
   const unsigned grid = (unsigned)(nblocks < slots ? nblocks : slots);
-  auto kernel = a.n > kRN * kGroupChunks ? k_rowprod<kTrsm, true> : k_rowprod<kTrsm, false>;
+  auto kernel = a.n > kRN * kGroupChunks ? k_rowprod<kTrsm, true, kCheck> : k_rowprod<kTrsm, false, kCheck>;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRSmem);
   launch_dep(kernel, grid, kRThreads, kRSmem, st, a, ctl, level);
 }
@@ -1017,7 +1137,7 @@ int rp_panels(int n) { return rp_n32(n) / kRN; }
 
 void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double* RT, const double* rinv, int* ints,
                     unsigned char* Rd, double* W, int64_t ldw, Ctl* ctl, int level, cudaStream_t st,
-                    uint32_t* colHiOut) {
+                    uint32_t* colHiOut, bool check) {
   const int n32 = rp_n32(n);
   const int nhi = (int)(syrk_oz_colhi_bytes(n) / sizeof(uint32_t));
   const RpInts I(ints, n);
@@ -1026,8 +1146,10 @@ void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double
     launch_dep(k_rp_row_scale, (n + 7) / 8, 256, 0, st, n, n32, RT, I.fN, I.eR, ctl, level);
   }
   cudaFuncSetAttribute(k_rp_prep_r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RpPrep));
-  launch_dep(k_rp_prep_r, n32 / kRN, 256, sizeof(RpPrep), st, n, n32, RT, rinv, I, Rd, colHiOut, nhi, ctl, level);
-  rp_launch<true>(rp_trsm_args(m, n, A, lda, W, ldw, ints, Rd, RT, rinv, colHiOut), ctl, level, st);
+  launch_dep(k_rp_prep_r, (check ? 2 : 1) * n32 / kRN, 256, sizeof(RpPrep), st, n, n32, RT, rinv, I, Rd, colHiOut, nhi, check ? 1 : 0, ctl, level);
+  const RpArgs a = rp_trsm_args(m, n, A, lda, W, ldw, ints, Rd, RT, rinv, colHiOut);
+  if (check) rp_launch<true, true>(a, ctl, level, st);
+  else rp_launch<true, false>(a, ctl, level, st);
 }
 
 void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* XT, int* colE, unsigned char* Xs,
@@ -1035,7 +1157,7 @@ void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* 
   const int n32 = rp_n32(n);
   const int nhi = (int)(syrk_oz_colhi_bytes(n) / sizeof(uint32_t));
   launch_dep(k_rp_prep_x, n32, 128, 0, st, n, n32, XT, colE, Xs, colHiOut, nhi, ctl, level);
-  rp_launch<false>(rp_fin_args(m, n, Q, ldq, colE, Xs, colHiOut), ctl, level, st);
+  rp_launch<false, false>(rp_fin_args(m, n, Q, ldq, colE, Xs, colHiOut), ctl, level, st);
 }
 
 void prepare_g_rowprod() {

@@ -141,3 +141,26 @@ def test_batched_plan_and_cholqr2_of_columns_of_different_size(env):
         assert M.last_status()["status"] == "OK"
         e = np.frexp(d)[1]
         _check_factors(np.ldexp(A, -e), Q.cpu().numpy(), np.ldexp(R.cpu().numpy(), -e))
+
+
+# R that is no factor of A: its columns say nothing about A's.  Columns of A graded over 1e25 against the identity, a
+# triangle of its own, and a first block so ill-conditioned that W's columns differ by 1e12.
+@pytest.mark.parametrize("kind", ["identity", "triangle", "ill_block"])
+@pytest.mark.parametrize("m,n", [(300, 2), (130, 32), (257, 70), (400, 160)])
+def test_trsm_with_an_unrelated_triangle(env, m, n, kind):
+    torch, M = env
+    rng = np.random.default_rng(m + n)
+    A = rng.standard_normal((m, n)) * _scales(n, "random" if kind != "ill_block" else "ascending", 1e25, rng)
+    R = np.eye(n) if kind == "identity" else np.linalg.qr(rng.standard_normal((2 * n, n)))[1]
+    if kind == "ill_block":
+        A = rng.standard_normal((m, n))
+        k = min(32, n // 2)
+        R[:k, k:] = 0.0
+        R[:k, :k] *= (1e-12 ** (np.arange(k) / max(k - 1, 1)))[:, None]
+    A[m // 2:m // 2 + 3] *= 1e-30                     # rows of another size keep their own references
+    W = M.trsm(M.to_colmajor(A), M.to_colmajor(R)).cpu().numpy()
+    if kind == "identity":
+        np.testing.assert_array_equal(W, A)
+    d = 2.0 ** -np.frexp(np.abs(A).max(0))[1]         # exact: keeps the reference's products in range
+    res, scale = _column_residuals(A * d, W, R * d)
+    assert (res <= 4 * n * U * scale).all(), float((res / scale).max())
