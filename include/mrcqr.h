@@ -309,7 +309,7 @@ int mrcqr_cholqr_precond(int64_t m, int64_t n, const double* A, int64_t lda, con
  * Columns enter scaled by the powers of two of R's column maxima; a panel with a
  * column of A far from them within 128 rows is solved by substitution too, so the
  * backward error of every column is that of a triangular solve.  A
- * non-finite entry of A makes its row of W NaN from the entry's panel on.
+ * non-finite entry of A makes its row of W non-finite from its column on.
  * fp64_products = 1: FP64 substitution throughout.
  * 1 <= n <= 512, 1 <= m < 2^31.  Allocates its workspace with cudaMallocAsync
  * on `stream`. */

@@ -220,6 +220,24 @@ __device__ __noinline__ void rp_substitute(const RpArgs& a, double* sb, int c0, 
   }
 }
 
+// A row with a non-finite entry of A in the panel at c0: columns cb .. cb + 15 of the panel by FP64 substitution along
+// the row, into sb[c kM], so that the columns before the entry are those of the finite row.
+__device__ __noinline__ void rp_solve_row(const RpArgs& a, double* sb, int64_t row, int c0, int cb) {
+  const int npad = rp_n32(a.n);
+  double x[kRN];
+  for (int c = 0; c < cb + 16; ++c) {
+    x[c] = 0.0;
+    if (c0 + c < a.n) {
+      const double* r = a.RT + c0 + c;
+      double v = a.A[row + (int64_t)(c0 + c) * a.lda];
+      for (int k = 0; k < c0; ++k) v = fma(-a.W[row + (int64_t)k * a.ldw], r[(int64_t)k * npad], v);
+      for (int k = 0; k < c; ++k) v = fma(-x[k], r[(int64_t)(c0 + k) * npad], v);
+      x[c] = v * a.rinv[c0 + c];
+    }
+    if (c >= cb) sb[c * kM] = x[c];
+  }
+}
+
 // Checked solve: the exponent that every column of A F^{-1} in the panel should reach in the row block.
 __device__ __forceinline__ int rp_threshold(const RpCta& S) {
   return max(max(max(S.rho[0], S.rho[1]), max(S.rho[2], S.rho[3])) - kBalance, -4000);
@@ -476,8 +494,13 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
 #pragma unroll
       for (int c = 0; c < 16; ++c) out[c] = nan64();
     }
+    double* sb = reinterpret_cast<double*>(S.as);     // the chunk's panels are free
+    if (kTrsm && !keep && rlive && max(S.red[0][rr], S.red[1][rr]) == kNonfinite) {   // in both threads of the row
+      rp_solve_row(a, sb + rr, r0 + rr, c0, 16 * g);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) out[c] = sb[(16 * g + c) * kM + rr];
+    }
     if (keep) {
-      double* sb = reinterpret_cast<double*>(S.as);   // the chunk's panels are free
 #pragma unroll
       for (int c = 0; c < 16; ++c)
         if (c0 + 16 * g + c < n)

@@ -164,3 +164,23 @@ def test_trsm_with_an_unrelated_triangle(env, m, n, kind):
     d = 2.0 ** -np.frexp(np.abs(A).max(0))[1]         # exact: keeps the reference's products in range
     res, scale = _column_residuals(A * d, W, R * d)
     assert (res <= 4 * n * U * scale).all(), float((res / scale).max())
+
+
+# A non-finite entry in either half of a panel, in the first panel or with W to its left: the columns before it are
+# those of the row without it.
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+@pytest.mark.parametrize("col", [0, 5, 17, 40, 56, 69])
+def test_nonfinite_entry_reaches_only_the_columns_after_it(env, col, value):
+    torch, M = env
+    rng = np.random.default_rng(col)
+    m, n, row = 300, 70, 133
+    R = _triangle(n, rng)
+    A = rng.standard_normal((m, n))
+    clean = M.trsm(M.to_colmajor(A), M.to_colmajor(R)).cpu().numpy()
+    A[row, col] = value
+    W = M.trsm(M.to_colmajor(A), M.to_colmajor(R)).cpu().numpy()
+    np.testing.assert_array_equal(np.delete(W, row, 0), np.delete(clean, row, 0))
+    assert not np.isfinite(W[row, col:]).any()
+    # two solutions with backward errors gamma_n |W| |R|: apart by at most that through |R^-1|
+    bound = 8 * n * U * (np.abs(clean[row]) @ np.abs(R)) @ np.abs(np.linalg.inv(R))
+    assert (np.abs(W[row, :col] - clean[row, :col]) <= bound[:col]).all()
