@@ -75,7 +75,7 @@ Plan make_plan(int64_t m, int n, int s, int tf = T_DCT, bool planes = false) {
   // the FP64 sketch from digit planes in row chunks: at most the chunks of a Q buffer with ldq = m, or
   // one chunk in the workspace's own planes
   const size_t q_bytes = sizeof(double) * (size_t)m * n;
-  const int64_t mr = (m + 31) / 32 * 32;
+  const int64_t mr = (m + 4095) / 4096 * 4096;   // the four-step form's words of all rows in one range
   if (planes) p.planes_bytes = 16ull * (size_t)n * (size_t)mr;
   p.ozpart_bytes = std::max({syrk_oz_part_bytes(p.oz), sketch_oz_part_bytes(p.sk), sketch_ozp_part_bytes(m, n, s, q_bytes),
                              planes ? sketch_ozp_part_bytes(m, n, s, p.planes_bytes) : size_t(0)});

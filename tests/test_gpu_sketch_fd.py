@@ -108,3 +108,25 @@ def test_sizes_the_four_step_form_does_not_take(env):
         Y = M.sketch(M.to_colmajor(A[:m]), s, "fp64", seed=2, variant=6).cpu().numpy()
         assert M.last_sketch_variant() == 5
         _check(Y, A[:m], s, 2)
+
+
+def _sketch_time(torch, M, m, n, s):
+    A = torch.randn((n, m), dtype=torch.float64, device="cuda").t()
+    M.sketch(A, s, "fp64", seed=1)
+    assert M.last_sketch_variant() == 6
+    t = []
+    for _ in range(7):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        M.sketch(A, s, "fp64", seed=1)
+        b.record()
+        b.synchronize()
+        t.append(a.elapsed_time(b))
+    return sorted(t)[len(t) // 2]
+
+
+# Heights off the multiples of 4096 cost what their rows cost: 5% fewer rows than 2^20 take at most a quarter more
+# (ragged last blocks, one more range), not twice the time.
+def test_time_follows_the_rows(env):
+    torch, M = env
+    assert _sketch_time(torch, M, 1000000, 128, 256) <= 1.25 * _sketch_time(torch, M, 1 << 20, 128, 256)
