@@ -281,9 +281,9 @@ __global__ void __launch_bounds__(256) k_sketch_simt(const double* __restrict__ 
                           tf);
 }
 
-// At least this many rows per chunk: a chunk's CTA first builds its transform tables, and every chunk is a term of
-// k_sketch_reduce.
-constexpr int kSkMinRows = 128;
+// At least this many rows per chunk, the granularity of a chunk: short matrices keep FP32 sums of 64 rows, added in
+// FP64 by k_sketch_reduce.  (128 halve the terms of that sum, for twice the rows per FP32 sum and a few us.)
+constexpr int kSkMinRows = 64;
 
 int sketch_chunks(int64_t m, int n, int s) {
   const int tiles = ((s + kSkST - 1) / kSkST) * ((n + kSkNT - 1) / kSkNT);

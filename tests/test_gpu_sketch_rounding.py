@@ -78,3 +78,20 @@ def test_dense_rows_over_chunks(env, m, n, s, ld):
     ref = coef * (F @ (d[rows, None] * A[rows]))
     # two TF32 parts (2^-21), FP32 twiddles of a few ulp, FP32 sums
     assert (np.abs(Y - ref) <= coef * 2.0 ** -18 * np.abs(A).sum(axis=0)[None, :]).all()
+
+
+# FP32 sums run over at most 64 rows of a short matrix: 64 odd 18-bit integers add up exactly in FP32 (24 bits), 128
+# of them to an odd sum above 2^24 do not.  Row k = 0 of the transform is all ones; variant 1: SIMT, 2: tensor cores.
+@pytest.mark.parametrize("variant", [1, 2])
+@pytest.mark.parametrize("m,s", [(384, 384), (1000, 600), (4096, 300)])   # m / 64 chunks at most 608 / (s / 64)
+def test_short_matrices_keep_fp32_sums_of_64_rows(env, variant, m, s):
+    torch, M = env
+    n = 5
+    seed = next(k for k in range(200) if 0 in O.sample_rows(m, s, k))
+    d, idx = O.rademacher(m, seed), O.sample_rows(m, s, seed)
+    X = (np.random.default_rng(m).integers(2 ** 16, 2 ** 17, (m, n)) * 2 + 1).astype(np.float64)
+    X[::128] -= 1.0                                   # an even term in every 128 rows: their sum is odd
+    Y = M.sketch(M.to_colmajor(d[:, None] * X), s, "fp32", seed=seed, variant=variant).cpu().numpy()
+    assert M.last_sketch_variant() == variant
+    want = np.sqrt(2.0 / s) * np.sqrt(0.5) * X.sum(axis=0)
+    assert (np.abs(Y[int(np.flatnonzero(idx == 0)[0])] - want) <= 2.0 ** -50 * want).all()
