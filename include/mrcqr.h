@@ -349,6 +349,11 @@ int mrcqr_finalize_q(int64_t m, int64_t n, double* Q, int64_t ldq, const double*
  * context stays usable.  INVALID on bad arguments. */
 int mrcqr_debug_wait_timeout(uint32_t polls, int32_t* status, mrcqr_stream_t stream);
 
+/* Test hook for the Cholesky pivot: p[i] = sqrt(d[i]) and y[i] = 1 / p[i]
+ * (-1 and -1 where d[i] is not positive and finite), 1 <= count <= 2^30, all
+ * DEVICE doubles. */
+int mrcqr_debug_pivot_sqrt(int64_t count, const double* d, double* p, double* y, mrcqr_stream_t stream);
+
 /* Allocation-free variant of mrcqr_sketch_qr.  The paper has no counterpart:
  * this entry point exists for callers that cannot allocate device memory
  * when they need R_s -- code running under another framework's memory

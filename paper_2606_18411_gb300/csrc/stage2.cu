@@ -9,6 +9,7 @@
 // plain SIMT kernel that keeps the DFMA pipe fed (independent accumulators,
 // broadcast operand loads), and memory traffic is secondary.
 #include "kernels.h"
+#include "pivot.cuh"
 
 namespace mrcqr {
 
@@ -263,34 +264,6 @@ __device__ __forceinline__ bool chol_block(int n, double* __restrict__ G) {
   }
   __syncthreads();
   return true;
-}
-
-// p = sqrt(d) and y = 1 / sqrt(d) of a pivot, y = -1 if d is not positive and
-// finite: an FP32 reciprocal square root of the significand, one cubically
-// convergent step (y0 (1 + r / 2 + 3 r^2 / 8), r = 1 - d y0^2 ~ 2^-21), then a
-// Heron step for p and a Newton step for y (both to about half an ulp).  A
-// dozen FP64 operations in place of the square root and the division, whose
-// sequences were most of an elimination step here (1/64-rate pipe).
-__device__ __forceinline__ void pivot_sqrt(double d, double& p, double& y) {
-  p = y = -1.0;
-  const int h = __double2hiint(d);
-  if (h < 0x00100000 || h >= 0x7FF00000) {          // not a positive normal number
-    if (d > 0.0 && h < 0x00100000) {                // subnormal
-      p = sqrt(d);
-      y = 1.0 / p;
-    }
-    return;
-  }
-  const int e2 = ((h >> 20) - 1023) & ~1;           // d = dm 2^e2, dm in [1, 4)
-  const double dm = __hiloint2double(h - (e2 << 20), __double2loint(d));
-  const double y0 = (double)rsqrtf((float)dm);
-  const double r = fma(-dm * y0, y0, 1.0);
-  double yy = fma(y0 * r, fma(0.375, r, 0.5), y0);
-  double pp = dm * yy;
-  pp = fma(fma(-pp, pp, dm) * 0.5, yy, pp);
-  yy = fma(yy, fma(-pp, yy, 1.0), yy);
-  p = __hiloint2double(__double2hiint(pp) + ((e2 / 2) << 20), __double2loint(pp));
-  y = __hiloint2double(__double2hiint(yy) - ((e2 / 2) << 20), __double2loint(yy));
 }
 
 // Cholesky of the w x w matrix in shared memory (S[j ld + i] = element (i, j),

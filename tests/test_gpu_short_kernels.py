@@ -65,3 +65,41 @@ def test_sketch_qr_sizes(env, prec, n, s):
     g = 4 * s * np.sqrt(n) * (2.0 ** -24 if prec == "fp32" else U)
     c = np.linalg.norm(Y, axis=0)
     assert (np.abs(R.T @ R - Y.T @ Y) <= 2 * g * np.outer(c, c)).all()
+
+
+def _hard_square_roots():
+    """d whose square roots lie closest to the middle of two doubles: p = N / 2^53, N odd, N^2 = k mod 2^e for small k."""
+    out = []
+    for e in (54, 55):                                # d in [1, 2) and in [2, 4)
+        M = 1 << e
+        for k in range(-2047, 2048, 8):               # k = 1 mod 8 has four roots
+            x = 1
+            for b in range(3, e):
+                if ((x * x - k) >> b) & 1:
+                    x += 1 << (b - 1)
+            for r in (x, -x, x + M // 2, M // 2 - x):
+                for N in {r % M, r % M + M}:
+                    D = (N * N - k) >> e
+                    if 1 << 53 <= N < 1 << 54 and 1 << 52 <= D < 1 << 53:
+                        out.append(np.ldexp(float(D), e - 106))
+    return out
+
+
+def test_pivot_is_correctly_rounded(env):
+    torch, M = env
+    from paper_2606_18411_gb300 import _lib
+    rng = np.random.default_rng(1)
+    one = 1.0 + np.arange(2000) * 2.0 ** -52
+    ones = 2.0 - (1 + np.arange(2000)) * 2.0 ** -52   # the last significands below 2, all ones first
+    d = np.concatenate([np.ldexp(1.0 + rng.random(400000), rng.integers(-1022, 1023, 400000)), _hard_square_roots(),
+                        one, one ** 2, ones, 2 * ones, ones ** 2, np.nextafter(ones ** 2, 4.0),
+                        [2.0 ** -1022, np.finfo(np.float64).max, 5e-324, 2.0 ** -1023, 1e-310]])
+    bad = np.array([0.0, -0.0, -1.0, -5e-324, np.inf, -np.inf, np.nan])
+    dev = torch.from_numpy(np.concatenate([d, bad])).cuda()
+    p, y = torch.empty_like(dev), torch.empty_like(dev)
+    assert _lib.load().mrcqr_debug_pivot_sqrt(dev.numel(), dev.data_ptr(), p.data_ptr(), y.data_ptr(), None) == 0
+    torch.cuda.synchronize()
+    p, y = p.cpu().numpy(), y.cpu().numpy()
+    np.testing.assert_array_equal(p[:len(d)], np.sqrt(d))          # IEEE square root and division
+    np.testing.assert_array_equal(y[:len(d)], 1.0 / np.sqrt(d))
+    assert (p[len(d):] == -1.0).all() and (y[len(d):] == -1.0).all()
