@@ -68,7 +68,7 @@ Plan make_plan(int64_t m, int n, int s, int tf = T_DCT, bool planes = false) {
   p.off_e = take(sizeof(double) * (size_t)n * n);
   p.off_feat = take(sizeof(float) * kNumFeatures);
   p.off_oze = take(rp_fin_ints_bytes(n));
-  p.off_ozx = take(rp_digit_bytes(n));
+  p.off_ozx = take(rp_fin_digit_bytes(n));
   p.oz = syrk_oz_plan(m, n);
   p.sk = sketch_oz_plan(m, n, s);
   p.off_colhi = take(syrk_oz_colhi_bytes(n));

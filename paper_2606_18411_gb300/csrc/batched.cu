@@ -48,7 +48,7 @@ enum Kind {
   K_FORK, K_JOIN, K_OZ_SKETCH, K_OZ_STAGE2A, K_OZ_STAGE2B,
   // grouped emulated-FP64 kernels (param = 1: the check's Gram)
   KG_OZ_COLHI, KG_OZ_SKETCH, KG_OZ_SKREDUCE, KG_OZ_COLSCALE, KG_OZ_ROWSCALE, KG_OZ_PREPR, KG_OZ_TRSM, KG_OZ_SYRK, KG_OZ_SYREDUCE,
-  KG_OZ_PREPX, KG_OZ_FINALIZE,
+  KG_OZ_PREPX, KG_OZ_FINALIZE, KG_FW_PREP, KG_FW_PRODUCT,
   // grouped tensor-core sketch, param = 2 precision + (MT - 1)
   KG_TC_SKETCH
 };
@@ -229,7 +229,7 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
     g[2] = take(rp_trsm_ints_bytes(P.n));
     g[3] = take(rp_trsm_digit_bytes(P.n));
     g[4] = take(rp_fin_ints_bytes(P.n));
-    g[5] = take(rp_digit_bytes(P.n));
+    g[5] = take(rp_fin_digit_bytes(P.n));
   }
   const size_t probs_off = take(sizeof(Prob) * (size_t)count);
   const size_t map_bytes = sketch_tc_map_bytes();
@@ -329,7 +329,7 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
     add(K_SQR, L, 0, q32);
     add(K_SQR, L, 1, q64);
     // emulated-FP64 stage 2 work lists (grouped form)
-    std::vector<int4> z_cs, z_rs, z_pr, z_tr, z_sy, z_gr, z_px, z_fi;
+    std::vector<int4> z_cs, z_rs, z_pr, z_tr, z_sy, z_gr, z_px, z_fi, z_pw, z_fw;
     if (pl.emu && pl.oz_grouped)
       for (int i : live) {
         const Prob& P = pl.probs[i];
@@ -342,8 +342,10 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
         for (int b = 0; b < blocks(P.m, 128); ++b) z_tr.push_back(make_int4(i, b, 0, 0));
         for (int t = 0; t < z.sp.ntiles * z.sp.slabs; ++t) z_sy.push_back(make_int4(i, t, 0, 0));
         for (int b = 0; b < blocks((int64_t)P.n * P.n, 256); ++b) z_gr.push_back(make_int4(i, b, 0, 0));
-        for (int j = 0; j < rp_cols(P.n); ++j) z_px.push_back(make_int4(i, j, 0, 0));
-        for (int b = 0; b < blocks(P.m, 128); ++b) z_fi.push_back(make_int4(i, b, 0, 0));
+        const bool wide = rp_wide(P.n);
+        for (int j = 0; j < (wide ? blocks(P.n, 64) * 64 : rp_cols(P.n)); ++j)
+          (wide ? z_pw : z_px).push_back(make_int4(i, j, 0, 0));
+        for (int b = 0; b < blocks(P.m, 128); ++b) (wide ? z_fw : z_fi).push_back(make_int4(i, b, 0, 0));
       }
     if (pl.emu && pl.oz_grouped) {   // W = A R_s^{-1} (folding W's column maxima), G = W^T W
       add(KG_OZ_COLSCALE, L, 0, z_cs);
@@ -375,6 +377,8 @@ void build(mrcqr_batched_plan_s& pl, int count, const int64_t* m, const int64_t*
     if (pl.emu && pl.oz_grouped) {   // Q = W R_c^{-1} (folding Q's column maxima), E = Q^T Q
       add(KG_OZ_PREPX, L, 0, z_px);
       add(KG_OZ_FINALIZE, L, 0, z_fi);
+      add(KG_FW_PREP, L, 0, z_pw);
+      add(KG_FW_PRODUCT, L, 0, z_fw);
       if (check) {
         add(KG_OZ_SYRK, L, 1, z_sy);
         add(KG_OZ_SYREDUCE, L, 1, z_gr);
@@ -525,6 +529,8 @@ void enqueue(mrcqr_batched_plan_s& pl, cudaStream_t st) {
       case KG_OZ_SYREDUCE: launch_g_oz_syrk_reduce(g, L.param == 1, L.level, st); break;
       case KG_OZ_PREPX: launch_g_oz_prep_x(g, L.level, st); break;
       case KG_OZ_FINALIZE: launch_g_oz_finalize(g, L.level, st); break;
+      case KG_FW_PREP: launch_g_fw_prep(g, L.level, st); break;
+      case KG_FW_PRODUCT: launch_g_fw_product(g, L.level, st); break;
     }
   }
   pl.kernels = (int)(mrcqr_launch_count() - c0);

@@ -117,8 +117,11 @@ void launch_g_publish(const Group& g, cudaStream_t st);
 //   trsm_oz      items {i, 128-row block}
 //   syrk_oz      items {i, item of the problem's SyrkOzPlan}     syrk_oz_reduce {i, 256-entry block}
 //   prep_x       items {i, column < n32}                         finalize_oz {i, 128-row block}
+//   fw_prep      items {i, column < n64}                         fw_product {i, 128-row block} (rp_wide problems)
 void prepare_g_rowprod();      // kernel attributes of rowprod.cu; call outside stream capture
 void prepare_g_oz_kernels();   // kernel attributes; call outside stream capture
+void launch_g_fw_prep(const Group& g, int level, cudaStream_t st);
+void launch_g_fw_product(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_colhi(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_sketch(const Group& g, int level, cudaStream_t st);
 void launch_g_oz_sketch_reduce(const Group& g, int level, cudaStream_t st);
@@ -232,9 +235,12 @@ void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, con
 // --- W = A R^{-1} and Q = W X in emulated FP64 (rowprod.cu) -----------------------
 // Workspace: digit panels of the multiplier (two sets for the TRSM), the TRSM's integers (column exponents,
 // row and column scalings, panel flags), the finalize's column exponents; columns and 32-column panels of n.
+// Q = W X: whether 64-column tiles (ozaki.cu, both measured there) beat the 32-column ones: from 161 columns where
+// they pad no further, from 289 always.
+inline bool rp_wide(int n) { return n > 160 && (n > 288 || (n + 31) / 32 % 2 == 0); }
 constexpr int kRpOwnScale = 128;   // up to this n the TRSM's preparation finds the scalings itself (no launches)
 // check: R need not be a factor of A (its column sizes may say nothing about A's or W's); the row blocks look.
-size_t rp_digit_bytes(int n);
+size_t rp_fin_digit_bytes(int n);
 size_t rp_trsm_digit_bytes(int n);
 size_t rp_trsm_ints_bytes(int n);
 size_t rp_fin_ints_bytes(int n);
@@ -243,6 +249,9 @@ int rp_panels(int n);
 void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double* RT, const double* rinv, int* ints,
                     unsigned char* Rd, double* W, int64_t ldw, Ctl* ctl, int level, cudaStream_t st,
                     uint32_t* colHiOut = nullptr, bool check = false);
+size_t fw_digit_bytes(int n);   // ozaki.cu
+void launch_finalize_wide(int64_t m, int n, double* Q, int64_t ldq, const double* XT, int* colE, unsigned char* Xs,
+                          Ctl* ctl, int level, cudaStream_t st, uint32_t* colHiOut);
 void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* XT, int* colE, unsigned char* Xs,
                         Ctl* ctl, int level, cudaStream_t st, uint32_t* colHiOut = nullptr);
 

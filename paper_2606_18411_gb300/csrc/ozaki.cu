@@ -1,16 +1,19 @@
 // FP64 products of the method on FP16 tensor cores with exact integer
 // slicing (ozaki.cuh): the Gram matrix and the check Q^T Q (Algorithm 1
-// step 1, Sec. II-C) and the FP64 sketch (Algorithm 2 steps 2-4 at p = FP64).
+// step 1, Sec. II-C), the FP64 sketch (Algorithm 2 steps 2-4 at p = FP64) and, for
+// wide W, Q = W R_c^{-1}.
 // Each result entry is the once-rounded value of a 63-bit fixed-point
-// evaluation of its sum.  (The row-block products W = A R_s^{-1} and
-// Q = W R_c^{-1} are in rowprod.cu.)
+// evaluation of its sum.  (The row-block products W = A R_s^{-1} and Q = W R_c^{-1}
+// of narrow W are in rowprod.cu.)
 //
-// All three run the same two-stage pipeline per CTA (one CTA per SM, 512
+// All of them run the same two-stage pipeline per CTA (one CTA per SM, 512
 // threads, all 512 TMEM columns = 8 level accumulators of 128 x 64): the
 // threads write the digit panels of K chunk c + 1 (32 deep, K-major
 // SWIZZLE_64B) into one shared-memory stage while the tensor cores run the
 // 36 digit-pair MMAs of chunk c from the other; every 4 chunks (K = 128, the
 // exactness limit) the level sums are read out of TMEM into 64-bit integers.
+#include <algorithm>
+
 #include "kernels.h"
 #include "ozaki.cuh"
 #include "tc.cuh"
@@ -19,6 +22,196 @@
 namespace mrcqr {
 
 namespace {
+
+// ---------------------------------------------------------------------------
+// Q = W X in place (X = R_c^{-1} upper, Algorithm 1 step 3) in 128 x 64 tiles by
+// one CTA per SM, for wide W (rp_wide; rowprod.cu has 128 x 32 tiles by two
+// CTAs).  A tile of twice the width slices every chunk of W half as often and issues
+// 10% fewer MMA cycles, but one CTA holds all of TMEM, so nothing covers its row
+// blocks' other phases: it pays once a block is many chunks long.  Measured at m = 2^20
+// (us, 32 / 64 columns): n = 128 1975 / 2135, 192 3786 / 3645, 256 5810 / 5290, 288
+// 7392 / 7557, 320 8786 / 7738, 384 11656 / 9945, 512 19111 / 15801; m = 2^18: n = 96 552 / 712,
+// 160 1033 / 1167, 352 3064 / 2988.  Integer work around the products bounds both.
+// Multiplier digits: block (t, kc), kc <= 2 t + 1, of columns [64 t, 64 t + 64) and
+// rows [32 kc, 32 kc + 32) of X as eight K-major SWIZZLE_64B panels.
+__host__ __device__ __forceinline__ size_t fw_block_offset(int t, int kc) {
+  return ((size_t)t * (t + 1) + kc) * (oz::kSlices * kBPanel);
+}
+
+__device__ __forceinline__ void fw_prep_col(int n, int npad, const double* __restrict__ XT, int* __restrict__ colE,
+                                            unsigned char* __restrict__ Xs, uint32_t* __restrict__ colHiOut, int nhi,
+                                            int j, uint32_t* red) {
+  if (colHiOut && j == 0)     // the product folds the column maxima of Q into these
+    for (int i = threadIdx.x; i < nhi; i += blockDim.x) colHiOut[i] = 0u;
+  __syncthreads();
+  uint32_t mx = 0u;
+  for (int k = threadIdx.x; k < n; k += blockDim.x)
+    if (j < n) mx = max(mx, (uint32_t)__double2hiint(XT[(int64_t)k * npad + j]) & 0x7FFFFFFFu);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  uint32_t all = 0u;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) all = max(all, red[w]);
+  const int E = (int)oz::exp_field(all), t = j / kN;
+  if (threadIdx.x == 0 && j < n) colE[j] = E;
+  for (int k = threadIdx.x; k < 2 * kK * (t + 1); k += blockDim.x) {
+    int dg[oz::kSlices];
+    const double v = (k < n && j < n) ? XT[(int64_t)k * npad + j] : 0.0;
+    oz::digits8((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v), E, dg);
+    unsigned char* panel = Xs + fw_block_offset(t, k / kK) + tc::sw64_offset(j % kN, k % kK, 2);
+#pragma unroll
+    for (int b = 0; b < oz::kSlices; ++b)
+      *reinterpret_cast<__half*>(panel + b * kBPanel) = __float2half_rn(oz::small_int_to_float(dg[b]));
+  }
+}
+
+__global__ void __launch_bounds__(128) k_fw_prep(int n, int npad, const double* __restrict__ XT, int* __restrict__ colE,
+                                                 unsigned char* __restrict__ Xs, uint32_t* __restrict__ colHiOut, int nhi,
+                                                 const Ctl* ctl, int level) {
+  if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
+  __shared__ uint32_t red[4];
+  fw_prep_col(n, npad, XT, colE, Xs, colHiOut, nhi, blockIdx.x, red);
+}
+
+// Row blocks of 128 from block rb0 on, every `step`; output tiles from right to left.  False when a wait gave up.
+__device__ __forceinline__ bool fw_blocks(int64_t m, int n, double* __restrict__ Q, int64_t ldq,
+                                          const int* __restrict__ colE, const unsigned char* __restrict__ Xs,
+                                          uint32_t* __restrict__ colHiOut, int64_t rb0, int64_t step, OzPipe& P,
+                                          unsigned char* smem, int* rowE, uint32_t (*red)[kM], uint32_t* cmax) {
+  const int tid = threadIdx.x, lane = tid & 31, ntiles = (n + kN - 1) / kN;
+  const int pr = tid & (kM - 1), pp = tid >> 7, rot = (lane >> 3) & 1;   // producer: row pr, columns 8 pp .. + 7
+  const int rr = P.q * 32 + lane;
+  __syncthreads();
+  for (int j = tid; j < n; j += kOzThreads) cmax[j] = 0u;   // read after the first row maxima's barrier
+  uint32_t off[2];
+  int gcol[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {   // rows r and r + 8 in opposite order: a half warp's 8-byte stores cover all banks
+    gcol[j] = 8 * pp + 4 * (j ^ rot);
+    off[j] = tc::sw64_offset(pr, gcol[j], 2);
+  }
+  for (int64_t rb = rb0; rb * kM < m; rb += step) {
+    const int64_t r0 = rb * kM, prow = min(r0 + pr, m - 1);   // rows beyond m: row m - 1 again, not stored
+    const int64_t rn = r0 + step * kM;
+    if (rn < m)   // the next block into L2
+      for (int e = tid; e < 8 * n; e += kOzThreads)
+        tc::prefetch_l2(Q + min(rn + 16 * (e & 7), m - 1) + (int64_t)(e >> 3) * ldq);
+    uint32_t mx = 0u;
+    const double* p = Q + prow + (int64_t)pp * ldq;
+#pragma unroll 8
+    for (int c = pp; c < n; c += 4) {
+      mx = max(mx, (uint32_t)__double2hiint(*p) & 0x7FFFFFFFu);
+      p += 4 * ldq;
+    }
+    red[pp][pr] = mx;
+    __syncthreads();
+    if (tid < kM) rowE[tid] = (int)oz::exp_field(max(max(red[0][tid], red[1][tid]), max(red[2][tid], red[3][tid])));
+    __syncthreads();
+    const int Er = rowE[pr], cr = oz_quad_cr(Er), Erow = rowE[rr];
+    const bool rlive = r0 + rr < m;
+    for (int t = ntiles - 1; t >= 0; --t) {
+      long long hi[16], lo[16];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0;
+      double v[2][4];
+      auto load_w = [&](int kc) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int k0 = kc * kK + gcol[j];
+          const double* w = Q + prow + (int64_t)k0 * ldq;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            v[j][c] = k0 + c < n ? *w : 0.0;
+            w += ldq;
+          }
+        }
+      };
+      load_w(0);
+      const int nch = 2 * (t + 1);
+      auto produce = [&](int kc, unsigned char* a, unsigned char* b) {
+        const unsigned char* src = Xs + fw_block_offset(t, kc);
+#pragma unroll
+        for (int i = 0; i < (int)(oz::kSlices * kBPanel / 16 / kOzThreads); ++i)
+          tc::cp_async16(b + 16 * (tid + kOzThreads * i), src + 16 * (tid + kOzThreads * i));
+        const uint32_t sa = tc::smem_u32(a);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) oz_store_quad(v[j], 0u, Er, cr, sa + off[j], kAPanel);
+        if (kc + 1 < nch) load_w(kc + 1);
+        tc::cp_async_wait_all();
+      };
+      if (!oz_run(P, smem, nch, produce, hi, lo)) return false;
+      const int c0 = t * kN + P.g * 16;
+      double* q = Q + r0 + rr + (int64_t)c0 * ldq;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        if (rlive && c0 + c < n) {
+          const int ce = colE[c0 + c], scale = Erow + ce - oz::kScaleBias;
+          double x = (c & 1) ? oz::t96_to_double_fp64(hi[c], lo[c], scale) : oz::t96_to_double(hi[c], lo[c], scale);
+          if (Erow == 2047 || ce == 2047) x = nan64();   // non-finite operands
+          *q = x;
+          const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+          if (h > cmax[c0 + c]) atomicMax(cmax + c0 + c, h);
+        }
+        q += ldq;
+      }
+      __syncthreads();   // the tile's Q before the next tile's loads, the panels free
+    }
+  }
+  __syncthreads();
+  if (colHiOut)
+    for (int j = tid; j < n; j += kOzThreads)
+      if (cmax[j]) atomicMax(colHiOut + j, cmax[j]);
+  return true;
+}
+
+__global__ void __launch_bounds__(kOzThreads, 1)
+    k_fw_product(int64_t m, int n, double* __restrict__ Q, int64_t ldq, const int* __restrict__ colE,
+                 const unsigned char* __restrict__ Xs, uint32_t* __restrict__ colHiOut, Ctl* ctl, int level) {
+  if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t mma_bar[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int rowE[kM];
+  __shared__ uint32_t red[4][kM], cmax[512];
+  OzPipe P = oz_begin(&tmem_slot, mma_bar);
+  const bool ok = fw_blocks(m, n, Q, ldq, colE, Xs, colHiOut, blockIdx.x, gridDim.x, P, oz_smem(smem_raw), rowE, red, cmax);
+  oz_end(P, !ok, ctl);
+}
+
+// Grouped forms for batched plans: items {i, column < n64} and {i, 128-row block}.
+__global__ void __launch_bounds__(128) kg_fw_prep(Group g, int level) {
+  __shared__ uint32_t red[4];
+  for (int it = blockIdx.x; it < g.nitems; it += gridDim.x) {
+    const int4 w = g.items[it];
+    const Prob& P = g.probs[w.x];
+    if (P.ctl->active != level || P.ctl->lvl_status != 0) continue;
+    fw_prep_col(P.n, P.npad, P.xt, P.oz_xe, P.oz_xs, P.check ? P.oz_colhi : nullptr, (P.n + kM - 1) / kM * kM, w.y, red);
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(kOzThreads, 1) kg_fw_product(Group g, int level) {
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t mma_bar[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int rowE[kM];
+  __shared__ uint32_t red[4][kM], cmax[512];
+  OzPipe P = oz_begin(&tmem_slot, mma_bar);
+  bool abort = false;
+  Ctl* actl = nullptr;
+  for (int it = blockIdx.x; it < g.nitems; it += gridDim.x) {
+    const int4 w = g.items[it];
+    const Prob& B = g.probs[w.x];
+    if (B.ctl->active != level || B.ctl->lvl_status != 0) continue;
+    if (!fw_blocks(B.m, B.n, B.Q, B.ldq, B.oz_xe, B.oz_xs, B.check ? B.oz_colhi : nullptr, w.y, (B.m + kM - 1) / kM, P,
+                   oz_smem(smem_raw), rowE, red, cmax)) {
+      abort = true;
+      actl = B.ctl;
+      break;
+    }
+  }
+  oz_end(P, abort, actl);
+}
 
 // ---------------------------------------------------------------------------
 // Gram G = W^T W (Algorithm 1 step 1) and the check matrix Q^T Q.  Every
@@ -541,6 +734,18 @@ void launch_syrk_oz(int64_t m, int n, const double* W, int64_t ldw, const SyrkOz
 }
 
 
+size_t fw_digit_bytes(int n) { return fw_block_offset((n + kN - 1) / kN, 0); }
+
+void launch_finalize_wide(int64_t m, int n, double* Q, int64_t ldq, const double* XT, int* colE, unsigned char* Xs,
+                          Ctl* ctl, int level, cudaStream_t st, uint32_t* colHiOut) {
+  const int nhi = (int)(syrk_oz_colhi_bytes(n) / sizeof(uint32_t)), npad = (n + 31) / 32 * 32;
+  launch_dep(k_fw_prep, (n + kN - 1) / kN * kN, 128, 0, st, n, npad, XT, colE, Xs, colHiOut, nhi, ctl, level);
+  set_smem(k_fw_product);
+  const int64_t nblocks = (m + kM - 1) / kM;
+  launch_dep(k_fw_product, (unsigned)std::min<int64_t>(nblocks, num_sms()), kOzThreads, kSmem, st, m, n, Q, ldq, colE, Xs,
+             colHiOut, ctl, level);
+}
+
 SketchOzPlan sketch_oz_plan(int64_t m, int n, int s) {
   SketchOzPlan P{};
   P.mblocks = (n + kM - 1) / kM;
@@ -575,8 +780,15 @@ unsigned grid_oz(int nitems, int per_sm) {
 void prepare_g_oz_kernels() {
   cudaFuncSetAttribute(kg_oz_sketch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
   cudaFuncSetAttribute(kg_oz_syrk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  cudaFuncSetAttribute(kg_fw_product, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
 }
 
+void launch_g_fw_prep(const Group& g, int level, cudaStream_t st) {
+  if (g.nitems) { ::mrcqr::note_launch(); kg_fw_prep<<<grid_oz(g.nitems, 16), 128, 0, st>>>(g, level); }
+}
+void launch_g_fw_product(const Group& g, int level, cudaStream_t st) {
+  if (g.nitems) { ::mrcqr::note_launch(); kg_fw_product<<<grid_oz(g.nitems, 1), kOzThreads, kSmem, st>>>(g, level); }
+}
 void launch_g_oz_colhi(const Group& g, int level, cudaStream_t st) {
   if (g.nitems) { ::mrcqr::note_launch(); kg_oz_colhi<<<grid_oz(g.nitems, 16), 256, 0, st>>>(g, level); }
 }

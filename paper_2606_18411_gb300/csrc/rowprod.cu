@@ -36,13 +36,13 @@
 //
 // Measured at m = 2^20 (before: substitution blocks of 16 columns; Q = W X in
 // 128 x 64 tiles by one CTA per SM): W = A R^{-1} 1.78 -> 0.75 ms at n = 64,
-// 4.53 -> 1.80 at 128, 12.7 -> 5.9 at 256, 41.3 -> 20.5 at 512 (m = 300001, n = 320: 2.94 ms
-// with one reference for all columns, 2.93 with the column scales, 2.99 with the check of
-// an R of the caller's); Q = W X
-// 0.99 -> 0.63, 2.19 -> 1.61, 5.67 -> 5.39, 17.3 -> 18.6.  What bounds them is
-// integer-pipe work around the products (slicing about 1100 cycles per SM and
-// chunk, conversion of the results about 2400 per tile, against 1340 of MMAs
-// per chunk) and, with two CTAs per SM, the latency of a block's phases.
+// 4.53 -> 1.80 at 128, 12.7 -> 5.9 at 256, 41.3 -> 20.5 at 512 (m = 300001,
+// n = 320: 2.94 ms with one reference for all columns, 2.93 with the column
+// scales, 2.99 with the check of an R of the caller's); Q = W X 0.99 -> 0.63 at
+// n = 64, 2.19 -> 1.61 at 128 (wide W takes 64-column tiles: ozaki.cu, rp_wide).
+// What bounds them is integer-pipe work around the products (slicing about 1100
+// cycles per SM and chunk, conversion of the results about 2400 per tile, against
+// 1340 of MMAs per chunk) and, with two CTAs per SM, the latency of a block's phases.
 #include <climits>
 
 #include "kernels.h"
@@ -1151,9 +1151,9 @@ unsigned rp_grid(int nitems, int per_sm) {
 }  // namespace
 
 // Workspace sizes: digit panels of the multiplier blocks (the TRSM has two sets), and the exponents.
-size_t rp_digit_bytes(int n) { return rp_digit_size(n); }
 size_t rp_trsm_digit_bytes(int n) { return 2 * rp_digit_size(n); }
 size_t rp_trsm_ints_bytes(int n) { return sizeof(int) * (size_t)(4 * rp_n32(n) + 16); }
+size_t rp_fin_digit_bytes(int n) { return rp_wide(n) ? fw_digit_bytes(n) : rp_digit_size(n); }
 size_t rp_fin_ints_bytes(int n) { return sizeof(int) * (size_t)rp_n32(n); }
 int rp_cols(int n) { return rp_n32(n); }
 int rp_panels(int n) { return rp_n32(n) / kRN; }
@@ -1177,6 +1177,10 @@ void launch_trsm_oz(int64_t m, int n, const double* A, int64_t lda, const double
 
 void launch_finalize_oz(int64_t m, int n, double* Q, int64_t ldq, const double* XT, int* colE, unsigned char* Xs,
                         Ctl* ctl, int level, cudaStream_t st, uint32_t* colHiOut) {
+  if (rp_wide(n)) {
+    launch_finalize_wide(m, n, Q, ldq, XT, colE, Xs, ctl, level, st, colHiOut);
+    return;
+  }
   const int n32 = rp_n32(n);
   const int nhi = (int)(syrk_oz_colhi_bytes(n) / sizeof(uint32_t));
   launch_dep(k_rp_prep_x, n32, 128, 0, st, n, n32, XT, colE, Xs, colHiOut, nhi, ctl, level);

@@ -108,3 +108,42 @@ def test_gram_quads_at_edges(env, m, n, ld):
     C = np.abs(W).max(0)
     upper = np.triu(np.ones((n, n), bool))
     assert np.all(np.abs(G - exact)[upper] <= (2 * U * np.abs(exact) + 2.0 ** -57 * m * C[:, None] * C[None, :])[upper])
+
+
+# The 64-column tiles of wide W: at and around their widths (161, 192, 256, 289, 512 take them, 160, 224 and 257 do
+# not), heights around a block of 128 rows, an odd leading dimension; a non-finite entry stays in its row.
+@pytest.mark.parametrize("m,n,ld", [(129, 160, 0), (127, 161, 128), (257, 192, 0), (130, 224, 131), (131, 256, 0),
+                                    (128, 257, 0), (200, 289, 0), (1, 320, 0), (150, 512, 151)])
+def test_finalize_of_wide_matrices(env, m, n, ld):
+    torch, M = env
+    rng = np.random.default_rng(m + n)
+    W = rng.standard_normal((m, n))
+    W[::3] *= 2.0 ** -45                              # each row has its own reference
+    W[:, ::4] *= 2.0 ** -40                           # columns below the fast slicing's range
+    W[rng.random((m, n)) < 0.05] = 0.0
+    X = np.triu(rng.standard_normal((n, n)))
+    Q = M.finalize_q(M.to_colmajor(W, ld=ld or None), M.to_colmajor(X)).cpu().numpy()
+    rows = np.arange(m)[::max(1, m * n // 16000)]
+    exact = O.product_rounded(W, X, rows=rows)
+    bound = 2 * U * np.abs(exact) + 2.0 ** -57 * n * np.abs(W[rows]).max(1)[:, None] * np.abs(X).max(0)[None, :]
+    assert np.all(np.abs(Q[rows] - exact) <= bound)
+    W[m // 2, n // 3] = np.nan
+    Qn = M.finalize_q(M.to_colmajor(W), M.to_colmajor(X)).cpu().numpy()
+    np.testing.assert_array_equal(np.delete(Qn, m // 2, 0), np.delete(Q, m // 2, 0))
+    assert np.isnan(Qn[m // 2]).all()
+
+
+def test_batched_wide_problems_match_single_launches(env):
+    torch, M = env
+    rng = np.random.default_rng(4)
+    shapes = [(900, 161), (700, 64), (1300, 320), (640, 224)]
+    As = [M.to_colmajor(rng.standard_normal(sh)) for sh in shapes]
+    out = []
+    for per_problem in (0, 1):
+        Qs, Rs = [M.empty_colmajor(*sh) for sh in shapes], [M.empty_colmajor(sh[1], sh[1]) for sh in shapes]
+        status = torch.full((len(shapes),), -1, dtype=torch.int32, device="cuda")
+        M.BatchedPlan(As, Qs, Rs, ["fp32"] * 4, [1, 2, 3, 4], status, oz_per_problem=per_problem).execute()
+        assert status.cpu().tolist() == [0] * 4
+        out.append([t.cpu().numpy() for t in Qs + Rs])
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
