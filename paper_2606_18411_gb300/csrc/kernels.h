@@ -7,6 +7,7 @@
 
 namespace mrcqr {
 
+int device_sms();   // SMs of the device (the first one asked for; a process uses GPUs of one kind)
 void note_launch();   // counts one kernel launch, called just before it (api.cu); read through mrcqr_launch_count
 
 // Launches a kernel whose first action is wait_prior_kernels() (level_inactive

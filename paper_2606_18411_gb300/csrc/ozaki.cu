@@ -21,6 +21,17 @@
 
 namespace mrcqr {
 
+int device_sms() {
+  static int cached = 0;
+  if (!cached) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cached = sms > 0 ? sms : 152;
+  }
+  return cached;
+}
+
 namespace {
 
 // ---------------------------------------------------------------------------
@@ -629,24 +640,13 @@ __global__ void __launch_bounds__(256) kg_oz_syrk_reduce(Group g, int check, int
   }
 }
 
-int num_sms() {
-  static int cached = 0;
-  if (!cached) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cached = sms > 0 ? sms : 152;
-  }
-  return cached;
-}
-
 int gcd_int(int a, int b) { return b ? gcd_int(b, a % b) : a; }
 
 // Row slabs so that tiles x slabs is a multiple of the SM count where the
 // rows allow it; at least 256 rows per slab, at most 2^20 (the 64-bit halves
 // of an item stay below 2^61).
 int choose_slabs(int64_t m, int tiles, int64_t* rows_per_slab) {
-  const int sms = num_sms();
+  const int sms = device_sms();
   int slabs = tiles >= sms ? 1 : sms / gcd_int(tiles, sms);
   const int64_t max_slabs = (m + 255) / 256;
   if (slabs > max_slabs) slabs = (int)max_slabs;
@@ -675,7 +675,7 @@ namespace {
 void launch_col_hi(int64_t m, int n, const double* X, int64_t ldx, uint32_t* colHi, const Ctl* ctl, int level,
                    cudaStream_t st) {
   cudaMemsetAsync(colHi, 0, syrk_oz_colhi_bytes(n), st);
-  int ysplit = (4 * num_sms() + n - 1) / n;
+  int ysplit = (4 * device_sms() + n - 1) / n;
   const int64_t max_y = (m + 4095) / 4096;
   if (ysplit > max_y) ysplit = (int)max_y;
   if (ysplit < 1) ysplit = 1;
@@ -727,7 +727,7 @@ void launch_syrk_oz(int64_t m, int n, const double* W, int64_t ldw, const SyrkOz
   if (!colhi_ready) launch_col_hi(m, n, W, ldw, colHi, ctl, level, st);
   set_smem(k_syrk_oz);
   const int nitems = P.ntiles * P.slabs;
-  launch_dep(k_syrk_oz, nitems < num_sms() ? nitems : num_sms(), kOzThreads, kSmem, st, m, n, W, ldw, colHi, P, part, ctl,
+  launch_dep(k_syrk_oz, nitems < device_sms() ? nitems : device_sms(), kOzThreads, kSmem, st, m, n, W, ldw, colHi, P, part, ctl,
                                                                                level);
   const int64_t nn = (int64_t)n * n;
   launch_dep(k_syrk_oz_reduce, (unsigned)((nn + 255) / 256), 256, 0, st, n, colHi, P, part, out, ctl, level);
@@ -742,7 +742,7 @@ void launch_finalize_wide(int64_t m, int n, double* Q, int64_t ldq, const double
   launch_dep(k_fw_prep, (n + kN - 1) / kN * kN, 128, 0, st, n, npad, XT, colE, Xs, colHiOut, nhi, ctl, level);
   set_smem(k_fw_product);
   const int64_t nblocks = (m + kM - 1) / kM;
-  launch_dep(k_fw_product, (unsigned)std::min<int64_t>(nblocks, num_sms()), kOzThreads, kSmem, st, m, n, Q, ldq, colE, Xs,
+  launch_dep(k_fw_product, (unsigned)std::min<int64_t>(nblocks, device_sms()), kOzThreads, kSmem, st, m, n, Q, ldq, colE, Xs,
              colHiOut, ctl, level);
 }
 
@@ -764,7 +764,7 @@ void launch_sketch_oz(int64_t m, int n, int s, const double* A, int64_t lda, con
   launch_col_hi(m, n, A, lda, colHi, ctl, level, st);
   set_smem(k_sketch_oz);
   const int nitems = P.mblocks * P.ntiles * P.slabs;
-  launch_dep(k_sketch_oz, nitems < num_sms() ? nitems : num_sms(), kOzThreads, kSmem, st, m, n, s, A, lda, colHi, idx, tab,
+  launch_dep(k_sketch_oz, nitems < device_sms() ? nitems : device_sms(), kOzThreads, kSmem, st, m, n, s, A, lda, colHi, idx, tab,
                                                                                  seed_key(seed), P, part, ctl, level, tf);
   launch_sketch_oz_reduce(n, s, colHi, idx, P, part, Y, ctl, level, st, tf, m);
 }
@@ -772,7 +772,7 @@ void launch_sketch_oz(int64_t m, int n, int s, const double* A, int64_t lda, con
 // ---- grouped launches -------------------------------------------------------
 namespace {
 unsigned grid_oz(int nitems, int per_sm) {
-  const int cap = num_sms() * per_sm;
+  const int cap = device_sms() * per_sm;
   return (unsigned)(nitems < cap ? nitems : cap);
 }
 }  // namespace

@@ -234,20 +234,16 @@ __device__ __forceinline__ void oz_load_cols(const double* __restrict__ X, int64
 }
 
 // Digits of the values loaded by oz_load_cols (reference exponent E[c], sign
-// flips f0 / f1 of the lane's two rows) into panel rows c.  With dup >= 0 the
-// rows c in [dup, dup + kN) are also written to rows c - dup of the B panels
-// at bpanel (a diagonal Gram tile, whose B operand is part of its A operand).
+// flips f0 / f1 of the lane's two rows) into panel rows c.
 template <int NC>
 __device__ __forceinline__ void oz_store_cols(const double (&v)[NC / 32][2], const uint32_t* E, uint32_t f0,
                                               uint32_t f1, unsigned char* panel, uint32_t pstride, int warp,
-                                              int lane, int dup = -1, unsigned char* bpanel = nullptr) {
+                                              int lane) {
   const int p = lane & 15, h = lane >> 4;
 #pragma unroll
   for (int it = 0; it < NC / 32; ++it) {
     const int c = 32 * it + 2 * warp + h;
-    const bool d = dup >= 0 && c >= dup && c < dup + kN;   // uniform per it (dup a multiple of 64)
-    oz_store_pair(v[it][0], v[it][1], f0, f1, E[c], tc::smem_u32(panel) + tc::sw64_offset(c, 2 * p, 2), pstride, 0, 0,
-                  d ? tc::smem_u32(bpanel) + tc::sw64_offset(c - dup, 2 * p, 2) : 0u, kBPanel);
+    oz_store_pair(v[it][0], v[it][1], f0, f1, E[c], tc::smem_u32(panel) + tc::sw64_offset(c, 2 * p, 2), pstride);
   }
 }
 
@@ -275,7 +271,7 @@ __device__ __forceinline__ void rp_issue(uint32_t tmem, uint32_t ab, uint32_t bb
 
 struct OzPipe {
   uint64_t* bar;      // [2]: oz_run commits every batch to bar[0]; two batches in flight alternate bar[0] / bar[1]
-  uint32_t tmem, idesc;
+  uint32_t tmem;
   uint32_t mph;       // bit b: parity of the next completion of bar[b] (the same in every thread)
   uint32_t mopen;     // issuing thread: bit b = a batch committed to bar[b] and not yet waited for
   int tid, q, g;
@@ -352,7 +348,6 @@ __device__ __forceinline__ OzPipe oz_begin(uint32_t* tmem_slot, uint64_t* bar) {
   OzPipe P;
   P.bar = bar;
   P.tmem = *tmem_slot;
-  P.idesc = tc::idesc(tc::F16, kM, kN);
   P.mph = 0;
   P.mopen = 0;
   P.tid = tid;

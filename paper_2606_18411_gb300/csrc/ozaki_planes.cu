@@ -280,17 +280,6 @@ EncodeFn encode_fn() {
   return fn;
 }
 
-int sm_count() {
-  static int cached = 0;
-  if (!cached) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    cached = v > 0 ? v : 152;
-  }
-  return cached;
-}
-
 constexpr int64_t kMinChunkRows = 1024;
 
 }  // namespace
@@ -343,7 +332,7 @@ bool launch_sketch_ozp(int64_t m, int n, int s, const double* A, int64_t lda, co
   const int64_t tq = (m + 2) / 2;   // table entries 0 .. m, two per thread
   launch_dep(k_oz_tab_digits, (unsigned)((tq + 255) / 256), 256, 0, st, m, tab, tabd, ctl, level);
   const uint2 key = seed_key(seed);
-  const int grid = items < sm_count() ? items : sm_count();
+  const int grid = items < device_sms() ? items : device_sms();
   for (int64_t k = 0; k < nch; ++k) {
     const int64_t row0 = k * R, mc = std::min(R, m - row0);
     const int64_t pairs = (mc + 1) / 2;

@@ -1023,17 +1023,6 @@ __global__ void __launch_bounds__(256) k_rp_prep_r(int n, int npad, const double
   }
 }
 
-int rp_sms() {
-  static int cached = 0;
-  if (!cached) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cached = sms > 0 ? sms : 152;
-  }
-  return cached;
-}
-
 // ---------------------------------------------------------------------------
 // Grouped forms for batched plans: persistent launches over {problem, block}
 // items; an item whose problem is not active at this level, or has raised a
@@ -1136,7 +1125,7 @@ __global__ void __launch_bounds__(256) kg_rp_prep_r(Group g, int level) {
 
 template <bool kTrsm, bool kCheck>
 void rp_launch(const RpArgs& a, Ctl* ctl, int level, cudaStream_t st) {
-  const int64_t nblocks = (a.m + kM - 1) / kM, slots = 2 * (int64_t)rp_sms();
+  const int64_t nblocks = (a.m + kM - 1) / kM, slots = 2 * (int64_t)device_sms();
   const unsigned grid = (unsigned)(nblocks < slots ? nblocks : slots);
   auto kernel = a.n > kRN * kGroupChunks ? k_rowprod<kTrsm, true, kCheck> : k_rowprod<kTrsm, false, kCheck>;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRSmem);
@@ -1144,7 +1133,7 @@ void rp_launch(const RpArgs& a, Ctl* ctl, int level, cudaStream_t st) {
 }
 
 unsigned rp_grid(int nitems, int per_sm) {
-  const int cap = rp_sms() * per_sm;
+  const int cap = device_sms() * per_sm;
   return (unsigned)(nitems < cap ? nitems : cap);
 }
 

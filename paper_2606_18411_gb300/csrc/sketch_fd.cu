@@ -525,17 +525,6 @@ __global__ void __launch_bounds__(256) k_fd_reduce(int n, int s, int cblocks, in
   }
 }
 
-int fd_sms() {
-  static int cached = 0;
-  if (!cached) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    cached = v > 0 ? v : 152;
-  }
-  return cached;
-}
-
 // The split of a problem: equal ranges of at most Jc rows j1 (a multiple of
 // 128) that fit the scratch, each in slabs; about four items per CTA over all
 // tiles.  Only the rows left run in the last range (a range of Jc rows each time
@@ -559,7 +548,7 @@ FdPlan fd_plan(int64_t m, int n, int s, size_t scratch_bytes) {
   p.Jc = ((J128 + p.chunks - 1) / p.chunks + kM - 1) / kM * kM;
   p.cblocks = (n + kM - 1) / kM;
   p.max_tiles = kClasses + s / kFdTile;
-  const int64_t want = (8 * (int64_t)fd_sms() + p.max_tiles * p.cblocks * p.chunks - 1) / (p.max_tiles * p.cblocks * p.chunks);
+  const int64_t want = (8 * (int64_t)device_sms() + p.max_tiles * p.cblocks * p.chunks - 1) / (p.max_tiles * p.cblocks * p.chunks);
   const int64_t slabs = std::max<int64_t>(1, std::min(want, p.Jc / kM));
   p.rows = (p.Jc + slabs - 1) / slabs;
   p.rows = (p.rows + kM - 1) / kM * kM;
@@ -618,12 +607,12 @@ void launch_sketch_fd(int64_t m, int n, int s, const double* A, int64_t lda, con
     const int64_t j0 = (int64_t)k * p.Jc;
     const int nblocks = (int)(p.range(k) / kM), slabs = p.range_slabs(k);   // rows j1 >= J give zero words
     const int64_t items = (int64_t)nblocks * n;
-    launch_dep(k_fd_pass1, (unsigned)std::min<int64_t>(items, 2 * fd_sms()), kRThreads, kFdSmem, st, p.J, j0, p.Jc, nblocks, n, A, lda, colHi, colU, sgn, U, cs, ctl, level);
+    launch_dep(k_fd_pass1, (unsigned)std::min<int64_t>(items, 2 * device_sms()), kRThreads, kFdSmem, st, p.J, j0, p.Jc, nblocks, n, A, lda, colHi, colU, sgn, U, cs, ctl, level);
     const Fd2Args a{m, p.J, j0, p.Jc, p.rows, p.range(k), n, p.cblocks, slabs, U, cs, idx, tabd, ntiles, cls, slots, part,
                     slab0, slabs_all};
     slab0 += slabs;
     const int64_t most = (int64_t)p.max_tiles * p.cblocks * slabs;
-    launch_dep(k_fd_pass2, (unsigned)std::min<int64_t>(most, 2 * fd_sms()), kRThreads, kFdSmem, st, a, ctl, level);
+    launch_dep(k_fd_pass2, (unsigned)std::min<int64_t>(most, 2 * device_sms()), kRThreads, kFdSmem, st, a, ctl, level);
   }
   const dim3 rg((unsigned)(kFdTile * p.max_tiles / 2), (unsigned)p.cblocks);
   launch_dep(k_fd_reduce, rg, 256, 0, st, n, s, p.cblocks, slabs_all, ntiles, slots, colHi, colU, idx, part, Y, ctl, level);

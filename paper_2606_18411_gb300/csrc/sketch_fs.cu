@@ -504,17 +504,6 @@ EncodeFn fs_encode_fn() {
   return fn;
 }
 
-int sms() {
-  static int cached = 0;
-  if (!cached) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    cached = v > 0 ? v : 152;
-  }
-  return cached;
-}
-
 template <int PREC>
 bool launch_fs(const double* A, int64_t lda, int64_t m, int n, int s, const uint32_t* idx, const double* tab,
                uint64_t seed, int chunks, double* Ypart, Ctl* ctl, int level, cudaStream_t st) {
@@ -538,7 +527,7 @@ bool launch_fs(const double* A, int64_t lda, int64_t m, int n, int s, const uint
   const int ntiles = (int)(m1 / kB);
   const int tpc = ntiles / chunks;
   const int nitems = ((n + F::C - 1) / F::C) * chunks;
-  const int grid = nitems < sms() ? nitems : sms();
+  const int grid = nitems < device_sms() ? nitems : device_sms();
   launch_dep(k_sketch_fs<PREC>, grid, kThreads, smem, st, map, m, n, s, idx, tab, seed_key(seed), chunks, tpc, Ypart, ctl, level);
   return true;
 }
