@@ -303,9 +303,8 @@ __device__ __forceinline__ bool chol_shared(int w, double* S, int ld, double* ro
 }
 
 // The whole elimination in one CTA's shared memory (n <= kCholSmemN).
-// Measured (before: square root and division by one thread between barriers; n > 64 blocked):
-// the figures stand at launch_chol.
-constexpr int kCholSmemN = 160;
+// The figures stand at launch_chol.
+constexpr int kCholSmemN = 88;
 
 __global__ void __launch_bounds__(1024) k_chol_smem(int n, double* __restrict__ G, Ctl* ctl, int level) {
   if (level_inactive(ctl, level) || ctl->lvl_status != 0) return;
@@ -414,13 +413,16 @@ __global__ void __launch_bounds__(256) k_chol_update(int n, int c0, double* __re
   }
 }
 
-// One CTA with the triangle in shared memory up to kCholSmemN columns (one
-// launch; the longest n whose padded square fits beside nothing else), blocked
+// One CTA with the triangle in shared memory up to kCholSmemN columns, blocked
 // over the chip beyond.  FP64 has 1/64 of the FP32 rate, so one warp's FP64
 // instruction holds a quadrant's pipe for 64 clocks: the pivot's reciprocal
-// square root and the column scaling are done once, not per thread.  Measured
-// (one level, us, before / now): n = 32 50 / 35, 64 117 / 88, 128 280 / 249
-// (all one launch over global memory before), 256 561 / 397, 512 1129 / 814.
+// square root and the column scaling are done once, not per thread.  Measured (us,
+// one CTA / blocked; a skipped level 5 against 7 to 15): n = 40 45 / 53, 64 90 / 81,
+// 80 120 / 109, 96 157 / 128, 128 253 / 175, 160 388 / 223; a factorization with two
+// skipped levels, m = 8192: n = 80 776 / 784, 96 891 / 887, 128 1126 / 1073.  So the line
+// lies between 80 and 96.  (The pivot by square root and division between barriers, in
+// shared memory up to n = 64 and by one warp per panel beyond: n = 32 50, 64 117,
+// 128 280, 256 561, 512 1129; now 35, 90, 175, 397, 814.)
 // 512 threads up to n = 48 (35 us, 38 with 1024: fewer warps at the barriers).
 void launch_chol(int n, double* G, Ctl* ctl, int level, cudaStream_t st) {
   if (n > kCholSmemN) {

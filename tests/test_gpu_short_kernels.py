@@ -103,3 +103,8 @@ def test_pivot_is_correctly_rounded(env):
     np.testing.assert_array_equal(p[:len(d)], np.sqrt(d))          # IEEE square root and division
     np.testing.assert_array_equal(y[:len(d)], 1.0 / np.sqrt(d))
     assert (p[len(d):] == -1.0).all() and (y[len(d):] == -1.0).all()
+
+
+@pytest.mark.parametrize("n", [87, 88, 89, 96, 97])   # one CTA up to 88, panels of 32 beyond
+def test_cholesky_at_the_switch(env, n):
+    test_cholesky_sizes(env, n)
