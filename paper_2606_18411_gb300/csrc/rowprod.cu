@@ -211,13 +211,21 @@ __device__ __forceinline__ void rp_end(const RpArgs& a, RpCta& S) {
 // and receives B R_tt^{-1} in its first w columns.
 __device__ __noinline__ void rp_substitute(const RpArgs& a, double* sb, int c0, int row) {
   const int npad = (a.n + 31) / 32 * 32, w = min(kRN, a.n - c0);
-  for (int c = 0; c < w; ++c) {
-    const double x = sb[c * kM + row] * a.rinv[c0 + c];
-    sb[c * kM + row] = x;
-    const double* r = a.RT + (int64_t)(c0 + c) * npad + c0;
-#pragma unroll 4
-    for (int c2 = c + 1; c2 < w; ++c2) sb[c2 * kM + row] = fma(-x, r[c2], sb[c2 * kM + row]);
+  double b[kRN];   // the row in registers: in shared memory every step waited for its load and store
+#pragma unroll
+  for (int c = 0; c < kRN; ++c) b[c] = sb[c * kM + row];
+#pragma unroll
+  for (int c = 0; c < kRN; ++c) {
+    if (c < w) {
+      const double x = b[c] * a.rinv[c0 + c];
+      b[c] = x;
+      const double* r = a.RT + (int64_t)(c0 + c) * npad + c0;   // row c0 + c of R, zeros from column n to npad
+#pragma unroll
+      for (int c2 = c + 1; c2 < kRN; ++c2) b[c2] = fma(-x, __ldg(r + c2), b[c2]);
+    }
   }
+#pragma unroll
+  for (int c = 0; c < kRN; ++c) sb[c * kM + row] = b[c];
 }
 
 // A row with a non-finite entry of A in the panel at c0: columns cb .. cb + 15 of the panel by FP64 substitution along
