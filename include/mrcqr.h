@@ -305,7 +305,7 @@ int mrcqr_cholqr_precond(int64_t m, int64_t n, const double* A, int64_t lda, con
  * FP64 product on the FP16 tensor cores, W_t = A_t X_t + W_{<t} Z_t with X_t =
  * R_tt^{-1} and Z_t = -R_{<t,t} X_t formed to 2^-61 of their column maxima (one
  * rounding per entry); a panel whose X_t would amplify the product's error more
- * than 512-fold is solved by FP64 substitution on its diagonal block instead.
+ * than 1024-fold is solved by FP64 substitution on its diagonal block instead.
  * Columns enter scaled by the powers of two of R's column maxima; a panel with a
  * column of A far from them within 128 rows is solved by substitution too, so the
  * backward error of every column is that of a triangular solve.  A

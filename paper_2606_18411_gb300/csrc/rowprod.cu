@@ -25,10 +25,13 @@
 //    digits, about 2^-60 max|row| max|column| per entry.  Seen as a backward error
 //    of A F^{-1} it is amplified by at most
 //      amp = max_j sum_c max|column c of (Z_t; X_t)| |(R F^{-1})_tt[c][j]|,
-//    and a panel whose amp exceeds 512 (measured: below 400 for the R of sketched
-//    matrices with kappa up to 1e16, four spectra, n = 32 .. 512) keeps the
-//    substitution: the product is W_{<t} (-R_{<t,t}) alone (A's digits are
-//    zeros in it), A_t is added and R_tt solved with in FP64.
+//    and a panel whose amp exceeds 1024 keeps the substitution: the product is
+//    W_{<t} (-R_{<t,t}) alone (A's digits are zeros in it), A_t is added and R_tt solved
+//    with in FP64.  (Largest column error of 288 solves, n = 8 .. 64, two spectra, kappa
+//    to 1e16, in units of u |W| |R|: amp below 256 0.7, 512 .. 1024 1.9, 1024 .. 2048 3.1,
+//    2048 .. 4096 7.1; FP64 substitution 1.0.  Among R of sketched matrices with kappa of
+//    1e12 and 1e16 17% pass 1024 at n = 32, 7% at 64, 1% at 100, in their first panels;
+//    a kept panel costs about three of the others.)
 //    F fits A where W's columns are of one size, as for a factor R of A.  Where R is
 //    the caller's (mrcqr_trsm, mrcqr_cholqr_precond) a row block checks it: a panel with a
 //    column of A F^{-1} below 2^-10 of the largest entry of the block's A F^{-1} or W D
@@ -61,7 +64,7 @@ namespace {
 // leaves the tensor cores idle in every other phase of a row block.
 constexpr size_t kRSmem = (size_t)kRABytes + 2 * (size_t)kRBBytes + 1024;
 constexpr int kNoEntry = -100000, kNonfinite = 100000;
-constexpr float kAmpLimit = 512.0f;
+constexpr float kAmpLimit = 1024.0f;
 // Binades a column of A F^{-1} may lie below the block's largest entry: 2^-62 2^10 amp sqrt(n) stays at the n u of a
 // triangular solve, and a matched R reaches 2^7 (largest of 128 n Gaussians times sqrt(n) against a column's largest).
 constexpr int kBalance = 10;
