@@ -214,21 +214,29 @@ __device__ __forceinline__ void rp_end(const RpArgs& a, RpCta& S) {
 // and receives B R_tt^{-1} in its first w columns.
 __device__ __noinline__ void rp_substitute(const RpArgs& a, double* sb, int c0, int row) {
   const int npad = (a.n + 31) / 32 * 32, w = min(kRN, a.n - c0);
-  double b[kRN];   // the row in registers: in shared memory every step waited for its load and store
+  for (int h = 0; h < kRN; h += 16) {   // half a row in registers: a whole one takes them from the kernel's hot path
+    double b[16];
 #pragma unroll
-  for (int c = 0; c < kRN; ++c) b[c] = sb[c * kM + row];
+    for (int c = 0; c < 16; ++c) b[c] = sb[(h + c) * kM + row];
+    const double* r0 = a.RT + (int64_t)c0 * npad + c0 + h;
+#pragma unroll 1
+    for (int c = 0; c < h && c < w; ++c) {
+      const double x = sb[c * kM + row];
 #pragma unroll
-  for (int c = 0; c < kRN; ++c) {
-    if (c < w) {
-      const double x = b[c] * a.rinv[c0 + c];
-      b[c] = x;
-      const double* r = a.RT + (int64_t)(c0 + c) * npad + c0;   // row c0 + c of R, zeros from column n to npad
-#pragma unroll
-      for (int c2 = c + 1; c2 < kRN; ++c2) b[c2] = fma(-x, __ldg(r + c2), b[c2]);
+      for (int c2 = 0; c2 < 16; ++c2) b[c2] = fma(-x, __ldg(r0 + (int64_t)c * npad + c2), b[c2]);
     }
-  }
 #pragma unroll
-  for (int c = 0; c < kRN; ++c) sb[c * kM + row] = b[c];
+    for (int c = 0; c < 16; ++c)
+      if (h + c < w) {
+        const double x = b[c] * a.rinv[c0 + h + c];
+        b[c] = x;
+        const double* r = r0 + (int64_t)(h + c) * npad;
+#pragma unroll
+        for (int c2 = c + 1; c2 < 16; ++c2) b[c2] = fma(-x, __ldg(r + c2), b[c2]);
+      }
+#pragma unroll
+    for (int c = 0; c < 16; ++c) sb[(h + c) * kM + row] = b[c];
+  }
 }
 
 // A row with a non-finite entry of A in the panel at c0: columns cb .. cb + 15 of the panel by FP64 substitution along
@@ -382,6 +390,7 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
           const uint32_t h = (uint32_t)__double2hiint(v[j][c]) & 0x7FFFFFFFu;
           mx = max(mx, h);
           if (h != 0u) me = max(me, (int)(h >> 2) + f[c] * (1 << 18));   // >> 2: room for both exponents
+          if (keep) v[j][c] = 0.0;
         }
       }
       S.red[ph][pr] = keep || mx == 0u ? kNoEntry : mx >= 0x7FF00000u ? kNonfinite : me >> 18;
@@ -411,12 +420,6 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
         if (rot) mask = (mask & 0x0F0Fu) << 4 | ((mask >> 4) & 0x0F0Fu);   // from the lane's order to the columns'
         mask = __reduce_or_sync(0xffffffffu, mask);
         if (lane == 0) S.mask[ph] = mask;
-      }
-      if (keep) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) v[j][c] = 0.0;
       }
     } else {
       load(a.W, a.ldw, 0);
