@@ -363,7 +363,7 @@ constexpr int kRedWays = 8;
 __device__ __forceinline__ double sketch_reduce_chain(int64_t total, int chunks, const double* __restrict__ Ypart,
                                                       int64_t e, int way) {
   double acc = 0.0;
-#pragma unroll 4
+#pragma unroll 8
   for (int c = way; c < chunks; c += kRedWays) acc += Ypart[(size_t)c * total + e];
   return acc;
 }
