@@ -75,7 +75,8 @@ Plan make_plan(int64_t m, int n, int s, int tf = T_DCT, bool planes = false) {
   // the FP64 sketch from digit planes in row chunks: at most the chunks of a Q buffer with ldq = m, or
   // one chunk in the workspace's own planes
   const size_t q_bytes = sizeof(double) * (size_t)m * n;
-  const int64_t mr = (m + 4095) / 4096 * 4096;   // the four-step form's words of all rows in one range
+  // rows of the planes; where the four-step form may run, its words of all rows in one range
+  const int64_t unit = sketch_fd_ints_bytes(m, s) ? 4096 : 32, mr = (m + unit - 1) / unit * unit;
   if (planes) p.planes_bytes = 16ull * (size_t)n * (size_t)mr;
   p.ozpart_bytes = std::max({syrk_oz_part_bytes(p.oz), sketch_oz_part_bytes(p.sk), sketch_ozp_part_bytes(m, n, s, q_bytes),
                              planes ? sketch_ozp_part_bytes(m, n, s, p.planes_bytes) : size_t(0)});

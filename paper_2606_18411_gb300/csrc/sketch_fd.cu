@@ -570,14 +570,14 @@ bool sketch_fd_eligible(int64_t m, int n, int s, int tf, const void* scratch, si
 }
 
 size_t sketch_fd_part_bytes(int64_t m, int n, int s, size_t scratch_bytes) {
-  if (m % kR != 0 || s < kFdMinRows) return 0;
+  if (m % kR != 0 || m < (1 << 15) || s < kFdMinRows) return 0;
   const FdPlan p = fd_plan(m, n, s, scratch_bytes);
   if (p.Jc <= 0) return 0;
   return sizeof(long long) * kPartFd * (size_t)p.max_tiles * p.cblocks * p.slabs * p.chunks;
 }
 
 size_t sketch_fd_ints_bytes(int64_t m, int s) {
-  if (m % kR != 0 || s < kFdMinRows) return 0;
+  if (m % kR != 0 || m < (1 << 15) || s < kFdMinRows) return 0;
   const int tiles = kClasses + s / kFdTile;
   return sizeof(int) * (size_t)(64 + 512 + tiles + (size_t)kFdTile * tiles) + sizeof(uint32_t) * (size_t)(m / kR) + 1024;
 }
