@@ -116,6 +116,7 @@ struct RpCta {
   int (*red)[kM];               // [2][128]
   int* eRs;                     // e_k, padded to 512
   int* fNs;                     // -f_c, padded to 512
+  uint32_t* fKs;                // (1024 - f_c) << 20: added to a high word it orders |A F^-1|, without overflow
   uint32_t* cmax;               // column maxima of the result over this CTA's rows
   int* colE;                    // reference exponents of the multiplier columns
   int* emax;                    // largest of the scalings e_k, -f_c and 0
@@ -194,6 +195,7 @@ __device__ __forceinline__ void rp_begin(const RpArgs& a, RpCta& S) {
       S.colE[k] = keep ? E2 : E1;
       S.eRs[k] = e;
       S.fNs[k] = f;
+      S.fKs[k] = (uint32_t)(f + 1024) << 20;
       if (max(e, f) > 0) atomicMax(S.emax, max(e, f));
       if (keep && k % kRN == 0) atomicOr(S.keep, 1u << (k / kRN));
     }
@@ -379,21 +381,30 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
     bool keep = kTrsm && ((*S.keep >> t) & 1u) != 0u;
     if (kTrsm) {   // the rows' reference exponents: W D so far and A_t F^{-1} (W D alone in a kept panel)
       load(a.A, a.lda, c0);
-      uint32_t mx = 0u;
-      int me = INT_MIN;
+      uint32_t mx = 0u, mk = 0u;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int4 f4 = *reinterpret_cast<const int4*>(S.fNs + c0 + gcol[j]);
-        const int f[4] = {f4.x, f4.y, f4.z, f4.w};
+        const uint4 f4 = *reinterpret_cast<const uint4*>(S.fKs + c0 + gcol[j]);
+        const uint32_t f[4] = {f4.x, f4.y, f4.z, f4.w};
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const uint32_t h = (uint32_t)__double2hiint(v[j][c]) & 0x7FFFFFFFu;
           mx = max(mx, h);
-          if (h != 0u) me = max(me, (int)(h >> 2) + f[c] * (1 << 18));   // >> 2: room for both exponents
+          mk = max(mk, h + f[c]);
           if (keep) v[j][c] = 0.0;
         }
       }
-      S.red[ph][pr] = keep || mx == 0u ? kNoEntry : mx >= 0x7FF00000u ? kNonfinite : me >> 18;
+      if ((int)(mk >> 20) - 1024 <= *S.emax && mx != 0u) {   // no entry's exponent, or a zero's 0 - f_c: without zeros
+        mk = 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const uint32_t h = (uint32_t)__double2hiint(v[j][c]) & 0x7FFFFFFFu;
+            if (h != 0u) mk = max(mk, h + S.fKs[c0 + gcol[j] + c]);
+          }
+      }
+      S.red[ph][pr] = keep || mx == 0u ? kNoEntry : mx >= 0x7FF00000u ? kNonfinite : (int)(mk >> 20) - 1024;
       __syncthreads();
       if (tid < kM) {
         const int E = max(S.rowX[tid], max(S.red[0][tid], S.red[1][tid]));
@@ -531,8 +542,7 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
       double* wp = a.W + r0 + rr + (int64_t)(c0 + 16 * g) * a.ldw;
       uint32_t* cm = S.cmax + c0 + 16 * g;
       const int* er = S.eRs + c0 + 16 * g;
-      int mxE = INT_MIN;
-      uint32_t mxh = 0u;
+      uint32_t mxh = 0u, mk = 0u;
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
         if (c0 + 16 * g + c < n) {
@@ -541,13 +551,23 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
           if (h > cm[c]) atomicMax(cm + c, h);
           if (kTrsm) {
             mxh = max(mxh, h);
-            if (h != 0u) mxE = max(mxE, (int)(h >> 2) + er[c] * (1 << 18));   // >> 2: room for both exponents
+            mk = max(mk, (h | 0x80000000u) + ((uint32_t)er[c] << 20));   // exponent + e_k + 2048 (e_k <= 0: no overflow)
           }
         }
         wp += a.ldw;
       }
-      // zeros do not count: with e_k over more than 2^1000 a zero's 0 + e_k could pass every entry's exponent
-      if (kTrsm && mxh != 0u) atomicMax(&S.rowX[rr], mxh >= 0x7FF00000u ? kNonfinite : mxE >> 18);
+      if (kTrsm && mxh != 0u) {
+        // zeros do not count: with e_k over more than 2^1000 a zero's 0 + e_k could pass every entry's exponent
+        if (mk >> 20 <= 2048u) {
+          mk = 0u;
+#pragma unroll
+          for (int c = 0; c < 16; ++c) {
+            const uint32_t h = (uint32_t)__double2hiint(out[c]) & 0x7FFFFFFFu;
+            if (c0 + 16 * g + c < n && h != 0u) mk = max(mk, (h | 0x80000000u) + ((uint32_t)er[c] << 20));
+          }
+        }
+        atomicMax(&S.rowX[rr], mxh >= 0x7FF00000u ? kNonfinite : (int)(mk >> 20) - 2048);
+      }
     }
     if (__syncthreads_or(*(volatile int*)S.dead)) return false;   // the tile's W is visible to the next tile's loads
     if (kCheck && keep && ((*S.keep >> t) & 1u) == 0u && tid < kRN && c0 + tid < n) S.colE[c0 + tid] = a.colE[c0 + tid];
@@ -568,6 +588,7 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   __shared__ int red_s[2][kM];                                                 \
   __shared__ __align__(16) int eRs_s[512];                                     \
   __shared__ __align__(16) int fNs_s[512];                                     \
+  __shared__ __align__(16) uint32_t fKs_s[512];                                \
   __shared__ __align__(16) uint32_t cmax_s[512];                               \
   __shared__ __align__(16) int colE_s[512];                                             \
   if ((threadIdx.x >> 5) == 0) tc::tmem_alloc(&tmem_slot, kRTmem);             \
@@ -592,6 +613,7 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   S.red = red_s;                                                               \
   S.eRs = eRs_s;                                                               \
   S.fNs = fNs_s;                                                               \
+  S.fKs = fKs_s;                                                               \
   S.cmax = cmax_s;                                                             \
   S.colE = colE_s;                                                             \
   S.emax = &emax_s;                                                            \
@@ -668,15 +690,21 @@ __global__ void __launch_bounds__(128) k_rp_prep_x(int n, int npad, const double
 }
 
 // ---------------------------------------------------------------------------
-// -f_c = minus the unbiased exponent of max_k |R[k][c]| (0 for a zero or
-// non-finite column), 32 columns by the block's 256 threads; red: [8][32].
+// -f_c = minus the unbiased exponent of the largest finite |R[k][c]| (0 for a zero
+// column), so that no entry of R F^{-1} reaches 2 and e_k <= 0; 32 columns by the
+// block's 256 threads; red: [8][32].
+__device__ __forceinline__ uint32_t rp_finite_hi(double x) {   // |x|'s high word, 0 for a non-finite x
+  const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+  return h < 0x7FF00000u ? h : 0u;
+}
+
 __device__ __forceinline__ void rp_col_scale_block(int n, int npad, const double* __restrict__ RT, int* fN, int blk,
                                                    int (*red)[kRN]) {
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, c = kRN * blk + lane;
   uint32_t mx = 0u;
   if (c < n)
 #pragma unroll 8
-    for (int k = g; k <= c; k += 8) mx = max(mx, (uint32_t)__double2hiint(RT[(int64_t)k * npad + c]) & 0x7FFFFFFFu);
+    for (int k = g; k <= c; k += 8) mx = max(mx, rp_finite_hi(RT[(int64_t)k * npad + c]));
   __syncthreads();
   red[g][lane] = (int)mx;
   __syncthreads();
@@ -684,7 +712,7 @@ __device__ __forceinline__ void rp_col_scale_block(int n, int npad, const double
     int all = 0;
     for (int w = 0; w < 8; ++w) all = max(all, red[w][lane]);
     const int E = (int)oz::exp_field((uint32_t)all);
-    fN[c] = (E == 0 || E == 2047) ? 0 : 1023 - E;
+    fN[c] = E == 0 ? 0 : 1023 - E;
   }
 }
 
@@ -792,6 +820,31 @@ __device__ __forceinline__ __int128 rp_dot(const RpPrep& P, int k, int c, int j0
 // finds them (they agree).
 __device__ __forceinline__ void rp_own_scales(RpPrep& P, int n, int npad, const double* __restrict__ RT, const RpInts& I,
                                               int rows) {
+  if (n <= kRN) {   // one panel: rows 4 g .. of column c in this thread, loaded once
+    const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+    double x[4];
+    uint32_t mx = 0u;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int k = 4 * g + r;
+      x[r] = c < n && k <= c ? RT[(int64_t)k * npad + c] : 0.0;
+      mx = max(mx, rp_finite_hi(x[r]));
+    }
+    P.red[g][c] = (int)mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) mx = max(mx, (uint32_t)P.red[w][c]);
+    const int E = (int)oz::exp_field(mx), f = E == 0 ? 0 : 1023 - E;
+    if (g == 0 && c < n) P.fN[c] = I.fN[c] = f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const uint32_t h = (uint32_t)__double2hiint(x[r]) & 0x7FFFFFFFu;
+      const uint32_t all = __reduce_max_sync(0xffffffffu, h);
+      const int me = __reduce_max_sync(0xffffffffu, h >= 0x00100000u ? (int)(h >> 20) + f : INT_MIN);
+      if (c == 0 && 4 * g + r < n) I.eR[4 * g + r] = (all >= 0x7FF00000u || me == INT_MIN) ? 0 : me - 1023;
+    }
+    return;
+  }
   for (int blk = 0; blk < (n + kRN - 1) / kRN; ++blk) rp_col_scale_block(n, npad, RT, P.fN, blk, P.red);
   __syncthreads();
   for (int c = threadIdx.x; c < n; c += 256) I.fN[c] = P.fN[c];
