@@ -34,8 +34,8 @@
 //    a kept panel costs about three of the others.)
 //    F fits A where W's columns are of one size, as for a factor R of A.  Where R is
 //    the caller's (mrcqr_trsm, mrcqr_cholqr_precond) a row block checks it: a panel with a
-//    column of A F^{-1} below 2^-10 of the largest entry of the block's A F^{-1} or W D
-//    would lose that column's digits, and is solved by substitution as well.
+//    column of A F^{-1} that is zero or below 2^-10 of the largest entry of the block's A F^{-1}
+//    or W D could lose that column's digits, and is solved by substitution as well.
 //
 // Measured at m = 2^20 (before: substitution blocks of 16 columns; Q = W X in
 // 128 x 64 tiles by one CTA per SM): W = A R^{-1} 1.78 -> 0.75 ms at n = 64,
@@ -122,7 +122,7 @@ struct RpCta {
   int* emax;                    // largest of the scalings e_k, -f_c and 0
   uint32_t* keep;               // bit t: panel t keeps its substitution
   int* rho;                     // checked solve: largest rowRef of each 32 rows
-  uint32_t* mask;               // columns 16 h .. of the panel with an entry near them [h]; with any entry [2 + h]
+  uint32_t* mask;               // [2] columns 16 h .. of the panel with an entry near it
 };
 
 __device__ __forceinline__ void rp_wait(RpCta& S, uint64_t* bar, uint32_t parity) {
@@ -259,42 +259,44 @@ __device__ __noinline__ void rp_solve_row(const RpArgs& a, double* sb, int64_t r
   }
 }
 
-// Checked solve: the exponent that every column of A F^{-1} in the panel should reach in the row block.
+// Checked solve: the exponent that every column of A F^{-1} in the panel should reach in the row block (kAllZero:
+// neither A nor W D has an entry).
+constexpr int kAllZero = -4000;
 __device__ __forceinline__ int rp_threshold(const RpCta& S) {
-  return max(max(max(S.rho[0], S.rho[1]), max(S.rho[2], S.rho[3])) - kBalance, -4000);
+  return max(max(max(S.rho[0], S.rho[1]), max(S.rho[2], S.rho[3])) - kBalance, kAllZero);
 }
 
-// Whether every column of the panel at c0 that has an entry in the row block
-// has one near the block's largest (every thread).  The full look, for panels
-// where the first 32 rows do not show it.
+// Whether every column of the panel at c0 has an entry near the block's largest
+// (every thread); a column of zeros has none: W there is as large as the
+// others make it, which nothing here bounds.  The full look, for panels where
+// the first 32 rows do not show it.
 __device__ __noinline__ bool rp_balanced_full(const RpArgs& a, const int* fNs, uint32_t* mask, int thr, int64_t r0,
                                               int c0) {
   const int tid = threadIdx.x, pr = tid & (kM - 1), ph = tid >> 7;
   __syncthreads();
-  if (tid < 4) mask[tid] = 0u;
+  if (tid < 2) mask[tid] = 0u;
   __syncthreads();
   const double* p = a.A + min(r0 + pr, a.m - 1) + (int64_t)(c0 + 16 * ph) * a.lda;
-  uint32_t near = 0u, any = 0u;
-  for (int c = 0; c < 16 && c0 + 16 * ph + c < a.n; ++c, p += a.lda) {
+  uint32_t near = 0u;
+  for (int c = 0; c < 16; ++c, p += a.lda) {
+    if (c0 + 16 * ph + c >= a.n) {   // beyond the last panel's columns
+      near |= 0xFFFFu << c & 0xFFFFu;
+      break;
+    }
     const uint32_t h = (uint32_t)__double2hiint(*p) & 0x7FFFFFFFu;
-    if (h == 0u || h >= 0x7FF00000u) continue;
-    any |= 1u << c;
-    if ((int)(h >> 2) + fNs[c0 + 16 * ph + c] * (1 << 18) >= thr) near |= 1u << c;
+    if (h != 0u && h < 0x7FF00000u && (int)(h >> 2) + fNs[c0 + 16 * ph + c] * (1 << 18) >= thr) near |= 1u << c;
   }
   near = __reduce_or_sync(0xffffffffu, near);
-  any = __reduce_or_sync(0xffffffffu, any);
-  if ((tid & 31) == 0) {
-    atomicOr(&mask[ph], near);
-    atomicOr(&mask[2 + ph], any);
-  }
+  if ((tid & 31) == 0) atomicOr(&mask[ph], near);
   __syncthreads();
-  return ((mask[2] & ~mask[0]) | (mask[3] & ~mask[1])) == 0u;
+  return (mask[0] & mask[1]) == 0xFFFFu;
 }
 
 __device__ __forceinline__ bool rp_balanced(const RpArgs& a, const RpCta& S, int64_t r0, int c0) {
   const uint32_t all = min(kRN, a.n - c0) == kRN ? 0xFFFFFFFFu : (1u << (a.n - c0)) - 1u;
-  return ((S.mask[0] | S.mask[1] << 16) & all) == all ||
-         rp_balanced_full(a, S.fNs, S.mask, rp_threshold(S) * (1 << 18), r0, c0);
+  const int thr = rp_threshold(S);
+  return thr == kAllZero || ((S.mask[0] | S.mask[1] << 16) & all) == all ||
+         rp_balanced_full(a, S.fNs, S.mask, thr * (1 << 18), r0, c0);
 }
 
 // One block of 128 rows from r0; the CTA's next block is `next` blocks further (0: unknown).  False when a wait
@@ -582,7 +584,7 @@ __device__ __forceinline__ bool rp_block(const RpArgs& a, RpCta& S, int64_t r0, 
   __shared__ int dead_s, emax_s;                                               \
   __shared__ uint32_t keep_s;                                                  \
   __shared__ int rho_s[kM / 32];                                               \
-  __shared__ uint32_t mask_s[4];                                               \
+  __shared__ uint32_t mask_s[2];                                               \
   __shared__ int rowX_s[kM];                                                   \
   __shared__ int rowRef_s[kM];                                                 \
   __shared__ int red_s[2][kM];                                                 \

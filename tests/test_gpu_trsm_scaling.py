@@ -184,3 +184,18 @@ def test_nonfinite_entry_reaches_only_the_columns_after_it(env, col, value):
     # two solutions with backward errors gamma_n |W| |R|: apart by at most that through |R^-1|
     bound = 8 * n * U * (np.abs(clean[row]) @ np.abs(R)) @ np.abs(np.linalg.inv(R))
     assert (np.abs(W[row, :col] - clean[row, :col]) <= bound[:col]).all()
+
+
+# A column of A that is zero in a row block: W there is what the columns before it make it, here 2^-40 of them.
+@pytest.mark.parametrize("m,n,j", [(1, 20, 10), (150, 64, 31), (300, 70, 68)])
+def test_trsm_zero_column_of_a(env, m, n, j):
+    torch, M = env
+    rng = np.random.default_rng(n)
+    A = rng.standard_normal((m, n))
+    A[:128, j] = 0.0
+    A[128:, j] *= 2.0 ** -40
+    R = np.eye(n)
+    R[:j, j] = rng.standard_normal(j) * 2.0 ** -40
+    W = M.trsm(M.to_colmajor(A), M.to_colmajor(R)).cpu().numpy()
+    res, scale = _column_residuals(A, W, R)
+    assert (res <= 4 * n * U * scale).all(), float((res / scale).max())
